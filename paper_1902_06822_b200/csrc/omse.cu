@@ -48,7 +48,7 @@ struct Workspace {
 // What the per-tensor search remembers between calls: launch shapes and attributes that cost more to ask for than a launch.
 struct TensorLaunches {
     int occ_pass[3];                                        // blocks per SM of the three pass kernels (0 = not yet asked)
-    struct { size_t smem; int occ; } hist[2];               // the histogram kernel's last launch shape, per variant
+    struct { size_t smem; int occ; } hist[4];               // the histogram kernel's last launch shape, per variant
     bool attr_hist, attr_resident;
 };
 
@@ -259,15 +259,18 @@ constexpr int kHistWindow = 8192;    // bins of one histogram launch
 constexpr int kHistBlocks = 1024;    // its blocks at most (room for their sums)
 
 int launch_hist(const TensorEnv& env, const omse::TensorArgs& a, bool full, int* n_blocks) {
+    typedef void (*Kernel)(const omse::TensorArgs);
+    const Kernel kernels[4] = {omse::tensor_hist_kernel<false, false>, omse::tensor_hist_kernel<false, true>,
+                               omse::tensor_hist_kernel<true, false>, omse::tensor_hist_kernel<true, true>};
     const size_t smem = (size_t)a.win * 20 + 8 * omse::kHotWords + (size_t)a.n_bins2 * 12;
     if (!env.seen->attr_hist) {
-        if (cudaFuncSetAttribute(omse::tensor_hist_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess ||
-            cudaFuncSetAttribute(omse::tensor_hist_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess)
-            return OMSE_ECUDA;
+        for (const auto k : kernels)
+            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess) return OMSE_ECUDA;
         env.seen->attr_hist = true;
     }
-    auto kernel = full ? omse::tensor_hist_kernel<true> : omse::tensor_hist_kernel<false>;
-    auto& seen = env.seen->hist[full ? 1 : 0];
+    const int id = (full ? 2 : 0) + (a.lo < 0 ? 1 : 0);
+    const Kernel kernel = kernels[id];
+    auto& seen = env.seen->hist[id];
     if (seen.occ == 0 || seen.smem != smem) {
         int occ = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, omse::kHistThreads, smem) != cudaSuccess || occ < 1) return OMSE_ECUDA;
@@ -310,7 +313,7 @@ int enqueue_tensor_search(const TensorEnv& env, omse::TensorArgs& a, int refine_
     a.hist = reinterpret_cast<unsigned long long*>(at);
     a.above = (at += hist_words);
     a.block_sums = (at += hist_words);
-    a.levels = (at += 5 * kHistBlocks);
+    a.levels = (at += omse::kBlockSums * kHistBlocks);
     if (at + 2 * a.n_cand > a.partials + a.partial_doubles) return OMSE_ELIMIT;
     long long absmax_grid = (n + 1023) / 1024;
     if (absmax_grid > (long long)env.n_sm * 8) absmax_grid = (long long)env.n_sm * 8;

@@ -38,6 +38,7 @@ struct TensorState {          // lives in the context workspace
     int key_min, key_max;                // offset mode: order-preserving integer keys of min and max of the tensor
     float delta;                         // offset subtracted from every element (0 without offset)
     double sum_sq;                       // sum x^2
+    double near;                         // sum of floor(|x|/h) over the values next to an edge of a bin (see tensor_noise)
     // state of the scan at the first bin of the window processed last (bins are taken in windows from the top down)
     double scan_n, scan_s, scan_f;
     long long scan_pos;
@@ -57,7 +58,8 @@ struct TensorArgs {
     TensorState* st;
     unsigned long long* hist;   // [2][win] counts and fractional sums, then [2][n_bins2]
     double* above;          // [2][win] N and P of the window, then [2][n_bins2]
-    double* block_sums;     // [grid][5]: sum x^2, number and excess of the values above the bins, the same for the coarse ones
+    double* block_sums;     // [grid][kBlockSums]: sum x^2, number and excess of the values above the bins, the same for the coarse
+                            // ones, sum of the bins of the values next to an edge
     int n_blocks;           // blocks of the histogram launch
     double* levels;         // [2][n_cand] <x,q>/h and <q,q>
     double* partials;       // passes: [blocks][listed candidates] doubles + [blocks] int64
@@ -87,6 +89,7 @@ __device__ __forceinline__ void tensor_state_init(TensorState* st) {
     st->key_max = (int)0x80000000;
     st->delta = 0.f;
     st->sum_sq = 0.0;
+    st->near = 0.0;
 }
 __global__ void tensor_init_kernel(TensorState* st) {
     if (threadIdx.x == 0) tensor_state_init(st);
@@ -165,12 +168,22 @@ __global__ void __launch_bounds__(256) tensor_absmax_kernel(const float* __restr
     }
 }
 
-// Fractional parts are kept exactly: h = H*2^e with an integer 2^23 <= H < 2^24, a value a >= h is a multiple of 2^e, and so
-// is a - m*h, which fma() forms without rounding: an integer k of 24 bits (up to 1.001*H, see inv_dn).
-//
+// Bins and fractional parts are exact: h = H*2^e with an integer 2^23 <= H < 2^24, so |x|/h = a/H with a = |x|*2^-e, and a - m*H,
+// which fma() forms without rounding, is an integer k for every a >= H.  inv_up exceeds 1/H by 2.3e-7 to 4.8e-7 of it, so
+// floor(a*inv_up) is the value's bin m or, for a value just below an edge, the bin above; a negative k tells.
+// hist_near: the rare values that need the correction, or lie above an edge by so little that a scale's rounding or the rounding
+// of x/alpha could put them below it (1.2e-7*|x|, up to 2.1*m units of k): their bins are added up for tensor_noise.
+__device__ __forceinline__ bool hist_near(int k, int m) { return k < 3 * m; }       // (false for a bin below the first)
+__device__ __forceinline__ void hist_correct(int& k, int& m, unsigned int hk) {
+    if (k < 0) {
+        k += (int)hk;
+        --m;
+    }
+}
+
 // hist_put adds one value to bin word `w`: k is spread over two 32-bit words, count and low six bits in the first, the rest
 // in the second.  Up to kHistChunk values fit in one bin without overflow (8160*63 < 2^19, 8160 < 2^13,
-// 8160*1.001*2^18 < 2^32), and an insertion costs two shared-memory atomics instead of three.
+// 8160*2^18 < 2^32), and an insertion costs two shared-memory atomics instead of three.
 __device__ __forceinline__ void hist_put(unsigned int* w1, unsigned int* w2, int w, unsigned int k) {
     atomicAdd(w1 + w, (1u << 19) + (k & 63u));
     atomicAdd(w2 + w, k >> 6);
@@ -188,18 +201,19 @@ __device__ __forceinline__ void hist_put3(unsigned int* c, unsigned int* lo, uns
 
 // What the insertions need to know about the grid.
 struct HistGeometry {
-    float pre, h, inv_dn, to_k;   // |x| -> bin: floor(|x|*pre*inv_dn); remainder -> k: r*to_k
+    float pre, scale, h, inv_up;  // a = |x*pre*scale|, h = H; bin floor(a*inv_up)
+    float far;                    // bins from here on are above all histograms
     int sgn, d, d_from, n_bins, n_bins2, base, top;
     unsigned int rd, hk;          // 2^32/D; H
 };
 __device__ __forceinline__ HistGeometry hist_geometry(float step, const TensorArgs& a) {
     HistGeometry g;
-    g.pre = step > 1e-30f ? 1.0f : 18446744073709551616.0f;      // 2^64: keeps 1/h finite for the smallest steps
-    g.h = __fmul_rn(__fmul_rn(step, g.pre), 0.5f);
-    g.inv_dn = __fdiv_rn(1.0f, g.h) * (1.0f - 3.0e-7f);           // never above |x|/h: remainders are >= 0
-    const int hb = __float_as_int(g.h);
+    g.pre = step > 1e-30f ? 1.0f : 18446744073709551616.0f;      // 2^64: keeps the powers of two finite for the smallest steps
+    const int hb = __float_as_int(__fmul_rn(__fmul_rn(step, g.pre), 0.5f));
     g.hk = (hb & 0x7fffff) | 0x800000;
-    g.to_k = __int_as_float((277 - (hb >> 23)) << 23);            // 2^-e: h = hk*2^e with e = (hb >> 23) - 150
+    g.scale = __int_as_float((277 - (hb >> 23)) << 23);           // 2^-e: h*pre = hk*2^e with e = (hb >> 23) - 150
+    g.h = (float)g.hk;
+    g.inv_up = __fdiv_rn(1.0f, g.h) * (1.0f + 3.0e-7f);           // never below 1/H
     g.sgn = a.lo < 0;
     g.d = a.n_bins2 > 0 ? -2 * a.lo - 1 : 0;
     g.d_from = g.d > 0 ? g.d : 0x7fffffff;
@@ -208,6 +222,7 @@ __device__ __forceinline__ HistGeometry hist_geometry(float step, const TensorAr
     g.n_bins2 = a.n_bins2;
     g.base = a.win_base;
     g.top = a.win_base + a.win;
+    g.far = (float)(max(a.n_bins, g.d * (a.n_bins2 + 1)) + 2);    // (2,084,866 at most: 4.8e-7 of it is less than a bin)
     return g;
 }
 // one unit 2^e in units of h, as the factor of the fractional sums
@@ -217,58 +232,83 @@ __device__ __forceinline__ double hist_unit(float step) {
 }
 struct HistSums {
     double sq, over_n, over_s, over2_n, over2_s;
+    long long near;
 };
+constexpr int kBlockSums = 6;
 // Words of a block's histograms.
 struct HistWords {
     unsigned int *w1, *w2;            // fine window, hot copies first (two-word form)
     unsigned int *c2, *lo2, *hi2;     // coarse histogram (three-word form)
 };
 
-// One value into the words of the fine window and of the coarse histogram.
-// FULL: the window holds all bins and no value lies above them (the common case).
-template <bool FULL>
-__device__ __forceinline__ void hist_insert(float x, const HistGeometry& g, const HistWords& w, bool first, HistSums& s) {
-    const float y = x * g.pre;
-    const float a = g.sgn ? fabsf(y) : y;                 // an unsigned range codes negative values as 0
-    if (FULL || first) s.sq = fma((double)x, (double)x, s.sq);
-    float mf;
-    int m;
-    if (FULL) {
-        const float u = __fmaf_rd(a, g.inv_dn, kMagic);
-        m = magic_int(u);
-        mf = u - kMagic;
-        if (m < 1) return;
-        const unsigned int k = __float2uint_rz(fmaf(-mf, g.h, a) * g.to_k);
-        const int i = min(m, g.n_bins) - 1;
-        hist_put(w.w1, w.w2, i < kHotBins ? i * kHotCopies + (threadIdx.x & (kHotCopies - 1)) : kHotWords + i, k);
-        if (y < 0.f && m >= g.d_from) {
-            const unsigned int m2 = __umulhi((unsigned)m, g.rd), rem = (unsigned)m - m2 * (unsigned)g.d;
-            hist_put3(w.c2, w.lo2, w.hi2, min((int)m2, g.n_bins2) - 1, rem * g.hk + k);
-        }
-        return;
+// One value, its bin and remainder known, into the words of the fine window (bins base+1 ...) and of the coarse histogram.
+__device__ __forceinline__ void hist_put_fine(const HistGeometry& g, const HistWords& w, int i, int k) {
+    hist_put(w.w1, w.w2, g.base == 0 && i < kHotBins ? i * kHotCopies + (threadIdx.x & (kHotCopies - 1)) : kHotWords + i, (unsigned)k);
+}
+__device__ __forceinline__ void hist_put_coarse(const HistGeometry& g, const HistWords& w, int m, int k) {
+    const unsigned int m2 = __umulhi((unsigned)m, g.rd), rem = (unsigned)m - m2 * (unsigned)g.d;
+    hist_put3(w.c2, w.lo2, w.hi2, min((int)m2, g.n_bins2) - 1, rem * g.hk + (unsigned)k);
+}
+
+// Four values x*pre where the window holds all bins and no value lies above them (the common case).  One branch for the rare
+// values next to an edge, instead of four.  SIGNED: the range has negative codes; an unsigned one codes negative values as 0.
+template <bool SIGNED>
+__device__ __forceinline__ void hist_insert4(const float (&x)[4], const HistGeometry& g, const HistWords& w, HistSums& s) {
+    int m[4], k[4], least = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float y = x[j] * g.scale, a = SIGNED ? fabsf(y) : y, u = __fmaf_rd(a, g.inv_up, kMagic);
+        s.sq = fma((double)x[j], (double)x[j], s.sq);
+        m[j] = magic_int(u);
+        k[j] = __float2int_rz(fmaf(-(u - kMagic), g.h, a));
+        least = min(least, k[j] - 3 * m[j]);
     }
-    // generic path: values may lie above the last bin or outside the window
-    const float td = a * g.inv_dn;
+    if (least < 0) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (m[j] >= 1 && hist_near(k[j], m[j])) {
+                s.near += m[j];
+                hist_correct(k[j], m[j], g.hk);
+            }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (m[j] < 1) continue;
+        hist_put_fine(g, w, min(m[j], g.n_bins) - 1, k[j]);
+        if (SIGNED && x[j] < 0.f && m[j] >= g.d_from) hist_put_coarse(g, w, m[j], k[j]);
+    }
+}
+// One value x*pre where values may lie above the last bin or outside the window.
+template <bool SIGNED>
+__device__ __forceinline__ void hist_insert(float x, const HistGeometry& g, const HistWords& w, bool first, HistSums& s) {
+    const float y = x * g.scale, a = SIGNED ? fabsf(y) : y, td = a * g.inv_up;
+    if (first) s.sq = fma((double)x, (double)x, s.sq);
     if (!(td >= 1.0f)) return;
-    mf = floorf(td);
-    if (td >= (float)(g.n_bins + 1)) {
+    int m = 0x7fffffff, k = 0;                            // far above the bins
+    if (td < g.far) {
+        const float u = __fmaf_rd(a, g.inv_up, kMagic);
+        m = magic_int(u);
+        k = __float2int_rz(fmaf(-(u - kMagic), g.h, a));
+        if (hist_near(k, m)) {
+            if (first) s.near += m;
+            hist_correct(k, m, g.hk);
+            if (m < 1) return;
+        }
+    }
+    if (m > g.n_bins) {
         if (first) {
             s.over_n += 1.0;
             s.over_s += (double)a / (double)g.h - (double)(g.n_bins + 1);
         }
-    } else if (td >= (float)(g.base + 1) && td < (float)(g.top + 1)) {
-        const int i = (int)mf - 1 - g.base;
-        hist_put(w.w1, w.w2, g.base == 0 && i < kHotBins ? i * kHotCopies + (threadIdx.x & (kHotCopies - 1)) : kHotWords + i,
-                 __float2uint_rz(fmaf(-mf, g.h, a) * g.to_k));
+    } else if (m > g.base && m <= g.top) {
+        hist_put_fine(g, w, m - 1 - g.base, k);
     }
-    if (first && y < 0.f && g.d > 0 && td >= (float)g.d) {
-        if (td >= (float)g.d * (float)(g.n_bins2 + 1)) {
+    if (SIGNED && first && x < 0.f && g.d > 0 && m >= g.d) {
+        if (m >= g.d * (g.n_bins2 + 1)) {
             s.over2_n += 1.0;
             s.over2_s += (double)a / ((double)g.h * (double)g.d) - (double)(g.n_bins2 + 1);
         } else {
-            m = (int)mf;
-            const unsigned int m2 = (unsigned)m / (unsigned)g.d, rem = (unsigned)m - m2 * (unsigned)g.d;
-            hist_put3(w.c2, w.lo2, w.hi2, min((int)m2, g.n_bins2) - 1, rem * g.hk + __float2uint_rz(fmaf(-mf, g.h, a) * g.to_k));
+            hist_put_coarse(g, w, m, k);
         }
     }
 }
@@ -276,7 +316,7 @@ __device__ __forceinline__ void hist_insert(float x, const HistGeometry& g, cons
 // Histogram of one window of bins.  A block takes chunks of the tensor in turn; after each the 32-bit words are folded into
 // the block's 64-bit sums, and at the end those go to the global histogram by integer atomics (any order, same result).
 // Bound: one read of the tensor from HBM beside two shared-memory atomics per value (2.7 clocks per warp each).
-template <bool FULL>
+template <bool FULL, bool SIGNED>
 __global__ void __launch_bounds__(kHistThreads, 2) tensor_hist_kernel(const TensorArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double dscratch[64];
@@ -292,10 +332,10 @@ __global__ void __launch_bounds__(kHistThreads, 2) tensor_hist_kernel(const Tens
     unsigned int* acc_n = w.hi2 + a.n_bins2;
     const float m = fmaxf(__uint_as_float(st->mpos_bits), __uint_as_float(st->mneg_bits));
     const Grid gr = grid_of(m, a.hi_frac, a.n_cand);
-    HistSums s = {0.0, 0.0, 0.0, 0.0, 0.0};
+    HistSums s = {0.0, 0.0, 0.0, 0.0, 0.0, 0ll};
     if (gr.usable && !st->bad) {
         const HistGeometry g = hist_geometry(gr.step, a);
-        const float delta = st->delta;
+        const float delta = st->delta, off = -delta * g.pre;        // fmaf(x, pre, off) = pre*fl(x - delta): pre is a power of two
         const bool first = a.first_window != 0;
         for (int i = tid; i < 2 * words + 3 * a.n_bins2; i += kHistThreads) w.w1[i] = 0u;      // all words
         for (int i = tid; i < a.win; i += kHistThreads) {
@@ -320,14 +360,20 @@ __global__ void __launch_bounds__(kHistThreads, 2) tensor_hist_kernel(const Tens
             __syncthreads();                                        // words are clear
 #pragma unroll
             for (int j = 0; j < per; ++j) {
-                hist_insert<FULL>(v[j].x - delta, g, w, first, s);
-                hist_insert<FULL>(v[j].y - delta, g, w, first, s);
-                hist_insert<FULL>(v[j].z - delta, g, w, first, s);
-                hist_insert<FULL>(v[j].w - delta, g, w, first, s);
+                const float x[4] = {fmaf(v[j].x, g.pre, off), fmaf(v[j].y, g.pre, off), fmaf(v[j].z, g.pre, off), fmaf(v[j].w, g.pre, off)};
+                if (FULL) {
+                    hist_insert4<SIGNED>(x, g, w, s);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) hist_insert<SIGNED>(x[e], g, w, first, s);
+                }
             }
             if (c0 + (long long)gridDim.x * chunk4 < n4_all) fetch(c0 + (long long)gridDim.x * chunk4);   // next chunk on its way
-            if (c0 + chunk4 > n4 && tid < (int)(a.n - 4 * n4))      // the last one to three values
-                hist_insert<FULL>(a.x[4 * n4 + tid] - delta, g, w, first, s);
+            if (c0 + chunk4 > n4 && tid < (int)(a.n - 4 * n4)) {    // the last one to three values
+                const float x[4] = {fmaf(a.x[4 * n4 + tid], g.pre, off), 0.f, 0.f, 0.f};
+                if (FULL) hist_insert4<SIGNED>(x, g, w, s);
+                else hist_insert<SIGNED>(x[0], g, w, first, s);
+            }
             __syncthreads();
             if (a.win_base == 0 && tid < kHotBins && tid < a.win) {
                 unsigned int c = 0u;
@@ -379,15 +425,17 @@ __global__ void __launch_bounds__(kHistThreads, 2) tensor_hist_kernel(const Tens
                     atomicAdd(a.hist + 2 * a.win + b, (unsigned long long)w.c2[b]);
                     atomicAdd(a.hist + 2 * a.win + a.n_bins2 + b, ((unsigned long long)w.hi2[b] << 16) + w.lo2[b]);
                 }
+        s.sq *= 1.0 / ((double)g.pre * (double)g.pre);
         if (blockIdx.x == 0 && tid == 0 && a.evals && first) atomicAdd(a.evals, (unsigned long long)a.n);
     }
     if (a.first_window) {
         double v[5] = {s.sq, s.over_n, s.over_s, s.over2_n, s.over2_s};
 #pragma unroll
         for (int j = 0; j < 5; ++j) {
-            long long zero = 0;
-            block_sum2(v[j], zero, dscratch);
-            if (tid == 0) a.block_sums[5 * blockIdx.x + j] = v[j];
+            long long near = j == 0 ? s.near : 0ll;
+            block_sum2(v[j], near, dscratch);
+            if (tid == 0) a.block_sums[kBlockSums * blockIdx.x + j] = v[j];
+            if (tid == 0 && j == 0) a.block_sums[kBlockSums * blockIdx.x + 5] = (double)near;
         }
     }
 }
@@ -481,18 +529,21 @@ __global__ void __launch_bounds__(kScanThreads) tensor_scan_kernel(const TensorA
     const double unit = hist_unit(grid_of(m, a.hi_frac, a.n_cand).step);
     double cn = 0.0, cs = 0.0, cf = 0.0, gap = 0.0;
     if (a.first_window) {
-        double t[5];
+        double t[kBlockSums];
 #pragma unroll
-        for (int j = 0; j < 5; ++j) {                      // the blocks' sums, in a fixed order
+        for (int j = 0; j < kBlockSums; ++j) {             // the blocks' sums, in a fixed order
             long long zero = 0;
             t[j] = 0.0;
-            for (int b = threadIdx.x; b < a.n_blocks; b += kScanThreads) t[j] += __ldcg(a.block_sums + 5 * b + j);
-            if (j == 0 || a.clipped) block_sum2(t[j], zero, scratch);
+            for (int b = threadIdx.x; b < a.n_blocks; b += kScanThreads) t[j] += __ldcg(a.block_sums + kBlockSums * b + j);
+            if (j == 0 || j == 5 || a.clipped) block_sum2(t[j], zero, scratch);
         }
         cn = a.clipped ? t[1] : 0.0;
         cs = a.clipped ? t[2] : 0.0;
         gap = (double)(a.n_bins - a.win_base);
-        if (threadIdx.x == 0) st->sum_sq = t[0];
+        if (threadIdx.x == 0) {
+            st->sum_sq = t[0];
+            st->near = t[5];
+        }
         if (a.n_bins2 > 0) {
             const double d = (double)(-2 * a.lo - 1);
             double dn = a.clipped ? t[3] : 0.0, ds = a.clipped ? t[4] : 0.0, df = 0.0;
@@ -565,9 +616,18 @@ __device__ __forceinline__ double tensor_error(float step, int c, double sum_sq,
     const double al = (double)ac, h = 0.5 * (double)step;
     return fmax(fma(al * al, sq, fma(-2.0 * al * h, sx, sum_sq)), 0.0);
 }
-// Candidates up to this may be the minimum: near-ties, and what the rounding of the binary64 sums can amount to (their
-// terms are exact; a value within 4e-7 of a threshold may be counted on either side of it, which moves an error by less
-// than 4e-7*|x| times twice the distance of the value from the threshold, itself below 4e-7*|x|).
+// What separates the curve at candidate c from the error that exact_code's codes give.  The curve counts a value above the
+// threshold m*h, m = (2j-1)*(c+1); the codes follow the IEEE quotient by alpha_c = fl((c+1)*step), whose threshold lies within
+// 2^-23 of m*h.  A value in between is coded to the other neighbour, which moves its error by 2*alpha_c times its distance from
+// the midpoint, 1.8e-7*m*h at most.  Such values are next to an edge of a bin; `near` is the sum of their m, so the sum of these
+// terms is at most 4*(c+1)*1.8e-7*h^2*near.  Among values drawn from a density one in a million lies there and the bound is far
+// below the band; among values on a lattice of their own all may.
+__device__ __forceinline__ double tensor_noise(float step, int c, double near) {
+    const double h = 0.5 * (double)step;
+    return 8e-7 * (double)(c + 1) * h * h * near;
+}
+// Candidates whose value less their noise is up to this may be the minimum (bv: the smallest value, its noise added): near-ties,
+// and what the rounding of the binary64 sums can amount to.
 __device__ __forceinline__ double tensor_band(double bv, double sum_sq) {
     return bv * (1.0 + kRescoreBand) + 1e-13 * sum_sq;
 }
@@ -603,11 +663,11 @@ __global__ void __launch_bounds__(1024) tensor_finish_kernel(const TensorArgs a)
         }
         return;
     }
-    const double band = tensor_band(bv, sum_sq);
+    const double near = st->near, band = tensor_band(bv + tensor_noise(g.step, bi, near), sum_sq);
     const double tiny = a.curve_out ? kTinyShare * sum_sq : 0.0;
     for (int c = threadIdx.x; c < a.n_cand; c += blockDim.x) {
         const double v = a.curve[c];
-        if (v <= band || v < tiny) a.list[atomicAdd(&cnt, 1)] = c;   // at most n_cand entries: the list holds them all
+        if (v - tensor_noise(g.step, c, near) <= band || v < tiny) a.list[atomicAdd(&cnt, 1)] = c;   // at most n_cand entries: the list holds them all
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -965,13 +1025,20 @@ __global__ void __launch_bounds__(kResidentThreads) tensor_resident_kernel(const
         unsigned int* wc = reinterpret_cast<unsigned int*>(above);
         unsigned int *wl = wc + bins, *wh = wl + bins, *c2 = wh + bins, *l2 = c2 + a.n_bins2, *h2 = l2 + a.n_bins2;
         double sq = 0.0;
+        long long near = 0;
         auto insert = [&](float x) {
-            const float y = x * g.pre, v = g.sgn ? fabsf(y) : y;
+            const float y = x * g.pre * g.scale, v = g.sgn ? fabsf(y) : y;
             sq = fma((double)x, (double)x, sq);
-            const float u = __fmaf_rd(v, g.inv_dn, kMagic);
-            const int mm = magic_int(u);
+            const float u = __fmaf_rd(v, g.inv_up, kMagic);
+            int mm = magic_int(u);
             if (mm < 1) return;
-            const unsigned int k = __float2uint_rz(fmaf(-(u - kMagic), g.h, v) * g.to_k);
+            int ks = __float2int_rz(fmaf(-(u - kMagic), g.h, v));
+            if (hist_near(ks, mm)) {
+                near += mm;
+                hist_correct(ks, mm, g.hk);
+                if (mm < 1) return;
+            }
+            const unsigned int k = (unsigned)ks;
             hist_put3(wc, wl, wh, min(mm, g.n_bins) - 1, k);
             if (y < 0.f && mm >= g.d_from) {
                 const unsigned int m2 = __umulhi((unsigned)mm, g.rd), rem = (unsigned)mm - m2 * (unsigned)g.d;
@@ -1011,7 +1078,7 @@ __global__ void __launch_bounds__(kResidentThreads) tensor_resident_kernel(const
         __threadfence();                                            // this thread's additions before the block's slot
         long long none = 0;
         double sum_sq = sq;
-        ok = resident_sum(team, sum_sq, none, scratch) && ok;       // every block's additions are in L2 after this
+        ok = resident_sum(team, sum_sq, near, scratch) && ok;       // every block's additions are in L2 after this (near < 2^29 per block)
         __threadfence();
         // ---- N, P and the curve, in every block
         const double unit = hist_unit(gr.step);
@@ -1052,10 +1119,11 @@ __global__ void __launch_bounds__(kResidentThreads) tensor_resident_kernel(const
         block_argmin(bv, bi, scratch);
         __syncthreads();
         best = bi;
-        const double band = tensor_band(bv, sum_sq), tiny = a.curve_out ? kTinyShare * sum_sq : 0.0;
+        const double near_sum = (double)near, tiny = a.curve_out ? kTinyShare * sum_sq : 0.0;
+        const double band = tensor_band(bv + tensor_noise(gr.step, bi, near_sum), sum_sq);
         // ---- candidates to re-score, in increasing order: thread t looks at candidates 2t and 2t+1
         static_assert(kResidentCands <= 2 * kResidentThreads, "two candidates per thread");
-        auto wanted = [&](int c) { return c < a.n_cand && (curve[c] <= band || curve[c] < tiny); };
+        auto wanted = [&](int c) { return c < a.n_cand && (curve[c] - tensor_noise(gr.step, c, near_sum) <= band || curve[c] < tiny); };
         const bool in0 = wanted(2 * tid), in1 = wanted(2 * tid + 1);
         const unsigned int b0 = __ballot_sync(0xffffffffu, in0), b1 = __ballot_sync(0xffffffffu, in1), below = (1u << lane) - 1u;
         if (lane == 0) s_count[warp] = __popc(b0) + __popc(b1);
