@@ -8,12 +8,13 @@
 // the whole curve is  SSE(c)/h^2 = sum_i (x_i/h)^2 - 4*(c+1) * sum_{j <= L} P((2j-1)*(c+1)),
 // and P is the second-order suffix sum of a histogram of |x|/h with unit bins that keeps, per bin, the number of values
 // and the sum of their fractional parts.  So the C candidates cost K insertions, a scan of 2C bins and at most L
-// look-ups per candidate instead of C*K evaluations of the error.  (x - m)_+ is continuous in x: a value that falls on
-// the wrong side of a bin's edge by a rounding contributes the same to every P.
+// look-ups per candidate instead of C*K evaluations of the error.  A value has to be in its own bin: one at m + d that is put into
+// bin m - 1 is missing from P(m) with all of d, 4*(c+1)*d in the error of the candidate c whose threshold m is, and rows whose
+// values repeat add that up.  So bins are exact (lattice_bin).
 //
 // The counts and the fractional sums are integers in shared memory (32-bit shared atomics run at 12 values per clock
 // and SM, 64-bit and floating ones are compare-and-swap loops at a fifth of that or less), so the curve does not depend
-// on the order of the insertions.  What the fixed point and the binary32 bin edges can change is bounded by
+// on the order of the insertions.  What the fixed point and the rounding of the scales can change is bounded by
 // lattice_band(); the candidates within the bound of the smallest value are re-scored exactly by the caller.
 //
 // Measured on one B200 against a sweep of all candidates over all values that they do not code as 0, 1024 candidates: 4096 x
@@ -233,17 +234,28 @@ __device__ __forceinline__ void lattice_each(const BlockTeam& tm, const LatticeR
     }
 }
 
+// The bin m of a >= h and the remainder r = a - m*h, 0 <= r < h.  inv_up exceeds 1/h by 2.3e-7 to 4.8e-7 of it, so floor(a*inv_up)
+// is m or, where it is the bin above, the remainder is negative (a/h < 2^21).  No rounding: r is a multiple of the last place of h.
+__device__ __forceinline__ float lattice_inv_up(float inv) { return inv * (1.0f + 3.0e-7f); }
+__device__ __forceinline__ float lattice_bin(float a, float h, float inv_up, int& m) {
+    const float u = __fmaf_rd(a, inv_up, kMagic), r = fmaf(-(u - kMagic), h, a);    // M + floor
+    const bool above = r < 0.f;
+    m = magic_int(u) - (above ? 1 : 0);
+    return above ? r + h : r;
+}
+
 // Most the curve (in units of h^2) can be off by at a candidate that could be the minimum.  T = |x|/h, E = sum T^2.
 // A value's fractional part is off by at most 2^-(F+1) (rounding to the fixed point) + 2e-7 (binary32 evaluation), which
 // enters sum_j P_j once per level below it, times 4(c+1) <= 4T per level: 4*err*sum T <= 4*err*sqrt(K*E).  The extra
 // level's fixed point has D times fewer levels at D times larger T.  P itself is truncated to 2^-s: 4(c+1)*2^-s for at
 // most n_bins/(2(c+1)) + 2 levels.  The scale alpha_c differs from (c+1)*step by 2^-24, which moves the error by at most
-// 2*2^-24*sqrt(E*SSE) to first order.
+// 2*2^-24*sqrt(E*SSE) to first order.  The IEEE quotient x/alpha rounds a value within 2^-24*|x| of a threshold to either side; its
+// error, half a step squared, moves by 2*alpha*2^-24*|x|, and over the row again by at most 4*2^-24*sqrt(E*SSE).
 // st = sqrt(K*E), inv_f = 2^-F, inv_d_f2 = the coarse histogram's 2^-F divided by D.
 __device__ __forceinline__ float lattice_band(float dmin, float e, float st, float inv_f, float inv_d_f2, float truncation) {
     const float d = fmaxf(dmin, 0.f) + 1e-6f * e;            // e is a binary32 sum: the curve's zero is known to this
     const float noise = (2.0f * inv_f + 8e-7f + 4.0f * inv_d_f2) * st + truncation +
-                        2.4e-7f * sqrtf(d * e) + 1e-9f * e;
+                        3.6e-7f * sqrtf(d * e) + 1e-9f * e;
     return dmin + (float)kRescoreBand * d + 2.0f * noise;    // both the minimum's and the candidate's value may be off
 }
 
@@ -362,7 +374,7 @@ __device__ __forceinline__ float lattice_insert(const BlockTeam& tm, const Latti
     const float pre = TINY ? 18446744073709551616.0f : 1.0f;       // 2^64: keeps 1/h finite for the smallest steps
     const float h = __fmul_rn(__fmul_rn(step, pre), 0.5f);
     const float inv = __fdiv_rn(1.0f, h);
-    const float inv_dn = inv * (1.0f - 3.0e-7f);                    // never above |x|/h: fractional parts are >= 0
+    const float inv_up = lattice_inv_up(inv);
     const float inv_fix = inv * (float)(1 << fbits);
     const unsigned int rd = d > 0 ? (unsigned)((0x100000000ull + d - 1) / d) : 0u;   // m/d = (m*rd) >> 32 for m < 2^24
     const int d_from = d > 0 ? d : 0x7fffffff;
@@ -376,10 +388,9 @@ __device__ __forceinline__ float lattice_insert(const BlockTeam& tm, const Latti
             const float a = sgn ? fabsf(y) : y;                     // an unsigned range codes negative values as 0
             const float t = a * inv;
             e = fmaf(t, t, e);
-            const float u = __fmaf_rd(a, inv_dn, kMagic);           // M + floor(|x|/h)
-            const int m = magic_int(u);
-            if (m >= 1) {
-                const float r = fmaf(-(u - kMagic), h, a);
+            if (a >= h) {
+                int m;
+                const float r = lattice_bin(a, h, inv_up, m);
                 const unsigned int fi = (unsigned)magic_int(fmaf(r, inv_fix, kMagic));
                 const int w = lattice_word(min(m, n_bins) - 1, lb);
                 Counts<PACKED>::add(sm.n, w);
@@ -559,11 +570,12 @@ __device__ __forceinline__ LatticeResult lattice_search_wide(const BlockTeam& tm
     res.step = gr.step;
     const bool tiny = !(gr.step > 1e-30f);
     const float pre = tiny ? 18446744073709551616.0f : 1.0f;
-    const float h = __fmul_rn(__fmul_rn(gr.step, pre), 0.5f), inv = __fdiv_rn(1.0f, h), inv_dn = inv * (1.0f - 3.0e-7f);
+    const float h = __fmul_rn(__fmul_rn(gr.step, pre), 0.5f), inv = __fdiv_rn(1.0f, h), inv_up = lattice_inv_up(inv);
     const int fbits = lattice_fbits(k);
     const float inv_fix = inv * (float)(1 << fbits);
     const int win = g.window, lb = lattice_log_run(win, tm.n), padded = lattice_padded(win, tm.n);
-    const int n_bins = g.n_bins, n_win = (n_bins + win - 1) / win;
+    const int n_bins = g.n_bins, n_win = (n_bins + win - 1) / win;      // (2,084,864 bins at most)
+    const float far = (float)(n_bins + 2);
     for (int c = tm.t; c < g.n_cand; c += tm.n) sm.curve[c] = 0.f;      // explained share of E, per candidate
     double e_inv = 0.0;
     int windows = 0;
@@ -579,7 +591,9 @@ __device__ __forceinline__ LatticeResult lattice_search_wide(const BlockTeam& tm
             for (int j = 0; j < 4; ++j) {
                 const float a = x[j] * sg, t = a * inv;
                 e = fma((double)t, (double)t, e);
-                if (a * inv_dn >= (float)(n_bins + 1)) {
+                int m = 0;
+                if (a * inv_up < far) lattice_bin(a, h, inv_up, m);
+                if (m > n_bins || !(a * inv_up < far)) {
                     over_n += 1.0;
                     over_s += (double)t - (double)(n_bins + 1);
                 }
@@ -614,12 +628,14 @@ __device__ __forceinline__ LatticeResult lattice_search_wide(const BlockTeam& tm
                 const float x[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const float a = x[j] * sg, td = a * inv_dn;
-                    if (td >= (float)(base + 1) && td < (float)(base + win + 1) && td < (float)(n_bins + 1)) {
-                        const float mf = floorf(td);
-                        const int w = lattice_word((int)mf - 1 - base, lb);
+                    const float a = x[j] * sg;
+                    if (!(a >= h) || !(a * inv_up < far)) continue;
+                    int m;
+                    const float r = lattice_bin(a, h, inv_up, m);
+                    if (m > base && m <= base + win && m <= n_bins) {
+                        const int w = lattice_word(m - 1 - base, lb);
                         atomicAdd(sm.n + w, 1u);
-                        atomicAdd(sm.f + w, (unsigned)magic_int(fmaf(fmaf(-mf, h, a), inv_fix, kMagic)));
+                        atomicAdd(sm.f + w, (unsigned)magic_int(fmaf(r, inv_fix, kMagic)));
                     }
                 }
             }

@@ -89,3 +89,17 @@ def test_per_tensor_search_on_lattice_values(case, path):
         ref = orc.phi(x, bits, signed, n_cand, hi_frac, 3, start_idx=idx, want_codes=False)
     assert alpha == pytest.approx(ref.alpha, rel=1e-5, abs=0)
     assert sse == pytest.approx(ref.sse, rel=1e-5, abs=1e-37)
+
+
+@pytest.mark.parametrize("hi_frac", [1.0, 0.03])           # all bins at once; bins in windows, values above the last threshold
+@pytest.mark.parametrize("case", range(len(TENSORS)), ids=[t[0] for t in TENSORS])
+def test_rows_on_lattice_values(case, hi_frac):
+    import gpu_util
+    from parity import check_rows
+    _, make, bits, signed, n_cand = TENSORS[case]
+    x = make().astype(np.float32)
+    n_cand = n_cand if hi_frac == 1.0 else 4000
+    w = np.resize(np.random.default_rng(5).permutation(x), (3, 900))
+    w[:, 0] = np.abs(x).max() / np.float32(hi_frac)
+    alpha, sse, idx, q, _ = gpu_util.quantize_weights(w, bits, signed, n_cand, hi_frac, 3, True, False)
+    check_rows(w, alpha, sse, idx, q, None, bits, signed, n_cand, hi_frac, 3)
