@@ -926,8 +926,10 @@ int omse_dual_quantize(omse_ctx* ctx, const float* d_t, int64_t n_kernels, int64
     a.packed = d_packed;
     a.status = &ctx->ws->status;
     a.rows_per_unit = (d_packed && (kernel_len & 1)) ? 2 : 1;
-    // Which of the two kernels: see dual_bound_kernel
-    const bool bound = kernel_len >= OMSE_DUAL_BOUND_K && bits1 + bits2 <= 8 && grid->hi_frac2 <= 1.0f;
+    // Which of the two kernels: see dual_bound_kernel.  Where alpha1 comes near the last place of max|x| (2^-23 of it) binary32 cannot
+    // tell neighbouring first codes apart and the reference takes the lowest one, which only the full enumeration finds.
+    const bool bound = kernel_len >= OMSE_DUAL_BOUND_K && bits1 + bits2 <= 8 && grid->hi_frac2 <= 1.0f &&
+                       (double)grid->hi_frac1 * 1048576.0 >= (double)grid->n_cand1;
     const long long n_units = (n_kernels + a.rows_per_unit - 1) / a.rows_per_unit;
     const bool few = n_units <= 3ll * ctx->n_sm;
     const int id = !bound ? 0 : few ? 1 : 2;

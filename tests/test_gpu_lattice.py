@@ -153,6 +153,9 @@ def test_per_tensor_searches_of_every_kind(n, bits, signed, n_cand, hi_frac, sca
     (3, 600, 4, 4, True, 12, 12, 3.0, 0.25, 1.0),       # scales beyond max|x|
     (3, 600, 4, 4, True, 8, 8, 1.0, 0.25, 2.0 ** -95),  # small values
     (2, 28672, 2, 3, True, 6, 6, 1.0, 0.25, 1.0),       # the longest row
+    (3, 400, 4, 4, True, 4, 4, 1e-5, 0.25, 1.0),        # first scale far below max|x| ...
+    (3, 400, 4, 4, True, 5, 5, 1e-7, 0.25, 1.0),        # ... and below its last place: equal errors take the lowest first code
+    (3, 400, 3, 3, False, 5, 5, 1e-9, 0.5, 1.0),
 ])
 def test_dual_search_by_bounds(s, k, bits1, bits2, signed, c1, c2, hf1, hf2, scale):
     import gpu_util
