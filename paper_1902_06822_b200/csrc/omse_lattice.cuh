@@ -576,8 +576,9 @@ __device__ __forceinline__ LatticeResult lattice_search_wide(const BlockTeam& tm
     const int win = g.window, lb = lattice_log_run(win, tm.n), padded = lattice_padded(win, tm.n);
     const int n_bins = g.n_bins, n_win = (n_bins + win - 1) / win;      // (2,084,864 bins at most)
     const float far = (float)(n_bins + 2);
+    const double inv_d = 1.0 / (double)h;
     for (int c = tm.t; c < g.n_cand; c += tm.n) sm.curve[c] = 0.f;      // explained share of E, per candidate
-    double e_inv = 0.0;
+    double e_inv = 0.0, root = 0.0;
     int windows = 0;
     for (int side = 0; side < (g.flo < 0 ? 2 : 1); ++side) {
         const int levels = side == 0 ? g.fhi : -g.flo;
@@ -589,13 +590,14 @@ __device__ __forceinline__ LatticeResult lattice_search_wide(const BlockTeam& tm
             const float x[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const float a = x[j] * sg, t = a * inv;
-                e = fma((double)t, (double)t, e);
+                const float a = x[j] * sg;
+                const double t = (double)a * inv_d;                // (may leave binary32: the grid can end anywhere below max|x|)
+                e = fma(t, t, e);
                 int m = 0;
                 if (a * inv_up < far) lattice_bin(a, h, inv_up, m);
                 if (m > n_bins || !(a * inv_up < far)) {
                     over_n += 1.0;
-                    over_s += (double)t - (double)(n_bins + 1);
+                    over_s += t - (double)(n_bins + 1);
                 }
             }
         }
@@ -617,6 +619,7 @@ __device__ __forceinline__ LatticeResult lattice_search_wide(const BlockTeam& tm
             et += ts->wide_e[w];
         }
         e_inv = 1.0 / et;
+        root = sqrt(e_inv);                                        // P is kept as P/sqrt(E): at most sqrt(K)
         for (int wi = n_win - 1; wi >= 0; --wi) {
             const int base = wi * win;                             // bins m = base+1 .. base+win
             ++windows;
@@ -674,7 +677,7 @@ __device__ __forceinline__ LatticeResult lattice_search_wide(const BlockTeam& tm
                 ds += dn;
                 dn += (double)sm.n[w];
                 df += (double)sm.f[w];
-                reinterpret_cast<float*>(sm.f)[w] = (float)fma(df, fq, ds);
+                reinterpret_cast<float*>(sm.f)[w] = (float)(fma(df, fq, ds) * root);
             }
             __syncthreads();
             const int top = min(base + win, n_bins);
@@ -684,7 +687,7 @@ __device__ __forceinline__ LatticeResult lattice_search_wide(const BlockTeam& tm
                 double acc = 0.0;
                 for (; j <= levels && (2 * j - 1) * a1 <= top; ++j)
                     acc += (double)reinterpret_cast<const float*>(sm.f)[lattice_word((2 * j - 1) * a1 - 1 - base, lb)];
-                sm.curve[c] += (float)(4.0 * (double)a1 * acc * e_inv);
+                sm.curve[c] += (float)(4.0 * (double)a1 * acc * root);
             }
         }
     }

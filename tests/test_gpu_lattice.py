@@ -15,6 +15,9 @@ pytestmark = pytest.mark.gpu
     (5, 700, 4, False, 4096, 1.0 / 15, 1.0),
     (3, 9001, 8, True, 4096, 1.0 / 127, 1.0),
     (4, 300, 2, True, 4096, 1e-3, 1.0),             # most values beyond the last threshold of every candidate
+    (3, 300, 8, True, 4096, 1e-36, 1.0),            # ... by more than binary32 holds
+    (3, 300, 4, True, 4096, 1e-37, 2.0 ** 50),
+    (2000, 300, 8, True, 4096, 1e-36, 1.0),
     (4, 28672, 3, True, 4096, 1.0, 1.0),            # the longest row with the most candidates
     (6, 500, 4, True, 256, 3.0, 1.0),               # fewer bins than candidates
     (6, 500, 4, True, 1000, 40.0, 1.0),
