@@ -865,7 +865,9 @@ struct ResidentArgs {
 // block polls the slot of block b.  No counter that all blocks would have to add to one after the other, no fence between
 // data and flag, and one trip to L2 each way.  Slots alternate between two sets: a block can only be one exchange ahead,
 // since it waits for everybody's slot of this one.  Tags count the exchanges of a call from 1; the last block of a call
-// clears the slots.  A slot that does not appear within kSpinLimit polls sets s_bad, and the search ends without a result.
+// clears the slots.  Slots are stored and loaded with relaxed order.  Where an exchange stands for more than its slots (DATA: the
+// histogram, the errors of the re-scored candidates), thread 0 fences between the barrier behind which the block's writes lie
+// and its slot, and the polling threads fence between the slots they saw and the barrier that lets the block read.  A slot that does not appear within kSpinLimit polls sets s_bad, and the search ends without a result.
 struct ResidentTeam {
     ResidentExchange* ex;
     unsigned int step;               // exchanges so far
@@ -877,13 +879,18 @@ __device__ __forceinline__ void slot_store(ResidentSlot* p, unsigned long long a
 __device__ __forceinline__ void slot_load(const ResidentSlot* p, unsigned long long& a, unsigned long long& b) {
     asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}" : "=l"(a), "=l"(b) : "l"(p) : "memory");
 }
-// publishes (thread 0 of the block)
+__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+// publishes (thread 0 of the block, after a barrier)
+template <bool DATA>
 __device__ __forceinline__ void resident_publish(ResidentTeam& t, unsigned long long a, unsigned long long b40) {
     ++t.step;
-    if (threadIdx.x == 0)
+    if (threadIdx.x == 0) {
+        if (DATA) fence_gpu();
         slot_store(&t.ex->slot[t.step & 1][blockIdx.x], a, ((unsigned long long)t.step << 40) | b40);
+    }
 }
-// thread b < gridDim.x gets block b's slot; others get `none`
+// thread b < gridDim.x gets block b's slot; others get `none`.  A barrier has to follow before the block reads what came with them.
+template <bool DATA>
 __device__ __forceinline__ void resident_collect(ResidentTeam& t, unsigned long long& a, unsigned long long& b40,
                                                  unsigned long long none_a) {
     a = none_a;
@@ -901,15 +908,17 @@ __device__ __forceinline__ void resident_collect(ResidentTeam& t, unsigned long 
         } else {
             *t.s_bad = 1;
         }
+        if (DATA) fence_gpu();
     }
 }
 // Sum of a double and of a non-negative integer below 2^40 over all threads of all blocks, in a fixed order; every thread
 // gets it.  False: see above.
+template <bool DATA>
 __device__ __forceinline__ bool resident_sum(ResidentTeam& t, double& d, long long& q, double* scratch) {
     block_sum2(d, q, scratch);
-    resident_publish(t, (unsigned long long)__double_as_longlong(d), (unsigned long long)q);
+    resident_publish<DATA>(t, (unsigned long long)__double_as_longlong(d), (unsigned long long)q);
     unsigned long long ua, ub;
-    resident_collect(t, ua, ub, 0ull);
+    resident_collect<DATA>(t, ua, ub, 0ull);
     d = __longlong_as_double((long long)ua);
     q = (long long)ub;
     block_sum2(d, q, scratch);
@@ -997,9 +1006,9 @@ __global__ void __launch_bounds__(kResidentThreads) tensor_resident_kernel(const
     };
     block_extremes();
     {
-        resident_publish(team, ((unsigned long long)(unsigned)kmax << 32) | (unsigned)kmin, nonfinite);
+        resident_publish<false>(team, ((unsigned long long)(unsigned)kmax << 32) | (unsigned)kmin, nonfinite);
         unsigned long long ua, ub;
-        resident_collect(team, ua, ub, 0x800000007fffffffull);
+        resident_collect<false>(team, ua, ub, 0x800000007fffffffull);
         kmin = (int)(unsigned)ua;
         kmax = (int)(unsigned)(ua >> 32);
         nonfinite = (unsigned)ub;
@@ -1075,11 +1084,9 @@ __global__ void __launch_bounds__(kResidentThreads) tensor_resident_kernel(const
             atomicAdd(gh + (coarse ? 2 * kResidentBins : 0) + b, (unsigned long long)c);
             atomicAdd(gh + (coarse ? 3 * kResidentBins : kResidentBins) + b, f);
         }
-        __threadfence();                                            // this thread's additions before the block's slot
         long long none = 0;
         double sum_sq = sq;
-        ok = resident_sum(team, sum_sq, near, scratch) && ok;       // every block's additions are in L2 after this (near < 2^29 per block)
-        __threadfence();
+        ok = resident_sum<true>(team, sum_sq, near, scratch) && ok; // every block's additions are known after this (near < 2^29 per block)
         // ---- N, P and the curve, in every block
         const double unit = hist_unit(gr.step);
         double cn = 0.0, cs = 0.0, cf = 0.0;
@@ -1161,11 +1168,9 @@ __global__ void __launch_bounds__(kResidentThreads) tensor_resident_kernel(const
                 const double ss = slice_error(__fmul_rn((float)(list[l] + 1), gr.step));
                 if (tid == 0) r.rescore[(size_t)l * nblk + blockIdx.x] = ss;
             }
-            __threadfence();
             double nothing = 0.0;
             none = 0;
-            ok = resident_sum(team, nothing, none, scratch) && ok;  // (only its waiting is wanted)
-            __threadfence();
+            ok = resident_sum<true>(team, nothing, none, scratch) && ok;     // (only its waiting is wanted)
             double best_sse = INFINITY;
             int bc = 0x7fffffff;
             for (int l = warp; l < n_list; l += kResidentThreads / 32) {
@@ -1207,7 +1212,7 @@ __global__ void __launch_bounds__(kResidentThreads) tensor_resident_kernel(const
             }
             if (tid < tail) one(tailp[tid]);
             sqq += s32;
-            ok = resident_sum(team, sxq, sqq, scratch) && ok;
+            ok = resident_sum<false>(team, sxq, sqq, scratch) && ok;
             if (sqq == 0) break;
             const float a_new = (float)(sxq / (double)sqq);
             if (!(a_new >= FLT_MIN) || !(a_new <= FLT_MAX) || a_new == alpha) break;

@@ -1,0 +1,37 @@
+"""The exchanges between the blocks of the one-kernel per-tensor search."""
+import numpy as np
+import pytest
+
+from paper_1902_06822_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _outputs(n_cand):
+    import torch
+    return (torch.zeros(1, device="cuda"), torch.zeros(1, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda"),
+            torch.zeros(n_cand, dtype=torch.float64, device="cuda"))
+
+
+@pytest.mark.parametrize("n,bits,n_cand", [(1_605_633, 8, 500), (303_105, 4, 1024), (25_088, 4, 50)])
+def test_repeated_searches_give_the_same_bits(n, bits, n_cand):
+    """Every block sees all additions to the histogram and all re-scored errors: calls in a row on two tensors in turn."""
+    import torch
+
+    import gpu_util
+    from oracle import omse_oracle as orc
+    xs = [np.abs(synth.student_t3(n, seed=61 + i)) for i in range(2)]
+    xs[1] = np.round(xs[1] * np.float32(8)) * np.float32(0.125)        # many candidates to re-score
+    d_xs = [torch.from_numpy(x).cuda() for x in xs]
+    first = []
+    for rep in range(150):
+        for i, d_x in enumerate(d_xs):
+            out = _outputs(n_cand)
+            gpu_util.ctx().omse_activation_scale(d_x, n, bits, False, n_cand, 1.0, 3, *out)
+            if rep == 0:
+                first.append(out)
+            else:
+                assert all(torch.equal(a, b) for a, b in zip(out, first[i])), (rep, i)
+    for x, out in zip(xs, first):
+        ref = orc.activation_scale(x, bits, False, n_cand, 1.0, 3)
+        assert out[0].item() == pytest.approx(ref.alpha, rel=1e-5) and out[1].item() == pytest.approx(ref.sse, rel=1e-5)
