@@ -58,8 +58,8 @@ typedef enum {
 
 /* bits of the device status word */
 #define OMSE_DEV_NONFINITE 1u  /* a NaN or Inf was read from an input tensor                          */
-#define OMSE_DEV_INCOMPLETE 4u /* blocks of a per-tensor search gave up waiting for one another: its outputs are not valid */
 #define OMSE_DEV_DEGENERATE 2u /* a segment had max|x| = 0 (or below FLT_MIN*C): alpha=0, codes 0 */
+#define OMSE_DEV_INCOMPLETE 4u /* blocks of a per-tensor search gave up waiting for one another: its outputs are not valid */
 
 /* Largest supported sizes. */
 #define OMSE_MAX_CANDIDATES 4096   /* n_cand                                                        */
@@ -396,6 +396,12 @@ int omse_read_evaluations(omse_ctx* ctx, uint64_t* host_out);
  * row path present (long rows, rows of up to 1024 elements), the per-tensor search one, for tensors that fit on chip, or
  * ten or so. */
 int omse_read_launches(omse_ctx* ctx, uint64_t* host_out);
+
+/* Instrumentation (no counterpart in the paper): how often a block of a per-tensor search that runs in one kernel looks for what
+ * another block has to say before it gives up (default 2^22 times, some seconds; the blocks all run at once, so waiting is
+ * a matter of microseconds unless the GPU is stopped under them).  Such a call sets OMSE_DEV_INCOMPLETE in the device status, and
+ * the next call is not affected.  0: every wait ends at once. */
+int omse_set_poll_limit(omse_ctx* ctx, uint32_t polls);
 
 /* Instrumentation (no counterpart in the paper): runs a register-only loop of independent fma.rn.f32x2 on every SM
  * for about target_ms milliseconds (1..5000) on the context's stream, synchronises, and returns in *host_out the

@@ -15,7 +15,7 @@ import torch
 from . import build as _build
 
 OK, EINVAL, ECUDA, ENOMEM, ELIMIT = 0, -1, -2, -3, -4
-DEV_NONFINITE, DEV_DEGENERATE = 1, 2
+DEV_NONFINITE, DEV_DEGENERATE, DEV_INCOMPLETE = 1, 2, 4
 MAX_CANDIDATES, MAX_KERNEL_LEN, MAX_KERNEL_LEN_MULTISWEEP, MAX_TENSORS = 4096, 28672, 25600, 4
 STATIC_MAX_CANDIDATES = 2048
 
@@ -26,7 +26,7 @@ EXPORTS = [
     "omse_activation_scale", "omse_residual_quantize", "omse_pack_int4", "omse_last_device_status",
     "omse_status_string", "omse_activation_scale_static", "omse_alg1_quantize_converge",
     "omse_quantize_weights_solver", "omse_quantize_weights_affine", "omse_quantize_key_layers",
-    "omse_measure_fp32_peak", "omse_read_launches",
+    "omse_measure_fp32_peak", "omse_read_launches", "omse_set_poll_limit",
 ]
 SOLVER_GRID, SOLVER_UNIFORM, SOLVER_ALTERNATING, SOLVER_GOLDEN = 0, 1, 2, 3
 MAX_OFFSETS = 64
@@ -107,6 +107,7 @@ def load_library() -> C.CDLL:
     lib.omse_last_device_status.argtypes = [vp, C.POINTER(C.c_uint32)]
     lib.omse_read_evaluations.argtypes = [vp, C.POINTER(C.c_uint64)]
     lib.omse_measure_fp32_peak.argtypes = [vp, i32, C.POINTER(C.c_double)]
+    lib.omse_set_poll_limit.argtypes = [vp, C.c_uint32]
     lib.omse_read_launches.argtypes = [vp, C.POINTER(C.c_uint64)]
     lib.omse_status_string.argtypes = [i32]
     lib.omse_status_string.restype = C.c_char_p
@@ -368,6 +369,12 @@ class Context:
         if rc != OK:
             raise OmseError(rc, "omse_read_launches")
         return out.value
+
+    def omse_set_poll_limit(self, polls: int):
+        """Polls before a block of a one-kernel per-tensor search gives up (DEV_INCOMPLETE in the device status)."""
+        rc = load_library().omse_set_poll_limit(self._h, polls)
+        if rc != OK:
+            raise OmseError(rc, "omse_set_poll_limit")
 
     def omse_measure_fp32_peak(self, target_ms: int = 200) -> float:
         """Measured FP32 lane operations per second of the FMA pipe (packed fma loop on every SM)."""

@@ -70,6 +70,7 @@ struct omse_ctx {
     int n_seen, next_seen;
     TensorLaunches tensor;                          // the same for the per-tensor kernels
     unsigned long long n_launches;                  // kernels launched since the last omse_read_launches
+    unsigned int poll_limit;                        // polls of the one-kernel per-tensor search (omse_set_poll_limit)
 };
 
 namespace {
@@ -348,7 +349,7 @@ int enqueue_tensor_search(const TensorEnv& env, omse::TensorArgs& a, int refine_
 
 // The search in one kernel, for tensors that fit in the shared memory of all SMs together.  Returns OMSE_ELIMIT, with
 // nothing enqueued, when this one does not.
-int enqueue_resident_search(const TensorEnv& env, omse::TensorArgs a, omse::ResidentExchange* ex, int refine_iters) {
+int enqueue_resident_search(const TensorEnv& env, omse::TensorArgs a, omse::ResidentExchange* ex, unsigned int poll_limit, int refine_iters) {
     if (a.n < 1 || a.n_cand > omse::kResidentCands) return OMSE_ELIMIT;
     tensor_bins(a);
     if (a.clipped || a.n_bins > omse::kResidentBins) return OMSE_ELIMIT;
@@ -361,6 +362,7 @@ int enqueue_resident_search(const TensorEnv& env, omse::TensorArgs a, omse::Resi
     r.ex = ex;
     r.slice4 = (int)((n4 + blocks - 1) / blocks);
     r.rescore = a.partials;
+    r.spin_limit = poll_limit;
     if (!env.seen->attr_resident) {
         if (cudaFuncSetAttribute(omse::tensor_resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess)
             return OMSE_ECUDA;
@@ -555,6 +557,7 @@ int omse_create(omse_ctx** out, int device, void* cuda_stream) {
     c->ws = nullptr;
     c->partials = nullptr;
     c->d_tensors = nullptr;
+    c->poll_limit = omse::kSpinLimit;
     if (cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
         delete c;
         return OMSE_ECUDA;
@@ -628,6 +631,12 @@ int omse_read_launches(omse_ctx* ctx, uint64_t* host_out) {
     if (!ctx || !host_out) return OMSE_EINVAL;
     *host_out = ctx->n_launches;
     ctx->n_launches = 0;
+    return OMSE_OK;
+}
+
+int omse_set_poll_limit(omse_ctx* ctx, uint32_t polls) {
+    if (!ctx) return OMSE_EINVAL;
+    ctx->poll_limit = polls;
     return OMSE_OK;
 }
 
@@ -1052,7 +1061,7 @@ static int activation_impl(omse_ctx* ctx, const float* d_x, int64_t n, int bits,
     a.evals = &ctx->ws->evals;
     a.status = &ctx->ws->status;
     const TensorEnv env = {ctx->n_sm, ctx->stream, &ctx->tensor, &ctx->n_launches};
-    const int rc = enqueue_resident_search(env, a, &ctx->ws->exchange, grid->refine_iters);
+    const int rc = enqueue_resident_search(env, a, &ctx->ws->exchange, ctx->poll_limit, grid->refine_iters);
     if (rc != OMSE_ELIMIT) return rc;
     omse::tensor_init_kernel<<<1, 32, 0, ctx->stream>>>(a.st);
     ++ctx->n_launches;

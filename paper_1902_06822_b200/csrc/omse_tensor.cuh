@@ -842,7 +842,7 @@ __global__ void __launch_bounds__(256) tensor_pass_kernel(const TensorArgs a) {
 constexpr int kResidentBlocks = 160;     // blocks the exchange area has room for
 constexpr int kResidentBins = 4096;      // bins of the histogram in the exchange area (and as many coarse ones)
 constexpr int kResidentCands = 1024;
-constexpr unsigned int kSpinLimit = 1u << 22;   // polls of a slot before a block gives up (seconds)
+constexpr unsigned int kSpinLimit = 1u << 22;   // polls of a slot before a block gives up (seconds), by default
 
 struct __align__(16) ResidentSlot {      // one block's contribution to an exchange: 64 bits, and 40 bits under a 24-bit tag
     unsigned long long a, b;
@@ -859,6 +859,7 @@ struct ResidentArgs {
     ResidentExchange* ex;
     int slice4;                          // float4s per block
     double* rescore;                     // [listed candidates][gridDim.x]
+    unsigned int spin_limit;             // polls of a slot before a block gives up
 };
 
 // An exchange between the blocks: every block publishes a slot, data and tag in one 16-byte store, and thread b of every
@@ -867,11 +868,13 @@ struct ResidentArgs {
 // since it waits for everybody's slot of this one.  Tags count the exchanges of a call from 1; the last block of a call
 // clears the slots.  Slots are stored and loaded with relaxed order.  Where an exchange stands for more than its slots (DATA: the
 // histogram, the errors of the re-scored candidates), thread 0 fences between the barrier behind which the block's writes lie
-// and its slot, and the polling threads fence between the slots they saw and the barrier that lets the block read.  A slot that does not appear within kSpinLimit polls sets s_bad, and the search ends without a result.
+// and its slot, and the polling threads fence between the slots they saw and the barrier that lets the block read.  A block
+// that does not see a slot within the limit of polls sets s_bad, goes on to the end without further exchanges, and reports it.
 struct ResidentTeam {
     ResidentExchange* ex;
     unsigned int step;               // exchanges so far
     int* s_bad;                      // shared: some slot did not appear
+    unsigned int spin_limit;
 };
 __device__ __forceinline__ void slot_store(ResidentSlot* p, unsigned long long a, unsigned long long b) {
     asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(p), "l"(a), "l"(b) : "memory");
@@ -897,12 +900,13 @@ __device__ __forceinline__ void resident_collect(ResidentTeam& t, unsigned long 
     b40 = 0ull;
     if (threadIdx.x < gridDim.x) {
         const ResidentSlot* p = &t.ex->slot[t.step & 1][threadIdx.x];
-        unsigned long long va, vb;
-        unsigned int polls = 0u;
-        do {
+        unsigned long long va = 0ull, vb = 0ull;
+        bool there = false;
+        for (unsigned int polls = 0u; !there && polls < t.spin_limit; ++polls) {
             slot_load(p, va, vb);
-        } while ((unsigned int)(vb >> 40) != t.step && ++polls < kSpinLimit);
-        if ((unsigned int)(vb >> 40) == t.step) {
+            there = (unsigned int)(vb >> 40) == t.step;
+        }
+        if (there) {
             a = va;
             b40 = vb & 0xffffffffffull;
         } else {
@@ -931,7 +935,7 @@ __global__ void __launch_bounds__(kResidentThreads) tensor_resident_kernel(const
     __shared__ double part[32][3];
     __shared__ int s_bad, s_last, s_count[33];
     ResidentExchange* ex = r.ex;
-    ResidentTeam team = {ex, 0u, &s_bad};
+    ResidentTeam team = {ex, 0u, &s_bad, r.spin_limit};
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nblk = gridDim.x;
     const int bins = a.win;                                         // n_bins rounded up to a multiple of 4
     // shared memory: the slice | N, P of the bins and coarse bins (the words of the histogram before that) | the curve | the list
@@ -1243,6 +1247,7 @@ __global__ void __launch_bounds__(kResidentThreads) tensor_resident_kernel(const
     block_sum2(ss, zero, scratch);
     if (tid == 0) {
         ex->fin[blockIdx.x] = ss;
+        if (!ok) atomicOr(a.status, 4u);                            // any block's: its share of the outputs is not of this search
         __threadfence();
         s_last = atomicAdd(&ex->ticket, 1u) == (unsigned)nblk - 1u;
     }
@@ -1259,7 +1264,7 @@ __global__ void __launch_bounds__(kResidentThreads) tensor_resident_kernel(const
             *a.sse_out = (float)v;
             if (a.idx_out) *a.idx_out = best;
             if (a.delta_out) *a.delta_out = delta;
-            const unsigned int st = (nonfinite ? 1u : 0u) | (best < 0 ? 2u : 0u) | (ok ? 0u : 4u);
+            const unsigned int st = (nonfinite ? 1u : 0u) | (best < 0 ? 2u : 0u);
             if (st) atomicOr(a.status, st);
             if (a.evals && usable) atomicAdd(a.evals, (unsigned long long)a.n);
         }

@@ -35,3 +35,32 @@ def test_repeated_searches_give_the_same_bits(n, bits, n_cand):
     for x, out in zip(xs, first):
         ref = orc.activation_scale(x, bits, False, n_cand, 1.0, 3)
         assert out[0].item() == pytest.approx(ref.alpha, rel=1e-5) and out[1].item() == pytest.approx(ref.sse, rel=1e-5)
+
+
+@pytest.mark.parametrize("n", [303_105, 25_088, 100])
+def test_a_wait_that_runs_out_is_reported_and_leaves_no_trace(n):
+    """With few polls allowed (or none) blocks give up: the status says so, and calls before and after are not affected."""
+    import torch
+
+    from paper_1902_06822_b200 import binding
+    ctx = binding.Context(0)
+    d_x = torch.from_numpy(np.abs(synth.student_t3(n, seed=65))).cuda()
+
+    def search():
+        out = _outputs(300)
+        ctx.omse_activation_scale(d_x, n, 4, False, 300, 1.0, 3, *out)
+        return out, ctx.omse_last_device_status()
+
+    good, status = search()
+    assert status == 0
+    for polls in [0, 1, 2, 3, 4, 8, 16, 32, 64] * 3:
+        ctx.omse_set_poll_limit(polls)
+        out, status = search()
+        if polls == 0:
+            assert status & binding.DEV_INCOMPLETE
+        if not status & binding.DEV_INCOMPLETE:        # nobody gave up: the result is whole
+            assert status == 0 and all(torch.equal(a, b) for a, b in zip(out, good))
+        ctx.omse_set_poll_limit(1 << 22)
+        out, status = search()
+        assert status == 0 and all(torch.equal(a, b) for a, b in zip(out, good)), polls
+    ctx.close()
