@@ -403,6 +403,11 @@ int omse_read_launches(omse_ctx* ctx, uint64_t* host_out);
  * the next call is not affected.  0: every wait ends at once. */
 int omse_set_poll_limit(omse_ctx* ctx, uint32_t polls);
 
+/* Instrumentation (no counterpart in the paper): blocks that a per-tensor search in one kernel is launched with at most (1..160; default
+ * one per SM of the device).  Where the GPU cannot run that many at once - the number set here is too large, or a context
+ * or stream is limited to some of the SMs - the launch is refused and the search goes through a sequence of launches instead. */
+int omse_set_search_blocks(omse_ctx* ctx, int blocks);
+
 /* Instrumentation (no counterpart in the paper): runs a register-only loop of independent fma.rn.f32x2 on every SM
  * for about target_ms milliseconds (1..5000) on the context's stream, synchronises, and returns in *host_out the
  * measured FP32 lane operations per second of the FMA pipe (a packed instruction counts as two).  This is the

@@ -27,6 +27,7 @@ EXPORTS = [
     "omse_status_string", "omse_activation_scale_static", "omse_alg1_quantize_converge",
     "omse_quantize_weights_solver", "omse_quantize_weights_affine", "omse_quantize_key_layers",
     "omse_measure_fp32_peak", "omse_read_launches", "omse_set_poll_limit",
+    "omse_set_search_blocks",
 ]
 SOLVER_GRID, SOLVER_UNIFORM, SOLVER_ALTERNATING, SOLVER_GOLDEN = 0, 1, 2, 3
 MAX_OFFSETS = 64
@@ -107,6 +108,7 @@ def load_library() -> C.CDLL:
     lib.omse_last_device_status.argtypes = [vp, C.POINTER(C.c_uint32)]
     lib.omse_read_evaluations.argtypes = [vp, C.POINTER(C.c_uint64)]
     lib.omse_measure_fp32_peak.argtypes = [vp, i32, C.POINTER(C.c_double)]
+    lib.omse_set_search_blocks.argtypes = [vp, i32]
     lib.omse_set_poll_limit.argtypes = [vp, C.c_uint32]
     lib.omse_read_launches.argtypes = [vp, C.POINTER(C.c_uint64)]
     lib.omse_status_string.argtypes = [i32]
@@ -375,6 +377,12 @@ class Context:
         rc = load_library().omse_set_poll_limit(self._h, polls)
         if rc != OK:
             raise OmseError(rc, "omse_set_poll_limit")
+
+    def omse_set_search_blocks(self, blocks: int):
+        """Blocks of a one-kernel per-tensor search at most."""
+        rc = load_library().omse_set_search_blocks(self._h, blocks)
+        if rc != OK:
+            raise OmseError(rc, "omse_set_search_blocks")
 
     def omse_measure_fp32_peak(self, target_ms: int = 200) -> float:
         """Measured FP32 lane operations per second of the FMA pipe (packed fma loop on every SM)."""

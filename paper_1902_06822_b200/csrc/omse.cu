@@ -71,6 +71,7 @@ struct omse_ctx {
     TensorLaunches tensor;                          // the same for the per-tensor kernels
     unsigned long long n_launches;                  // kernels launched since the last omse_read_launches
     unsigned int poll_limit;                        // polls of the one-kernel per-tensor search (omse_set_poll_limit)
+    int search_blocks;                              // its blocks at most (omse_set_search_blocks)
 };
 
 namespace {
@@ -348,15 +349,17 @@ int enqueue_tensor_search(const TensorEnv& env, omse::TensorArgs& a, int refine_
 }
 
 // The search in one kernel, for tensors that fit in the shared memory of all SMs together.  Returns OMSE_ELIMIT, with
-// nothing enqueued, when this one does not.
-int enqueue_resident_search(const TensorEnv& env, omse::TensorArgs a, omse::ResidentExchange* ex, unsigned int poll_limit, int refine_iters) {
+// nothing enqueued, when this one does not, or when fewer SMs are there than the device has (a context or a stream limited to some
+// of them, other users of a shared GPU): the launch is then refused, since the blocks would wait for ones that cannot run.
+int enqueue_resident_search(const TensorEnv& env, omse::TensorArgs a, omse::ResidentExchange* ex, int max_blocks, unsigned int poll_limit,
+                            int refine_iters) {
     if (a.n < 1 || a.n_cand > omse::kResidentCands) return OMSE_ELIMIT;
     tensor_bins(a);
     if (a.clipped || a.n_bins > omse::kResidentBins) return OMSE_ELIMIT;
     a.win = (a.n_bins + 3) & ~3;
     const size_t fixed = (size_t)(a.win + a.n_bins2) * 16 + (size_t)a.n_cand * 12 + 16;
     const long long n4 = (a.n + 3) >> 2, fit4 = (long long)((kMaxSmem - fixed) / 16);
-    const long long blocks = std::min((long long)std::min(env.n_sm, omse::kResidentBlocks), (n4 + omse::kResidentThreads - 1) / omse::kResidentThreads);
+    const long long blocks = std::min((long long)max_blocks, (n4 + omse::kResidentThreads - 1) / omse::kResidentThreads);
     if ((n4 + blocks - 1) / blocks > fit4 || (long long)a.n_cand * blocks > a.partial_doubles) return OMSE_ELIMIT;
     omse::ResidentArgs r;
     r.ex = ex;
@@ -381,8 +384,12 @@ int enqueue_resident_search(const TensorEnv& env, omse::TensorArgs a, omse::Resi
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, omse::tensor_resident_kernel, (const omse::TensorArgs)a, (const omse::ResidentArgs)r, refine_iters);
+    if (e != cudaSuccess) {
+        cudaGetLastError();                         // not left for the next check of this thread
+        return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources || e == cudaErrorNotSupported ? OMSE_ELIMIT : OMSE_ECUDA;
+    }
     ++*env.launches;
-    return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? OMSE_OK : OMSE_ECUDA;
+    return OMSE_OK;
 }
 
 }  // namespace
@@ -562,6 +569,7 @@ int omse_create(omse_ctx** out, int device, void* cuda_stream) {
         delete c;
         return OMSE_ECUDA;
     }
+    c->search_blocks = std::min(c->n_sm, omse::kResidentBlocks);
     if (cudaMalloc(&c->ws, sizeof(Workspace)) != cudaSuccess || cudaMalloc(&c->partials, kPartialBytes) != cudaSuccess ||
         cudaMalloc(&c->d_tensors, sizeof(omse::RowTensor) * OMSE_MAX_BATCH) != cudaSuccess) {
         cudaFree(c->ws);
@@ -631,6 +639,12 @@ int omse_read_launches(omse_ctx* ctx, uint64_t* host_out) {
     if (!ctx || !host_out) return OMSE_EINVAL;
     *host_out = ctx->n_launches;
     ctx->n_launches = 0;
+    return OMSE_OK;
+}
+
+int omse_set_search_blocks(omse_ctx* ctx, int blocks) {
+    if (!ctx || blocks < 1 || blocks > omse::kResidentBlocks) return OMSE_EINVAL;
+    ctx->search_blocks = blocks;
     return OMSE_OK;
 }
 
@@ -1061,7 +1075,7 @@ static int activation_impl(omse_ctx* ctx, const float* d_x, int64_t n, int bits,
     a.evals = &ctx->ws->evals;
     a.status = &ctx->ws->status;
     const TensorEnv env = {ctx->n_sm, ctx->stream, &ctx->tensor, &ctx->n_launches};
-    const int rc = enqueue_resident_search(env, a, &ctx->ws->exchange, ctx->poll_limit, grid->refine_iters);
+    const int rc = enqueue_resident_search(env, a, &ctx->ws->exchange, ctx->search_blocks, ctx->poll_limit, grid->refine_iters);
     if (rc != OMSE_ELIMIT) return rc;
     omse::tensor_init_kernel<<<1, 32, 0, ctx->stream>>>(a.st);
     ++ctx->n_launches;

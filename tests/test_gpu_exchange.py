@@ -64,3 +64,37 @@ def test_a_wait_that_runs_out_is_reported_and_leaves_no_trace(n):
         out, status = search()
         assert status == 0 and all(torch.equal(a, b) for a, b in zip(out, good)), polls
     ctx.close()
+
+
+def test_a_refused_launch_takes_the_sequence_of_launches():
+    """More blocks than the GPU runs at once (each takes most of an SM's shared memory): the driver refuses, the call does not."""
+    import torch
+
+    from oracle import omse_oracle as orc
+    from paper_1902_06822_b200 import binding
+    n = 160 * 40_000                                    # 160 KB of values per block
+    if torch.cuda.get_device_properties(0).multi_processor_count >= 160:
+        pytest.skip("as many SMs as the search has blocks at most")
+    ctx = binding.Context(0)
+    x = np.abs(synth.student_t3(n, seed=66))
+    d_x = torch.from_numpy(x).cuda()
+    ctx.omse_set_search_blocks(160)
+    out = _outputs(100)
+    ctx.omse_read_launches()
+    ctx.omse_activation_scale(d_x, n, 4, False, 100, 1.0, 3, *out)
+    assert ctx.omse_last_device_status() == 0
+    assert ctx.omse_read_launches() > 5                 # not in one kernel
+    ref = orc.activation_scale(x, 4, False, 100, 1.0, 3)
+    assert out[2].item() == ref.best_idx and out[0].item() == pytest.approx(ref.alpha, rel=1e-5)
+    assert out[1].item() == pytest.approx(ref.sse, rel=1e-5)
+    # nothing of the refusal is left for the next call, whatever its path
+    w = torch.from_numpy(synth.student_t3(64 * 300, seed=67)).cuda()
+    a, s = torch.zeros(64, device="cuda"), torch.zeros(64, device="cuda")
+    ctx.omse_quantize_weights(w, 64, 300, 4, True, 100, 1.0, 3, a, s)
+    ctx.omse_set_search_blocks(20)                      # fewer blocks than SMs: in one kernel again
+    small = _outputs(100)
+    ctx.omse_activation_scale(d_x, 303_105, 4, False, 100, 1.0, 3, *small)
+    assert ctx.omse_last_device_status() == 0 and ctx.omse_read_launches() == 2
+    ref = orc.activation_scale(x[:303_105], 4, False, 100, 1.0, 3)
+    assert small[2].item() == ref.best_idx and small[0].item() == pytest.approx(ref.alpha, rel=1e-5)
+    ctx.close()
