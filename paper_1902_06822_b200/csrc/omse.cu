@@ -185,9 +185,21 @@ int launch_rows(omse_ctx* ctx, omse::RowArgs& a, long long max_k, int path) {
     if (path == kPathShort)
         return launch_rows_kernel(ctx, a, path, ext, omse::kShortThreads, (size_t)(omse::kShortThreads / 32) * a.short_bytes);
     const size_t fixed = (size_t)(a.keep_x0 ? 2 : 1) * k4 * 16 + omse::kScratchDoubles * 8 + 8 * 4;
-    int threads = max_k >= 8192 ? 512 : 128;
+    a.direct = -1;
+    a.window = 0;
+    int threads = 0;
     size_t smem = 0;
-    if (bins > 0 && (double)bins * (double)max_k < 2147483648.0) {
+    // Rows that are shorter than this evaluate candidates instead of making a histogram.  In a small launch a row's chain of steps
+    // counts, in a large one the barriers: 32 threads per row then.  (Two tensors of 4 bits, 1024 candidates, histogram and candidates:
+    // 38,836 rows of 27 values 993 us and 326, 16,384 of 64 429 and 203, 10,485 of 100 283 and 161, 7133 of 147 205 and 163; 64
+    // rows of 27 22.8 us and 18.7, of 64 22.7 and 18.7, of 100 22.7 and 23.)
+    const bool many = a.n_units >= 8ll * ctx->n_sm;
+    if (max_k <= (many ? 160 : 64)) {
+        ext = true;
+        a.direct = k4 >= 32 ? 2 : k4 >= 16 ? 1 : 0;
+        smem = fixed + (size_t)((a.n_cand + 3) & ~3) * 4;
+        threads = many ? 32 : max_k <= 36 ? 64 : 128;
+    } else if (bins > 0 && (double)bins * (double)max_k < 2147483648.0) {
         // blocks of this launch that an SM holds, by shared memory and by the rows there are
         const long long per_sm = std::max(1ll, (a.n_units + ctx->n_sm - 1) / ctx->n_sm);
         auto fits = [&](bool packed) {
@@ -196,25 +208,39 @@ int launch_rows(omse_ctx* ctx, omse::RowArgs& a, long long max_k, int path) {
         a.packed_counts = !ext && fits(false) == 1 && fits(true) > 1;
         threads = block_threads((int)fits(a.packed_counts), max_k);
         a.n_bins = bins;
-        a.window = 0;
         a.smem_bins = omse::lattice_padded(bins, threads);
         a.smem_bins2 = coarse_words(a, bins);
         smem = fixed + lattice_bytes(a, threads, bins, a.packed_counts);
     }
     if (smem == 0 || smem > (size_t)kMaxSmem) {
-        // the bins do not fit at once: windows, up to the last threshold that any candidate has
-        int top = 1;
-        for (int j = 0; j < a.n_tensors; ++j) top = std::max(top, std::max(a.hi[j], -a.lo[j]));
-        a.n_bins = (int)std::min(2.0 * (double)a.n_cand / (double)a.hi_frac * (1.0 + 1e-6), (double)(2 * top - 1) * (double)a.n_cand);
-        if (a.n_bins < 1) a.n_bins = 1;
-        a.smem_bins2 = 0;
-        for (a.window = 16384; ; a.window >>= 1) {
-            if (a.window < 512) return OMSE_EINVAL;
+        // The bins do not fit at once: windows of them, up to the last threshold that any candidate has, where the row leaves room
+        // for one block in any case and the windows are few; evaluations otherwise.  A window costs about what five evaluations do at
+        // 25,088 values, of which a search takes 45 (4 bits) to 110 (8 bits).  4096 candidates, 4 and 8 bits, windows and
+        // evaluations: 80 rows of 25,088, grid to a quarter of max|x| 165 us and 172, 178 and 296, to a tenth 297 and 192, 361 and 396,
+        // to a hundredth 189 and 64, 3546 and 472; 434 rows of 4608 values 220 and 137, 264 and 231; 366 and 160, 488 and 327; 545
+        // and 49, 7568 and 255.
+        ext = true;
+        a.packed_counts = 0;
+        a.smem_bins = a.smem_bins2 = 0;
+        int top = 1, sides = 1;
+        for (int j = 0; j < a.n_tensors; ++j) {
+            top = std::max(top, std::max(a.hi[j], -a.lo[j]));
+            if (a.lo[j] < 0) sides = 2;
+        }
+        a.n_bins = std::max(1, (int)std::min(2.0 * (double)a.n_cand / (double)a.hi_frac * (1.0 + 1e-6), (double)(2 * top - 1) * (double)a.n_cand));
+        threads = block_threads((int)std::max(1ll, (long long)(kSmSmem / (fixed + (size_t)a.n_cand * 4 + kBlockSmem))), max_k);
+        const size_t curve = (size_t)((a.n_cand + 3) & ~3) * 4;
+        for (a.window = 16384; a.window >= 4096; a.window >>= 1) {
             a.smem_bins = omse::lattice_padded(a.window, threads);
-            smem = fixed + (2 * (size_t)a.smem_bins + (size_t)((a.n_cand + 3) & ~3)) * 4;
+            smem = fixed + 2 * (size_t)a.smem_bins * 4 + curve;
             if (smem <= (size_t)kMaxSmem) break;
         }
-        ext = true;
+        const int n_win = (a.n_bins + a.window - 1) / a.window;
+        if (max_k < 12288 || a.window < 4096 || n_win * sides > (top < 64 ? 8 : 20)) {
+            a.direct = omse::kSplitRows;
+            a.window = a.smem_bins = 0;
+            smem = fixed + curve + omse::kSplitSlots * sizeof(omse::SplitPoint);
+        }
     }
     return launch_rows_kernel(ctx, a, path, ext, threads, smem);
 }

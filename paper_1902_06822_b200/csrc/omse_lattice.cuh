@@ -42,7 +42,10 @@ constexpr int kTeamWarps = 24;
 struct TeamScratch {
     unsigned int amax[kTeamWarps];
     float esum[kTeamWarps];
-    unsigned int scan_n[kTeamWarps], scan_s[kTeamWarps], scan_f[kTeamWarps];
+    union {
+        struct { unsigned int scan_n[kTeamWarps], scan_s[kTeamWarps], scan_f[kTeamWarps]; };
+        double energy[kTeamWarps];          // direct_begin
+    };
     union {
         struct {
             float dmin[2][kTeamWarps];
@@ -141,7 +144,8 @@ struct LatticeShape {
     int n_bins;           // bins m = 1 .. n_bins hold every |x|/h of a row; bin m is word m-1
     float hi_frac;
     int flo, fhi;         // range of the codes
-    int window;           // 0: all bins at once; > 0: bins per window of lattice_search_wide
+    int window;           // lattice_search_wide: bins per window
+    int direct;           // lattice_coarse: lanes per candidate (log2)
 };
 
 // Shared memory of the search of one row.
@@ -191,6 +195,7 @@ struct LatticeResult {
     int best;             // candidate with the smallest value on the curve (lowest index)
     float dmin, band;     // that value; candidates with curve[c] <= band may be the exact minimum
     int lo, hi;           // curve[] holds the coarse candidates (lattice_coarse) and all of [lo, hi]
+    int evaluated;        // looks at the row
 };
 
 // The candidates that are looked at first: c + 1 = 1 .. 16, then eight per octave, and the last one.
@@ -436,6 +441,7 @@ __device__ __forceinline__ LatticeResult lattice_search(const BlockTeam& tm, con
     res.dmin = res.band = 0.f;
     res.lo = 0;
     res.hi = -1;
+    res.evaluated = 1;
     const bool sgn = g.flo < 0;
     const int levels = g.fhi, d = sgn ? 2 * (-g.flo) - 1 : 0;       // common levels, spacing of the extra negative level
     const int n_bins = g.n_bins, lb = lattice_log_run(n_bins, tm.size()), padded = lattice_padded(n_bins, tm.size());
@@ -550,7 +556,7 @@ __device__ __forceinline__ LatticeResult lattice_search(const BlockTeam& tm, con
 // The same for grids whose bins do not fit in shared memory at once (many candidates with a grid that ends far below
 // max|x|): the bins are taken in windows from the top down, positive and negative values in turn, each window with an
 // insertion pass of its own; values above the last threshold are summed in registers.  P is kept in binary32 and the
-// curve is added up in binary32, so the band is wider than above.
+// curve is added up in binary32, so the band is wider than above.  For long rows and a few windows (see launch_rows).
 __device__ __forceinline__ LatticeResult lattice_search_wide(const BlockTeam& tm, const LatticeShape& g, const LatticeSmem& sm,
                                                              const float4* xs4, int k, int k4, unsigned int amax_bits, TeamScratch* ts) {
     LatticeResult res;
@@ -561,6 +567,7 @@ __device__ __forceinline__ LatticeResult lattice_search_wide(const BlockTeam& tm
     res.dmin = res.band = 0.f;
     res.lo = 0;
     res.hi = -1;
+    res.evaluated = 1;
     const int lane = tm.t & 31, warp = tm.t >> 5, nwarp = tm.n >> 5;
     const unsigned int mb = team_umax(tm, amax_bits, ts);
     const float m_abs = __uint_as_float(mb);
@@ -593,11 +600,14 @@ __device__ __forceinline__ LatticeResult lattice_search_wide(const BlockTeam& tm
                 const float a = x[j] * sg;
                 const double t = (double)a * inv_d;                // (may leave binary32: the grid can end anywhere below max|x|)
                 e = fma(t, t, e);
-                int m = 0;
-                if (a * inv_up < far) lattice_bin(a, h, inv_up, m);
-                if (m > n_bins || !(a * inv_up < far)) {
-                    over_n += 1.0;
-                    over_s += t - (double)(n_bins + 1);
+                const float td = a * inv_up;                       // not below |x|/h, and above it by less than a bin
+                if (td >= (float)(n_bins + 1)) {
+                    int m = n_bins + 1;
+                    if (td < far) lattice_bin(a, h, inv_up, m);
+                    if (m > n_bins) {
+                        over_n += 1.0;
+                        over_s += t - (double)(n_bins + 1);
+                    }
                 }
             }
         }
@@ -631,8 +641,8 @@ __device__ __forceinline__ LatticeResult lattice_search_wide(const BlockTeam& tm
                 const float x[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const float a = x[j] * sg;
-                    if (!(a >= h) || !(a * inv_up < far)) continue;
+                    const float a = x[j] * sg, td = a * inv_up;
+                    if (!(td >= (float)(base + 1) && td < (float)(base + win + 2) && td < far)) continue;
                     int m;
                     const float r = lattice_bin(a, h, inv_up, m);
                     if (m > base && m <= base + win && m <= n_bins) {
@@ -711,6 +721,233 @@ __device__ __forceinline__ LatticeResult lattice_search_wide(const BlockTeam& tm
     res.hi = g.n_cand - 1;
     res.band = lattice_band(bv, 1.0f, (float)sqrt((double)k * e_inv), __int_as_float((127 - fbits) << 23), 0.f, 0.f) +
                1.2e-7f * (float)(windows + 4);
+    return res;
+}
+
+// -------------------------------------------------------------------------------------------------
+// The same without a histogram, by evaluating candidates: for rows of so few values that clearing and scanning 2C bins costs more
+// (lattice_coarse), and for grids that end so far below max|x| that their bins would take many windows (lattice_split).
+// -------------------------------------------------------------------------------------------------
+// team_argmin for values that are not negative (nor NaN): they order like their bit patterns
+__device__ __forceinline__ void team_argmin_error(const BlockTeam& tm, float& v, int& idx, TeamScratch* ts, int slot) {
+    const unsigned int least = __reduce_min_sync(0xffffffffu, __float_as_uint(v));
+    idx = __reduce_min_sync(0xffffffffu, __float_as_uint(v) == least ? idx : 0x7fffffff);
+    v = __uint_as_float(least);
+    if ((tm.t & 31) == 0) {
+        ts->dmin[slot][tm.t >> 5] = v;
+        ts->didx[slot][tm.t >> 5] = idx;
+    }
+    __syncthreads();
+    for (int w = 0; w < (tm.n >> 5); ++w) {
+        const float ov = ts->dmin[slot][w];
+        const int oi = ts->didx[slot][w];
+        if (ov < v || (ov == v && oi < idx)) {
+            v = ov;
+            idx = oi;
+        }
+    }
+}
+template <bool SCALED>
+__device__ __forceinline__ float direct_part(const float4* xs4, int k4, int first, int stride, float al, float sc, float flo, float fhi) {
+    const float inv = __fdiv_rn(1.0f, al), clo = kMagic + flo, chi = kMagic + fhi;
+    const u64 M2 = pack2(kMagic, kMagic), NM2 = pack2(-kMagic, -kMagic), inv2 = pack2(inv, inv), na2 = pack2(-al, -al), sc2 = pack2(sc, sc),
+              z2 = pack2(-0.f, -0.f);
+    auto pair = [&](u64 x, u64 acc) {
+        if (SCALED) x = fma2(x, sc2, z2);
+        float a, b;
+        unpack2(fma2(x, inv2, M2), a, b);
+        const u64 d = fma2(na2, add2(pack2(fminf(fmaxf(a, clo), chi), fminf(fmaxf(b, clo), chi)), NM2), x);
+        return fma2(d, d, acc);
+    };
+    u64 total = 0ull;
+    for (int i = first; i < k4;) {                          // folds of 128 values: rounding noise near 1e-7
+        const int stop = min(k4, i + kFlushEvery4 * stride);
+        u64 acc_a = 0ull, acc_b = 0ull;
+#pragma unroll 4
+        for (; i < stop; i += stride) {
+            const float4 v = xs4[i];
+            acc_a = pair(pack2(v.x, v.y), acc_a);
+            acc_b = pair(pack2(v.z, v.w), acc_b);
+        }
+        total = add2(total, add2(acc_a, acc_b));
+    }
+    float a, b;
+    unpack2(total, a, b);
+    return a + b;
+}
+
+// Grid, scaling and energy of a row; false where there is nothing to search.
+struct DirectRow {
+    float step, sc;       // sc: a power of two that keeps squares in binary32
+    __device__ __forceinline__ float scale(int c) const { return fmaxf(__fmul_rn((float)(c + 1), step) * sc, FLT_MIN); }
+    __device__ __forceinline__ bool usable(int c) const { return usable_scale(__fmul_rn((float)(c + 1), step)); }
+};
+__device__ __forceinline__ bool direct_begin(const BlockTeam& tm, const LatticeShape& g, const float4* xs4, int k4, unsigned int amax_bits,
+                                             TeamScratch* ts, LatticeResult& res, DirectRow& row) {
+    res.degenerate = true;
+    res.best = -1;
+    res.step = 0.f;
+    res.dmin = res.band = 0.f;
+    res.lo = 0;
+    res.hi = -1;
+    res.evaluated = 0;
+    const unsigned int mb = team_umax(tm, amax_bits, ts);
+    const Grid gr = grid_of(__uint_as_float(mb), g.hi_frac, g.n_cand);
+    res.bad = mb >= 0x7f800000u;
+    if (res.bad || !gr.usable) return false;
+    res.step = row.step = gr.step;
+    const int ex = (int)(mb >> 23) - 127;
+    row.sc = ex < -40 || ex > 40 ? __int_as_float((127 - max(min(ex, 126), -126)) << 23) : 1.0f;
+    double e = 0.0;                                         // the warps' sums now, the row's after the next barrier
+    for (int i = tm.t; i < k4; i += tm.n) {
+        const float4 v = xs4[i];
+        const float y[4] = {v.x * row.sc, v.y * row.sc, v.z * row.sc, v.w * row.sc};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) e = fma((double)y[u], (double)y[u], e);
+    }
+    e = warp_sum(e);
+    if ((tm.t & 31) == 0) ts->energy[tm.t >> 5] = e;
+    return true;
+}
+__device__ __forceinline__ double direct_energy(const BlockTeam& tm, const TeamScratch* ts) {
+    double e = 0.0;
+    for (int w = 0; w < (tm.n >> 5); ++w) e += ts->energy[w];
+    return e;
+}
+__device__ __forceinline__ float direct_error(const float4* xs4, int k4, int first, int stride, const DirectRow& r, int c, int flo, int fhi) {
+    return r.sc != 1.0f ? direct_part<true>(xs4, k4, first, stride, r.scale(c), r.sc, (float)flo, (float)fhi)
+                        : direct_part<false>(xs4, k4, first, stride, r.scale(c), r.sc, (float)flo, (float)fhi);
+}
+
+// The coarse candidates, then all of the stretch of the grid that the chords between them leave open.  2^lanes neighbouring lanes
+// share a candidate: with fewer lanes there are more candidates under way than are wanted, with more the short rows leave lanes
+// without values.
+__device__ __forceinline__ LatticeResult lattice_coarse(const BlockTeam& tm, const LatticeShape& g, float* curve, const float4* xs4, int k4,
+                                                        unsigned int amax_bits, TeamScratch* ts) {
+    LatticeResult res;
+    DirectRow row;
+    if (!direct_begin(tm, g, xs4, k4, amax_bits, ts, res, row)) return res;
+    const int lanes = g.direct, groups = tm.n >> lanes, group = tm.t >> lanes, j = tm.t & ((1 << lanes) - 1);
+    float bv = INFINITY;
+    int bi = 0x7fffffff;
+    auto evaluate = [&](int c, bool wanted) {               // every lane of the warp takes part
+        float v = direct_error(xs4, wanted ? k4 : 0, j, 1 << lanes, row, c, g.flo, g.fhi);
+        for (int o = 1; o < 1 << lanes; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (!row.usable(c)) v = INFINITY;
+        if (!wanted || j != 0) return;
+        curve[c] = v;
+        if (v < bv || (v == bv && c < bi)) {
+            bv = v;
+            bi = c;
+        }
+    };
+    const int n_coarse = coarse_count(g.n_cand);
+    for (int i0 = 0; i0 < n_coarse; i0 += groups)
+        evaluate(coarse_a1(min(i0 + group, n_coarse - 1), g.n_cand) - 1, i0 + group < n_coarse);
+    float cv = bv;
+    int ci = bi;
+    team_argmin_error(tm, cv, ci, ts, 0);
+    if (ci == 0x7fffffff) return res;                       // every error is Inf
+    const float e = (float)direct_energy(tm, ts), keep = cv * 1.00001f + 2e-6f * e;    // binary32 in the sums and in the bound
+    int lo = g.n_cand, hi = -1;
+    for (int i = tm.t; i + 1 < n_coarse; i += tm.n) {
+        const int a0 = coarse_a1(i, g.n_cand), a1 = coarse_a1(i + 1, g.n_cand);
+        if (a1 - a0 >= 2 && !(chord_bound(e, a0, curve[a0 - 1], a1, curve[a1 - 1]) > keep)) {      // (an unusable end keeps the interval)
+            lo = min(lo, a0);
+            hi = max(hi, a1 - 2);
+        }
+    }
+    team_range(tm, lo, hi, ts);
+    for (int c0 = lo; c0 <= hi; c0 += groups) evaluate(min(c0 + group, hi), c0 + group <= hi);
+    team_argmin_error(tm, bv, bi, ts, 1);
+    res.degenerate = false;
+    res.best = bi;
+    res.dmin = bv;
+    res.lo = lo;
+    res.hi = hi;
+    res.evaluated = n_coarse + max(0, hi - lo + 1);
+    res.band = bv * (1.0f + (float)kRescoreBand);
+    return res;
+}
+
+// The powers of two of the grid, then splits of the intervals that their chord leaves open, near the minimum of its bound, depth
+// first (as in omse_rows_short.cuh): 30 to 60 evaluations by the whole block, one after the other, whatever C is.  The chords are
+// drawn in binary64 at the binary32 scales themselves, since the errors of fine grids are a millionth of E.
+// stack: kSplitSlots entries; a split leaves at most three quarters of an interval, below the fifth half.
+struct __align__(16) SplitPoint {
+    double w;             // (E - error)/scale
+    int c;
+    float v;
+};
+constexpr int kSplitSlots = 48, kSplitFree = 5;
+__device__ __forceinline__ LatticeResult lattice_split(const BlockTeam& tm, const LatticeShape& g, float* curve, SplitPoint* stack, const float4* xs4,
+                                                       int k4, unsigned int amax_bits, TeamScratch* ts) {
+    LatticeResult res;
+    DirectRow row;
+    if (!direct_begin(tm, g, xs4, k4, amax_bits, ts, res, row)) return res;
+    for (int c = tm.t; c < g.n_cand; c += tm.n) curve[c] = INFINITY;
+    __syncthreads();
+    const double e = direct_energy(tm, ts);
+    const int nwarp = tm.n >> 5;
+    float cv = INFINITY;
+    int ci = 0x7fffffff, slot = 0;
+    auto evaluate = [&](int c) -> SplitPoint {              // the same in all threads
+        const float part = warp_allsum(direct_error(xs4, k4, tm.t, tm.n, row, c, g.flo, g.fhi));
+        if ((tm.t & 31) == 0) ts->dmin[slot][tm.t >> 5] = part;
+        __syncthreads();
+        float v = 0.f;
+        for (int w = 0; w < nwarp; ++w) v += ts->dmin[slot][w];
+        slot ^= 1;
+        if (!row.usable(c)) v = INFINITY;
+        if (tm.t == 0) curve[c] = v;
+        if (v < cv || (v == cv && c < ci)) {
+            cv = v;
+            ci = c;
+        }
+        ++res.evaluated;
+        return SplitPoint{(e - (double)v) / (double)row.scale(c), c, v};
+    };
+    const int n_first = 33 - __clz(g.n_cand - 1);           // 2^i below n_cand, and n_cand
+    for (int i = 0; i < n_first; ++i) {
+        const SplitPoint p = evaluate(min(1 << i, g.n_cand) - 1);
+        if (tm.t == 0) stack[i] = p;
+    }
+    __syncthreads();
+    SplitPoint top = stack[n_first - 1];
+    int sp = n_first - 2;
+    while (sp >= 0) {
+        const SplitPoint low = stack[sp];
+        const int width = top.c - low.c;
+        bool open = width >= 2;
+        double at = 0.0;
+        if (open) {
+            const double a0 = (double)row.scale(low.c), a1 = (double)row.scale(top.c), slope = (low.w - top.w) / (a1 - a0);
+            at = slope > 0.0 ? fmin(fmax(0.5 * (low.w / slope + a0), a0), a1) : a1;
+            const double bound = e - at * (low.w - slope * (at - a0)), most = (double)fmaxf(low.v, top.v);
+            // what the chord has to be above: the best value so far, the noise of the sums, and values on the other side of a
+            // threshold (lattice_band); an unusable end keeps the interval
+            open = !(bound > (double)cv * 1.00001 + 4e-6 * most + 2.5e-7 * sqrt(e * most) + 1e-12 * e);
+            at = (at - a0) / (a1 - a0) * (double)width;
+        }
+        if (open) {
+            const int q = max(1, sp < n_first - 2 + kSplitFree ? width >> 2 : width >> 1);
+            const int c = low.c + min(max(__double2int_rn(at), q), width - q);
+            const SplitPoint p = evaluate(c);               // (its barrier lies between the reads of the stack above and the write)
+            ++sp;
+            if (tm.t == 0) stack[sp] = p;
+            __syncthreads();
+        } else {
+            top = low;
+            --sp;
+        }
+    }
+    if (ci == 0x7fffffff) return res;                       // every error is Inf
+    res.degenerate = false;
+    res.best = ci;
+    res.dmin = cv;
+    res.lo = 0;                                             // the candidates that were not evaluated read as Inf
+    res.hi = g.n_cand - 1;
+    res.band = cv * (1.0f + (float)kRescoreBand);
     return res;
 }
 

@@ -43,6 +43,7 @@ struct RowArgs {
     int max_k4;                 // float4s of the longest row in the launch (shared-memory carve-up)
     int n_bins;                 // bins of |x|/h (see LatticeShape)
     int window;                 // > 0: the bins are taken in windows of this many
+    int direct;                 // >= 0: no histogram; lanes per candidate (log2) of lattice_coarse, or kSplitRows for lattice_split
     int packed_counts;          // 16 bits per count (see Counts)
     int smem_bins, smem_bins2;  // words of the bin arrays in shared memory (fine, coarse)
     int solver;                 // 0: grid line search (Section 3.4); 1: uniform scale max|x|/L; 2: alternating from the
@@ -92,6 +93,7 @@ __device__ __forceinline__ void rows_done(const RowArgs& a, unsigned int st, uns
 namespace omse {
 
 constexpr int kScratchDoubles = 64;
+constexpr int kSplitRows = 31;                   // RowArgs::direct
 constexpr int kRowsThreads = 32 * kTeamWarps;    // sets the register budget; blocks have up to 512 threads
 
 struct PhiOut {
@@ -185,6 +187,7 @@ struct RowSmem {
     LatticeSmem lat;  // histograms and error curve
     double* scratch;  // [kScratchDoubles] reductions
     TeamScratch* ts;
+    SplitPoint* stack; // [kSplitSlots] lattice_split
     int* misc;        // [8]: 1..4 nibble carried to the next row, per tensor
 };
 
@@ -281,13 +284,15 @@ __device__ PhiOut phi_block(const RowArgs& a, const RowSmem& s, int k, int k4, i
     }
 
     // ---- the error curve; every candidate within its noise band of the minimum is re-scored in fp64 with exact codes
-    const LatticeShape shape = {a.n_cand, a.n_bins, a.hi_frac, lo, hi, a.window};
-    const LatticeResult r = EXT && a.window > 0 ? lattice_search_wide(team, shape, s.lat, xs4, k, k4, amax, s.ts)
-                                         : lattice_search<PACKED>(team, shape, s.lat, xs4, k, k4, amax, s.ts);
+    const LatticeShape shape = {a.n_cand, a.n_bins, a.hi_frac, lo, hi, a.window, a.direct};
+    const LatticeResult r = EXT && a.direct == kSplitRows ? lattice_split(team, shape, s.lat.curve, s.stack, xs4, k4, amax, s.ts)
+                            : EXT && a.direct >= 0        ? lattice_coarse(team, shape, s.lat.curve, xs4, k4, amax, s.ts)
+                            : EXT && a.window > 0         ? lattice_search_wide(team, shape, s.lat, xs4, k, k4, amax, s.ts)
+                                                          : lattice_search<PACKED>(team, shape, s.lat, xs4, k, k4, amax, s.ts);
     out.bad = r.bad;
     if (r.degenerate) return out;
     out.degenerate = false;
-    if (tid == 0) ev += (unsigned long long)k;
+    if (tid == 0) ev += (unsigned long long)k * (unsigned long long)r.evaluated;
     int best = r.best;
     double best_sse = INFINITY;
     bool other = false;                                     // a candidate beside the minimum lies in the band
@@ -411,8 +416,8 @@ __device__ double emit_block(const RowSmem& s, int k, float alpha, float flo, fl
 
 // EXT = false: the grid search with polish (and Algorithm 1 with a fixed number of sweeps) and nothing else, so that
 // the common launches keep their register allocation and code size; EXT = true adds the comparison solvers, the offset
-// search, Algorithm 1's loop condition, gated layers, rows that start from an earlier tensor's residual and grids whose
-// bins are taken in windows.  PACKED: counts of 16 bits (see Counts).
+// search, Algorithm 1's loop condition, gated layers, rows that start from an earlier tensor's residual the search without a
+// histogram and the one by windows.  PACKED: counts of 16 bits (see Counts).
 // 80 registers per thread: 24 warps per SM, in as many blocks as the rows leave shared memory for; the phases of a row are
 // separated by barriers, and the blocks of an SM fill each other's gaps.  Against 128 registers (16 warps): 29,127 rows of
 // 2304 values 811 -> 697 us, 14,563 of 4608 565 -> 488, 5592 of 12,000 700 -> 434, 2674 of 25,088 539 -> 443.
@@ -436,6 +441,7 @@ __global__ void __launch_bounds__(kRowsThreads) rows_kernel(const RowArgs a) {
     s.scratch = reinterpret_cast<double*>(windows ? s.lat.f2 + ((a.n_cand + 3) & ~3) : s.lat.n2 + a.smem_bins2);
     s.misc = reinterpret_cast<int*>(s.scratch + kScratchDoubles);
     s.ts = &s_team;
+    s.stack = reinterpret_cast<SplitPoint*>(s.misc + 8);
     unsigned int st = 0;
     unsigned long long ev = 0ull;      // evaluations this thread executed
 

@@ -172,3 +172,34 @@ def test_dual_search_by_bounds(s, k, bits1, bits2, signed, c1, c2, hf1, hf2, sca
     if pk is not None:
         for j in range(2):
             assert np.array_equal(pk[j], orc.pack_int4(ref.codes[j].reshape(-1)))
+
+
+@pytest.mark.parametrize("s,k,bits,n_cand,hi_frac,scale", [
+    (1300, 1, 4, 1024, 1.0, 1.0),                   # candidates evaluated, a warp per row: one value, one lane per candidate ...
+    (1300, 27, 4, 1024, 1.0, 1.0), (1201, 63, 8, 200, 1.0, 1.0),
+    (1201, 64, 3, 300, 1.0, 1.0), (1201, 65, 4, 1024, 1.0, 1.0),    # ... two lanes
+    (1201, 127, 4, 1, 1.0, 1.0), (1201, 128, 4, 2, 1.0, 1.0),       # ... four; one and two candidates
+    (1201, 160, 4, 4096, 1.0, 1.0), (1201, 161, 4, 4096, 1.0, 1.0), # one value more: by histogram
+    (9, 27, 8, 1024, 1.0, 1.0), (9, 36, 4, 17, 0.3, 1.0), (9, 64, 4, 1024, 1.0, 1.0),     # small launches: 64 and 128 threads
+    (1201, 31, 4, 300, 1.0, 2.0 ** -112), (9, 40, 2, 300, 0.5, 2.0 ** 59),                # squares outside binary32
+    (40, 700, 4, 4096, 0.1, 1.0), (40, 700, 8, 4096, 0.01, 2.0 ** -100),                  # by splits: bins do not fit
+    (3, 12_287, 4, 4096, 0.1, 1.0), (3, 12_289, 4, 4096, 0.25, 1.0),                      # the last row by splits, windows
+    (2, 25_600, 8, 4096, 0.05, 1.0), (2, 25_088, 4, 4096, 0.02, 1.0), (5, 5000, 4, 3, 1e-6, 1.0),
+])
+def test_residual_rows_by_every_search(s, k, bits, n_cand, hi_frac, scale):
+    """Two quantized tensors, which rows of any length take through a block per row."""
+    import gpu_util
+    from oracle import omse_oracle as orc
+    w = synth.student_t3(s * k, seed=101, tensor_id=k).reshape(s, k) * np.float32(scale)
+    alpha, sse, q, pk = gpu_util.residual_quantize(w, (bits, bits), True, n_cand, hi_frac, 3, 1, True, bits <= 4)
+    rows = np.unique(np.concatenate([np.arange(0, s, max(1, s // 40)), [s - 1]]))
+    ref = orc.residual_rows(np.ascontiguousarray(w[rows]), (bits, bits), True, n_cand, hi_frac, 3, 1)
+    # the two tensors of a row whose first scale differs by a rounding differ altogether: at most one row in fifty
+    same = (alpha[0][rows] == ref.alpha[0]) & (alpha[1][rows] == ref.alpha[1])
+    assert same.mean() >= 0.95 or (~same).sum() <= 1, same.mean()
+    assert np.array_equal(q.reshape(2, s, k)[:, rows][:, same], ref.codes[:, same])
+    np.testing.assert_allclose(sse[:, rows][:, same], ref.sse[:, same], rtol=1e-5, atol=1e-37)
+    np.testing.assert_allclose(alpha[:, rows], ref.alpha, rtol=2e-2)
+    if pk is not None:
+        for j in range(2):
+            assert np.array_equal(pk[j], orc.pack_int4(q[j]))
