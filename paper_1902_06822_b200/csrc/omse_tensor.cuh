@@ -39,9 +39,12 @@ struct TensorState {          // lives in the context workspace
     float delta;                         // offset subtracted from every element (0 without offset)
     double sum_sq;                       // sum x^2
     double near;                         // sum of floor(|x|/h) over the values next to an edge of a bin (see tensor_noise)
-    // state of the scan at the first bin of the window processed last (bins are taken in windows from the top down)
-    double scan_n, scan_s, scan_f;
-    long long scan_pos;
+    // state N, S, F of the scan at the bin `pos`, below which the next window lies (bins are taken in windows from the top down);
+    // windows read one of the two and write the other
+    struct Scan {
+        double n, s, f;
+        long long pos;
+    } scan[2];
 };
 
 struct TensorArgs {
@@ -53,11 +56,14 @@ struct TensorArgs {
     int n_bins, n_bins2;    // bins of the fine histogram and of the extra negative level's
     int clipped;            // values above the last bin exist (the grid ends below max|x|)
     int win, win_base;      // this launch's bins: m = win_base+1 .. win_base+win
+    int shared_win;         // so many of them, from the first on, are kept in shared memory; the others in the global histogram
     int first_window;       // 1: topmost window (sum x^2, values above the bins and the coarse histogram are taken with it)
-    int last_window;
+    int which;              // parity of the window: the scan state it reads
     TensorState* st;
     unsigned long long* hist;   // [2][win] counts and fractional sums, then [2][n_bins2]
-    double* above;          // [2][win] N and P of the window, then [2][n_bins2]
+    double* above;          // [2][win] N and P of the window, then [2][n_bins2] (may alias hist)
+    double* chunks;         // [n_chunks][3] sums of the chunks of a window
+    int n_chunks;
     double* block_sums;     // [grid][kBlockSums]: sum x^2, number and excess of the values above the bins, the same for the coarse
                             // ones, sum of the bins of the values next to an edge
     int n_blocks;           // blocks of the histogram launch
@@ -203,7 +209,8 @@ __device__ __forceinline__ void hist_put3(unsigned int* c, unsigned int* lo, uns
 struct HistGeometry {
     float pre, scale, h, inv_up;  // a = |x*pre*scale|, h = H; bin floor(a*inv_up)
     float far;                    // bins from here on are above all histograms
-    int sgn, d, d_from, n_bins, n_bins2, base, top;
+    int sgn, d, d_from, n_bins, n_bins2, base, top, shared_win;
+    unsigned long long *far_n, *far_f;   // the window's bins in global memory
     unsigned int rd, hk;          // 2^32/D; H
 };
 __device__ __forceinline__ HistGeometry hist_geometry(float step, const TensorArgs& a) {
@@ -222,6 +229,9 @@ __device__ __forceinline__ HistGeometry hist_geometry(float step, const TensorAr
     g.n_bins2 = a.n_bins2;
     g.base = a.win_base;
     g.top = a.win_base + a.win;
+    g.shared_win = a.shared_win;
+    g.far_n = a.hist;
+    g.far_f = a.hist + a.win;
     g.far = (float)(max(a.n_bins, g.d * (a.n_bins2 + 1)) + 2);    // (2,084,866 at most: 4.8e-7 of it is less than a bin)
     return g;
 }
@@ -250,32 +260,50 @@ __device__ __forceinline__ void hist_put_coarse(const HistGeometry& g, const His
     hist_put3(w.c2, w.lo2, w.hi2, min((int)m2, g.n_bins2) - 1, rem * g.hk + (unsigned)k);
 }
 
+// The same into the global histogram: the lanes that meet in a bin add once.  Values that repeat would queue for one address (51M
+// values, a twelfth of them equal: 3.2 ms, 1.5 so); uniform ones pay for it (0.8 ms, 1.45 so), heavy-tailed ones have few there.
+__device__ __forceinline__ void hist_put_far(const HistGeometry& g, int i, int k) {
+    const unsigned int peers = __match_any_sync(__activemask(), i);
+    const unsigned int sum = __reduce_add_sync(peers, (unsigned)k);            // at most 32*2^24
+    if ((int)(threadIdx.x & 31) == __ffs(peers) - 1) {
+        atomicAdd(g.far_n + i, (unsigned long long)__popc(peers));
+        atomicAdd(g.far_f + i, (unsigned long long)sum);
+    }
+}
+
 // Four values x*pre where the window holds all bins and no value lies above them (the common case).  One branch for the rare
 // values next to an edge, instead of four.  SIGNED: the range has negative codes; an unsigned one codes negative values as 0.
 template <bool SIGNED>
 __device__ __forceinline__ void hist_insert4(const float (&x)[4], const HistGeometry& g, const HistWords& w, HistSums& s) {
-    int m[4], k[4], least = 0;
+    float u[4], r[4], least = 0.f;                        // M + bin, remainder (an integer)
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        const float y = x[j] * g.scale, a = SIGNED ? fabsf(y) : y, u = __fmaf_rd(a, g.inv_up, kMagic);
+        const float y = x[j] * g.scale, a = SIGNED ? fabsf(y) : y;
         s.sq = fma((double)x[j], (double)x[j], s.sq);
-        m[j] = magic_int(u);
-        k[j] = __float2int_rz(fmaf(-(u - kMagic), g.h, a));
-        least = min(least, k[j] - 3 * m[j]);
+        u[j] = __fmaf_rd(a, g.inv_up, kMagic);
+        const float mf = u[j] - kMagic;
+        r[j] = fmaf(-mf, g.h, a);
+        least = fminf(least, fmaf(-3.0f, mf, r[j]));      // (not negative for a bin below the first)
     }
-    if (least < 0) {
+    if (least < 0.f) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (m[j] >= 1 && hist_near(k[j], m[j])) {
-                s.near += m[j];
-                hist_correct(k[j], m[j], g.hk);
+        for (int j = 0; j < 4; ++j) {
+            int m = magic_int(u[j]), k = (int)r[j];
+            if (m >= 1 && hist_near(k, m)) {
+                s.near += m;
+                hist_correct(k, m, g.hk);
+                u[j] = kMagic + (float)m;
+                r[j] = (float)k;
             }
+        }
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        if (m[j] < 1) continue;
-        hist_put_fine(g, w, min(m[j], g.n_bins) - 1, k[j]);
-        if (SIGNED && x[j] < 0.f && m[j] >= g.d_from) hist_put_coarse(g, w, m[j], k[j]);
+        const int m = magic_int(u[j]);
+        if (m < 1) continue;
+        const int k = __float2int_rz(r[j]);
+        hist_put_fine(g, w, min(m, g.n_bins) - 1, k);
+        if (SIGNED && x[j] < 0.f && m >= g.d_from) hist_put_coarse(g, w, m, k);
     }
 }
 // One value x*pre where values may lie above the last bin or outside the window.
@@ -301,7 +329,9 @@ __device__ __forceinline__ void hist_insert(float x, const HistGeometry& g, cons
             s.over_s += (double)a / (double)g.h - (double)(g.n_bins + 1);
         }
     } else if (m > g.base && m <= g.top) {
-        hist_put_fine(g, w, m - 1 - g.base, k);
+        const int i = m - 1 - g.base;
+        if (i < g.shared_win) hist_put_fine(g, w, i, k);
+        else hist_put_far(g, i, k);
     }
     if (SIGNED && first && x < 0.f && g.d > 0 && m >= g.d) {
         if (m >= g.d * (g.n_bins2 + 1)) {
@@ -321,10 +351,10 @@ __global__ void __launch_bounds__(kHistThreads, 2) tensor_hist_kernel(const Tens
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double dscratch[64];
     TensorState* st = a.st;
-    const int tid = threadIdx.x, words = kHotWords + a.win;                             // win is a multiple of 4
-    unsigned long long* acc_f = reinterpret_cast<unsigned long long*>(smem_raw);       // [win]
+    const int tid = threadIdx.x, swin = a.shared_win, words = kHotWords + swin;         // swin is a multiple of 4
+    unsigned long long* acc_f = reinterpret_cast<unsigned long long*>(smem_raw);       // [swin]
     HistWords w;
-    w.w1 = reinterpret_cast<unsigned int*>(acc_f + a.win);
+    w.w1 = reinterpret_cast<unsigned int*>(acc_f + swin);
     w.w2 = w.w1 + words;
     w.c2 = w.w2 + words;
     w.lo2 = w.c2 + a.n_bins2;
@@ -338,7 +368,7 @@ __global__ void __launch_bounds__(kHistThreads, 2) tensor_hist_kernel(const Tens
         const float delta = st->delta, off = -delta * g.pre;        // fmaf(x, pre, off) = pre*fl(x - delta): pre is a power of two
         const bool first = a.first_window != 0;
         for (int i = tid; i < 2 * words + 3 * a.n_bins2; i += kHistThreads) w.w1[i] = 0u;      // all words
-        for (int i = tid; i < a.win; i += kHistThreads) {
+        for (int i = tid; i < swin; i += kHistThreads) {
             acc_f[i] = 0ull;
             acc_n[i] = 0u;
         }
@@ -375,7 +405,7 @@ __global__ void __launch_bounds__(kHistThreads, 2) tensor_hist_kernel(const Tens
                 else hist_insert<SIGNED>(x[0], g, w, first, s);
             }
             __syncthreads();
-            if (a.win_base == 0 && tid < kHotBins && tid < a.win) {
+            if (a.win_base == 0 && tid < kHotBins && tid < swin) {
                 unsigned int c = 0u;
                 unsigned long long f = 0ull;
 #pragma unroll
@@ -389,7 +419,7 @@ __global__ void __launch_bounds__(kHistThreads, 2) tensor_hist_kernel(const Tens
                 acc_f[tid] += f;
             }
             const uint4* q1 = reinterpret_cast<const uint4*>(w.w1 + kHotWords);
-            for (int b = tid + (a.win_base == 0 ? kHotBins / 4 : 0); b < (a.win >> 2); b += kHistThreads) {
+            for (int b = tid + (a.win_base == 0 ? kHotBins / 4 : 0); b < (swin >> 2); b += kHistThreads) {
                 const uint4 q = q1[b];
                 if ((q.x | q.y | q.z | q.w) == 0u) continue;        // most bins of a heavy-tailed tensor stay empty
                 const unsigned int p[4] = {q.x, q.y, q.z, q.w};
@@ -414,7 +444,7 @@ __global__ void __launch_bounds__(kHistThreads, 2) tensor_hist_kernel(const Tens
             }
         }
         __syncthreads();
-        for (int b = tid; b < a.win; b += kHistThreads)
+        for (int b = tid; b < swin; b += kHistThreads)
             if (acc_n[b]) {
                 atomicAdd(a.hist + b, (unsigned long long)acc_n[b]);
                 atomicAdd(a.hist + a.win + b, acc_f[b]);
@@ -521,51 +551,98 @@ __device__ __forceinline__ void tensor_scan(const unsigned long long* hn, const 
     }
 }
 
+// What the histogram's blocks left beside the bins, by one block: sum x^2, the sum of the values next to an edge, the state of the
+// scan above the topmost window, N and P of the coarse bins.
+__device__ __forceinline__ void tensor_scan_begin(const TensorArgs& a, double unit, double (*part)[3], double* scratch) {
+    double t[kBlockSums];
+#pragma unroll
+    for (int j = 0; j < kBlockSums; ++j) {                 // the blocks' sums, in a fixed order
+        long long zero = 0;
+        t[j] = 0.0;
+        for (int b = threadIdx.x; b < a.n_blocks; b += kScanThreads) t[j] += __ldcg(a.block_sums + kBlockSums * b + j);
+        if (j == 0 || j == 5 || a.clipped) block_sum2(t[j], zero, scratch);
+    }
+    if (threadIdx.x == 0) {
+        a.st->sum_sq = t[0];
+        a.st->near = t[5];
+        a.st->scan[a.which] = TensorState::Scan{a.clipped ? t[1] : 0.0, a.clipped ? t[2] : 0.0, 0.0, a.n_bins};
+    }
+    if (a.n_bins2 > 0) {
+        const double d = (double)(-2 * a.lo - 1);
+        double dn = a.clipped ? t[3] : 0.0, ds = a.clipped ? t[4] : 0.0, df = 0.0;
+        tensor_scan(a.hist + 2 * a.win, a.hist + 2 * a.win + a.n_bins2, a.n_bins2, unit / d, dn, ds, df, (double)a.n_bins2,
+                    a.above + 2 * a.win, a.above + 2 * a.win + a.n_bins2, part);
+    }
+}
+__device__ __forceinline__ double tensor_unit(const TensorArgs& a) {
+    const float m = fmaxf(__uint_as_float(a.st->mpos_bits), __uint_as_float(a.st->mneg_bits));
+    return hist_unit(grid_of(m, a.hi_frac, a.n_cand).step);
+}
+
+// A window that a block scans by itself.
 __global__ void __launch_bounds__(kScanThreads) tensor_scan_kernel(const TensorArgs a) {
     __shared__ double part[32][3];
     __shared__ double scratch[64];
-    TensorState* st = a.st;
-    const float m = fmaxf(__uint_as_float(st->mpos_bits), __uint_as_float(st->mneg_bits));
-    const double unit = hist_unit(grid_of(m, a.hi_frac, a.n_cand).step);
-    double cn = 0.0, cs = 0.0, cf = 0.0, gap = 0.0;
-    if (a.first_window) {
-        double t[kBlockSums];
-#pragma unroll
-        for (int j = 0; j < kBlockSums; ++j) {             // the blocks' sums, in a fixed order
-            long long zero = 0;
-            t[j] = 0.0;
-            for (int b = threadIdx.x; b < a.n_blocks; b += kScanThreads) t[j] += __ldcg(a.block_sums + kBlockSums * b + j);
-            if (j == 0 || j == 5 || a.clipped) block_sum2(t[j], zero, scratch);
-        }
-        cn = a.clipped ? t[1] : 0.0;
-        cs = a.clipped ? t[2] : 0.0;
-        gap = (double)(a.n_bins - a.win_base);
-        if (threadIdx.x == 0) {
-            st->sum_sq = t[0];
-            st->near = t[5];
-        }
-        if (a.n_bins2 > 0) {
-            const double d = (double)(-2 * a.lo - 1);
-            double dn = a.clipped ? t[3] : 0.0, ds = a.clipped ? t[4] : 0.0, df = 0.0;
-            tensor_scan(a.hist + 2 * a.win, a.hist + 2 * a.win + a.n_bins2, a.n_bins2, unit / d, dn, ds, df, (double)a.n_bins2,
-                        a.above + 2 * a.win, a.above + 2 * a.win + a.n_bins2, part);
-        }
-    } else {
-        cn = st->scan_n;
-        cs = st->scan_s;
-        cf = st->scan_f;
-        gap = (double)(st->scan_pos - a.win_base);
-    }
-    tensor_scan(a.hist, a.hist + a.win, a.win, unit, cn, cs, cf, gap, a.above, a.above + a.win, part);
+    const double unit = tensor_unit(a);
+    if (a.first_window) tensor_scan_begin(a, unit, part, scratch);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        st->scan_n = cn;
-        st->scan_s = cs;
-        st->scan_f = cf;
-        st->scan_pos = a.win_base;
+    const TensorState::Scan above = a.st->scan[a.which];
+    double cn = above.n, cs = above.s, cf = above.f;
+    tensor_scan(a.hist, a.hist + a.win, a.win, unit, cn, cs, cf, (double)(above.pos - a.win_base), a.above, a.above + a.win, part);
+    if (threadIdx.x == 0) a.st->scan[a.which ^ 1] = TensorState::Scan{cn, cs, cf, a.win_base};
+}
+
+// Windows of more bins, in two launches: the sums of chunks of kScanChunk bins, then the scan of every chunk from what lies above it.
+// (One more block of the first launch does what is beside the bins.)
+constexpr int kScanChunk = 4096;
+__global__ void __launch_bounds__(kScanThreads) tensor_chunks_kernel(const TensorArgs a) {
+    __shared__ double part[32][3];
+    __shared__ double scratch[64];
+    if ((int)blockIdx.x == a.n_chunks) {
+        tensor_scan_begin(a, tensor_unit(a), part, scratch);
+        return;
     }
-    if (!a.last_window)                                    // the next window's histogram starts from zero
-        for (int i = threadIdx.x; i < 2 * a.win; i += kScanThreads) a.hist[i] = 0ull;
+    const int first = blockIdx.x * kScanChunk, n = min(kScanChunk, a.win - first);
+    double cn = 0.0, cs = 0.0, cf = 0.0;
+    for (int i = threadIdx.x; i < n; i += kScanThreads) {
+        const double c = (double)__ldcg(a.hist + first + i);
+        cn += c;
+        cs = fma((double)i, c, cs);
+        cf += (double)__ldcg(a.hist + a.win + first + i);
+    }
+    long long zero = 0;
+    block_sum2(cn, zero, scratch);
+    block_sum2(cs, zero, scratch);
+    block_sum2(cf, zero, scratch);
+    if (threadIdx.x == 0) {
+        a.chunks[3 * blockIdx.x] = cn;
+        a.chunks[3 * blockIdx.x + 1] = cs;
+        a.chunks[3 * blockIdx.x + 2] = cf;
+    }
+}
+__global__ void __launch_bounds__(kScanThreads) tensor_chunk_scan_kernel(const TensorArgs a) {
+    __shared__ double part[32][3];
+    __shared__ double scratch[64];
+    const TensorState::Scan above = a.st->scan[a.which];
+    const int first = blockIdx.x * kScanChunk, n = min(kScanChunk, a.win - first);
+    // the state at this chunk's end: sums of T - position are linear in the position
+    double cn = 0.0, cs = 0.0, cf = 0.0;
+    const double end = (double)(first + n);
+    for (int c = blockIdx.x + 1 + threadIdx.x; c < a.n_chunks; c += kScanThreads) {
+        const double nn = __ldcg(a.chunks + 3 * c);
+        cn += nn;
+        cs += __ldcg(a.chunks + 3 * c + 1) + ((double)c * kScanChunk - end) * nn;
+        cf += __ldcg(a.chunks + 3 * c + 2);
+    }
+    long long zero = 0;
+    block_sum2(cn, zero, scratch);
+    block_sum2(cs, zero, scratch);
+    block_sum2(cf, zero, scratch);
+    cn += above.n;
+    cs += above.s + ((double)(above.pos - a.win_base) - end) * above.n;
+    cf += above.f;
+    tensor_scan(a.hist + first, a.hist + a.win + first, n, tensor_unit(a), cn, cs, cf, (double)n, a.above + first, a.above + a.win + first, part);
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.st->scan[a.which ^ 1] = TensorState::Scan{cn, cs, cf, a.win_base};
 }
 
 // <x,q>/h and <q,q> of candidate c from the window [base, base+win) of N and P, shared by `stride` threads.

@@ -127,6 +127,9 @@ def test_extra_negative_level_decides():
     (30_000, 8, False, 4096, 1.0 / 100, 1.0),       # ... many windows
     (30_000, 4, True, 1500, 1e-2, 1.0),             # values beyond the last threshold on both sides
     (66_000, 3, True, 64, 5.0, 1.0),                # fewer bins than candidates
+    (20_001, 4, True, 4096, 0.9999, 1.0),           # one bin more than a block keeps
+    (9_001, 8, False, 4096, 1.0 / 300, 1.0),        # more bins than the workspace holds at once
+    (9_001, 8, True, 4096, 1.0 / 300, 1.0),
 ])
 def test_per_tensor_searches_of_every_kind(n, bits, signed, n_cand, hi_frac, scale):
     import gpu_util
@@ -144,6 +147,32 @@ def test_per_tensor_searches_of_every_kind(n, bits, signed, n_cand, hi_frac, sca
     assert alpha == pytest.approx(ref.alpha, rel=1e-5, abs=0)
     # the error is a binary32 output: below its normal numbers (1.2e-38) it loses digits and then reads as 0
     assert sse == pytest.approx(ref.sse, rel=1e-5, abs=1e-37)
+
+
+@pytest.mark.parametrize("n,bits,signed,n_cand,hi_frac", [
+    (50_003, 8, False, 2048, 0.3), (50_003, 8, True, 2048, 0.01), (9_001, 4, True, 1000, 0.02), (9_001, 8, False, 2048, 0.004),
+])
+@pytest.mark.parametrize("values", ["uniform", "mostly_at_the_end"])
+def test_grids_below_the_largest_value(n, bits, signed, n_cand, hi_frac, values):
+    """Most values lie above the bins that a block keeps, spread out or equal; both workspaces."""
+    import torch
+
+    import gpu_util
+    from oracle import omse_oracle as orc
+    from paper_1902_06822_b200 import binding
+    rng = np.random.default_rng(n + bits)
+    x = rng.random(n, np.float32) if values == "uniform" else np.where(rng.random(n) < 0.7, 1.0, rng.random(n)).astype(np.float32)
+    x = np.where(rng.random(n) < 0.4, -x, x).astype(np.float32) if signed else x
+    ref = orc.activation_scale(x, bits, signed, n_cand, hi_frac, 3)
+    out = gpu_util.activation_scale(x, bits, signed, n_cand, hi_frac, 3)
+    d_x, d = torch.from_numpy(x).cuda(), torch.zeros(2, device="cuda")
+    d_idx, d_curve = torch.zeros(1, dtype=torch.int32, device="cuda"), torch.zeros(n_cand, dtype=torch.float64, device="cuda")
+    binding.omse_activation_scale_static(d_x, n, bits, signed, n_cand, hi_frac, 3, d[:1], d[1:], d_idx, d_curve)
+    for alpha, sse, idx, curve in (out, (d[0].item(), d[1].item(), d_idx.item(), d_curve.cpu().numpy())):
+        np.testing.assert_allclose(curve, ref.sse_curve, rtol=2e-6)
+        assert idx == ref.best_idx or abs(ref.sse_curve[idx] / ref.sse_curve[ref.best_idx] - 1.0) <= 1e-6
+        if idx == ref.best_idx:
+            assert alpha == pytest.approx(ref.alpha, rel=1e-5) and sse == pytest.approx(ref.sse, rel=1e-5)
 
 
 @pytest.mark.parametrize("s,k,bits1,bits2,signed,c1,c2,hf1,hf2,scale", [
