@@ -382,8 +382,11 @@ int enqueue_tensor_search(const TensorEnv& env, omse::TensorArgs& a, int refine_
                 omse::tensor_chunk_scan_kernel<<<(unsigned)a.n_chunks, omse::kScanThreads, 0, s>>>(a);
                 ++*env.launches;
             }
-            omse::tensor_levels_kernel<<<(unsigned)((8 * a.n_cand + 255) / 256), 256, 0, s>>>(a);
-            *env.launches += 2;
+            ++*env.launches;
+            if (!few || a.n_cand > omse::kLevelsHere) {
+                omse::tensor_levels_kernel<<<(unsigned)((8 * a.n_cand + 255) / 256), 256, 0, s>>>(a);
+                ++*env.launches;
+            }
         }
     }
     omse::tensor_finish_kernel<<<1, 1024, 0, s>>>(a);
@@ -1187,10 +1190,6 @@ __global__ void static_begin_kernel(StaticScratch* s) {
     }
 }
 
-__global__ void static_end_kernel(const StaticScratch* s, unsigned int* d_status) {
-    if (threadIdx.x == 0 && d_status) *d_status = s->status;
-}
-
 }  // namespace
 
 extern "C" int omse_activation_scale_static(int device, void* cuda_stream, const float* d_x, int64_t n, int bits,
@@ -1237,13 +1236,11 @@ extern "C" int omse_activation_scale_static(int device, void* cuda_stream, const
     a.sse_out = d_sse;
     a.idx_out = d_best_idx;
     a.status = &sc->status;
+    a.status_out = d_status;
 
     static_begin_kernel<<<1, 32, 0, s>>>(sc);
     unsigned long long not_counted = 0;
     const TensorEnv env = {sd.n_sm, s, &sd.tensor, &not_counted};
-    const int rc = enqueue_tensor_search(env, a, grid->refine_iters);
-    if (rc != OMSE_OK) return rc;
-    static_end_kernel<<<1, 32, 0, s>>>(sc, d_status);
-    return cudaGetLastError() == cudaSuccess ? OMSE_OK : OMSE_ECUDA;
+    return enqueue_tensor_search(env, a, grid->refine_iters);
 }
 

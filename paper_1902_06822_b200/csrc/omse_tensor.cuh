@@ -79,6 +79,7 @@ struct TensorArgs {
     float* delta_out;       // offset mode: receives delta; nullptr = no offset
     unsigned long long* evals;   // executed evaluations (instrumentation), nullable
     unsigned int* status;
+    unsigned int* status_out;    // receives the status word at the end, nullable
 };
 
 __device__ __forceinline__ void tensor_state_init(TensorState* st) {
@@ -551,6 +552,47 @@ __device__ __forceinline__ void tensor_scan(const unsigned long long* hn, const 
     }
 }
 
+// <x,q>/h and <q,q> of candidate c from the window [base, base+win) of N and P, shared by `stride` threads.
+__device__ __forceinline__ void tensor_levels(const double* above_n, const double* above_p, int base, int top, int a1, int levels,
+                                              int first, int stride, double& sx, double& sq) {
+    int j = (base + a1) / (2 * a1) + first;                 // (2j+1)*a1 > base
+    for (; j < levels; j += stride) {
+        const long long m = (long long)(2 * j + 1) * a1;
+        if (m > top) break;
+        const double nn = above_n[m - 1 - base];
+        sx += above_p[m - 1 - base] + (double)m * nn;
+        sq += (double)(2 * j + 1) * nn;
+    }
+}
+// Eight threads per candidate; i: this thread among all of them.  Later windows add to what earlier ones left.
+__device__ __forceinline__ void tensor_levels_of(const TensorArgs& a, int i) {
+    const int c = i >> 3, part = i & 7;
+    double sx = 0.0, sq = 0.0;
+    if (c < a.n_cand) {
+        const int top = min(a.win_base + a.win, a.n_bins);
+        tensor_levels(a.above, a.above + a.win, a.win_base, top, c + 1, a.hi, part, 8, sx, sq);
+        if (a.first_window && part == 0 && c < a.n_bins2) {
+            const double d = (double)(-2 * a.lo - 1), nn = a.above[2 * a.win + c];
+            sx += d * (a.above[2 * a.win + a.n_bins2 + c] + (double)(c + 1) * nn);
+            sq += d * nn;
+        }
+    }
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+        sx += __shfl_xor_sync(0xffffffffu, sx, o);
+        sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    }
+    if (part == 0 && c < a.n_cand) {
+        if (!a.first_window) {
+            sx += a.levels[c];
+            sq += a.levels[a.n_cand + c];
+        }
+        a.levels[c] = sx;
+        a.levels[a.n_cand + c] = sq;
+    }
+}
+__global__ void __launch_bounds__(256) tensor_levels_kernel(const TensorArgs a) { tensor_levels_of(a, blockIdx.x * 256 + threadIdx.x); }
+
 // What the histogram's blocks left beside the bins, by one block: sum x^2, the sum of the values next to an edge, the state of the
 // scan above the topmost window, N and P of the coarse bins.
 __device__ __forceinline__ void tensor_scan_begin(const TensorArgs& a, double unit, double (*part)[3], double* scratch) {
@@ -579,7 +621,8 @@ __device__ __forceinline__ double tensor_unit(const TensorArgs& a) {
     return hist_unit(grid_of(m, a.hi_frac, a.n_cand).step);
 }
 
-// A window that a block scans by itself.
+// A window that a block scans by itself; with few candidates it goes on to their sums.
+constexpr int kLevelsHere = 128;
 __global__ void __launch_bounds__(kScanThreads) tensor_scan_kernel(const TensorArgs a) {
     __shared__ double part[32][3];
     __shared__ double scratch[64];
@@ -590,6 +633,9 @@ __global__ void __launch_bounds__(kScanThreads) tensor_scan_kernel(const TensorA
     double cn = above.n, cs = above.s, cf = above.f;
     tensor_scan(a.hist, a.hist + a.win, a.win, unit, cn, cs, cf, (double)(above.pos - a.win_base), a.above, a.above + a.win, part);
     if (threadIdx.x == 0) a.st->scan[a.which ^ 1] = TensorState::Scan{cn, cs, cf, a.win_base};
+    if (a.n_cand > kLevelsHere) return;
+    __syncthreads();                                       // N and P
+    for (int i0 = 0; i0 < 8 * a.n_cand; i0 += kScanThreads) tensor_levels_of(a, i0 + threadIdx.x);
 }
 
 // Windows of more bins, in two launches: the sums of chunks of kScanChunk bins, then the scan of every chunk from what lies above it.
@@ -643,47 +689,6 @@ __global__ void __launch_bounds__(kScanThreads) tensor_chunk_scan_kernel(const T
     cf += above.f;
     tensor_scan(a.hist + first, a.hist + a.win + first, n, tensor_unit(a), cn, cs, cf, (double)n, a.above + first, a.above + a.win + first, part);
     if (blockIdx.x == 0 && threadIdx.x == 0) a.st->scan[a.which ^ 1] = TensorState::Scan{cn, cs, cf, a.win_base};
-}
-
-// <x,q>/h and <q,q> of candidate c from the window [base, base+win) of N and P, shared by `stride` threads.
-__device__ __forceinline__ void tensor_levels(const double* above_n, const double* above_p, int base, int top, int a1, int levels,
-                                              int first, int stride, double& sx, double& sq) {
-    int j = (base + a1) / (2 * a1) + first;                 // (2j+1)*a1 > base
-    for (; j < levels; j += stride) {
-        const long long m = (long long)(2 * j + 1) * a1;
-        if (m > top) break;
-        const double nn = above_n[m - 1 - base];
-        sx += above_p[m - 1 - base] + (double)m * nn;
-        sq += (double)(2 * j + 1) * nn;
-    }
-}
-
-// Eight threads per candidate.  Later windows add to what earlier ones left.
-__global__ void __launch_bounds__(256) tensor_levels_kernel(const TensorArgs a) {
-    const int i = blockIdx.x * 256 + threadIdx.x, c = i >> 3, part = i & 7;
-    double sx = 0.0, sq = 0.0;
-    if (c < a.n_cand) {
-        const int top = min(a.win_base + a.win, a.n_bins);
-        tensor_levels(a.above, a.above + a.win, a.win_base, top, c + 1, a.hi, part, 8, sx, sq);
-        if (a.first_window && part == 0 && c < a.n_bins2) {
-            const double d = (double)(-2 * a.lo - 1), nn = a.above[2 * a.win + c];
-            sx += d * (a.above[2 * a.win + a.n_bins2 + c] + (double)(c + 1) * nn);
-            sq += d * nn;
-        }
-    }
-#pragma unroll
-    for (int o = 1; o < 8; o <<= 1) {
-        sx += __shfl_xor_sync(0xffffffffu, sx, o);
-        sq += __shfl_xor_sync(0xffffffffu, sq, o);
-    }
-    if (part == 0 && c < a.n_cand) {
-        if (!a.first_window) {
-            sx += a.levels[c];
-            sq += a.levels[a.n_cand + c];
-        }
-        a.levels[c] = sx;
-        a.levels[a.n_cand + c] = sq;
-    }
 }
 
 // squared error of a candidate from its sums; INFINITY when its scale is not usable
@@ -904,6 +909,7 @@ __global__ void __launch_bounds__(256) tensor_pass_kernel(const TensorArgs a) {
             if (a.delta_out) *a.delta_out = st->delta;
             *a.sse_out = (float)total;
             if (a.idx_out) *a.idx_out = st->best_idx;
+            if (a.status_out) *a.status_out = *a.status;
         }
     }
 }
