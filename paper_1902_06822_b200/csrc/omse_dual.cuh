@@ -337,7 +337,7 @@ struct __align__(16) DualPoint {       // one midpoint, in units of alpha1
     float mid, gap_f;
 };
 struct DualPoints {
-    const DualPoint* p;                // [n_cand2][2][kDualPoints], outwards from 0: positive side, negative side
+    const DualPoint* p;                // [n_cand2][kDualPoints], outwards from 0: positive side, then negative side
     const int* n;                      // [n_cand2][2]
 };
 struct __align__(16) DualBin {
@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(kDualPoints) dual_points_kernel(DualPoint* out
         e.gap = sorted[i + 1] - sorted[i];
         e.mid = (float)(0.5 * (sorted[i] + sorted[i + 1]) * (neg ? -1.0 : 1.0));
         e.gap_f = (float)e.gap;
-        out[((size_t)d * 2 + (neg ? 1 : 0)) * kDualPoints + (neg ? below - 1 - i : i - below)] = e;
+        out[(size_t)d * kDualPoints + (neg ? n - 2 - i : i - below)] = e;
     }
     if (i == 0) {
         n_out[2 * d] = n - 1 - below;
@@ -584,8 +584,9 @@ __global__ void __launch_bounds__(kDualBoundThreads, BLOCKS) dual_bound_kernel(c
                     float lin = 0.f, wid = 0.f;
 #pragma unroll 1
                     for (int side = 0; side < 2; ++side) {
-                        const uint4* tab = reinterpret_cast<const uint4*>(pts.p + ((size_t)dv * 2 + side) * kDualPoints);
-                        const int n = __ldg(pts.n + 2 * dv + side);
+                        const int from = side ? __ldg(pts.n + 2 * dv) : 0, n = __ldg(pts.n + 2 * dv + side);
+                        const uint4* tab = reinterpret_cast<const uint4*>(pts.p + (size_t)dv * kDualPoints) + from;
+                        // (what is read beyond n is not used; kDualPoints + 8 entries behind the last table are the workspace's)
                         const DualBin* bs = bins + side * kDualBins;
                         bool go = valid && n > 0;
                         uint4 next[4];                               // the next four points are on their way meanwhile
@@ -597,7 +598,7 @@ __global__ void __launch_bounds__(kDualBoundThreads, BLOCKS) dual_bound_kernel(c
 #pragma unroll
                             for (int j = 0; j < 4; ++j) raw[j] = next[j];
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) next[j] = __ldg(tab + min(k0 + 4 + j, kDualPoints - 1));
+                            for (int j = 0; j < 4; ++j) next[j] = __ldg(tab + k0 + 4 + j);
                             // no branch, so that the four reads of the bins are in flight together: a point outside takes
                             // part with gap 0
 #pragma unroll

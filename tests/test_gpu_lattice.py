@@ -185,6 +185,8 @@ def test_grids_below_the_largest_value(n, bits, signed, n_cand, hi_frac, values)
     (3, 600, 4, 4, True, 12, 12, 3.0, 0.25, 1.0),       # scales beyond max|x|
     (3, 600, 4, 4, True, 8, 8, 1.0, 0.25, 2.0 ** -95),  # small values
     (2, 28672, 2, 3, True, 6, 6, 1.0, 0.25, 1.0),       # the longest row
+    (3, 300, 4, 4, True, 3, 1024, 1.0, 0.9, 1.0),       # most ratios: sorted points of all of them in the workspace
+    (3, 300, 2, 4, False, 2, 1024, 1.0, 1.0, 1.0),
     (3, 400, 4, 4, True, 4, 4, 1e-5, 0.25, 1.0),        # first scale far below max|x| ...
     (3, 400, 4, 4, True, 5, 5, 1e-7, 0.25, 1.0),        # ... and below its last place: equal errors take the lowest first code
     (3, 400, 3, 3, False, 5, 5, 1e-9, 0.5, 1.0),
