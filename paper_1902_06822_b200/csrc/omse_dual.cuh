@@ -476,10 +476,12 @@ __global__ void __launch_bounds__(kDualBoundThreads, BLOCKS) dual_bound_kernel(c
             float a1_last, a2_last;
             dual_scales(m, a, a.n_cand1 - 1, a.n_cand2 - 1, a1_last, a2_last);
             bool degenerate = any_bad || !(m > 0.f) || !(a2_last >= FLT_MIN);
-            // The reference squares errors in binary32: where that leaves its range, equal squares make it take the lowest
-            // code, and only the reference arithmetic itself can tell the pairs apart
-            const bool extreme = !(m > 1e-14f && m < 1e18f);
-            double bv = INFINITY;
+            // The reference squares errors in binary32.  Below its range squares that round to the same number make it take the
+            // lowest of their codes: a window of first codes may not hold it (`every`), and a value's error may be that much above
+            // its smallest one (in the margin).  Above its range every square may be infinite: a pair has an upper bound only if
+            // its whole error is finite.  What cannot be told apart by the bounds is left to the reference arithmetic.
+            const bool every = !(m > 1e-14f && m < 1e18f);
+            double bv = INFINITY, inv_es = 0.0;
             int bi = 0x7fffffff;
             if (!degenerate) {                                       // uniform over the block
                 // ---- histogram: bin b of a side holds the values with |x|/w in [b, b+1); a power of two keeps 1/w finite
@@ -567,7 +569,8 @@ __global__ void __launch_bounds__(kDualBoundThreads, BLOCKS) dual_bound_kernel(c
                 //      own rounding (es, the estimate) can add is in the margin.
                 const float scale_pre = pre;
                 const double w_true = (double)w / (double)scale_pre;
-                const double margin0 = 2e-7 * es + ls * w_true * fq;
+                const double margin0 = 2e-7 * es + ls * w_true * fq + 3e-45 * (double)k;
+                inv_es = 1.0 / es;
                 const float inv_w = __fdiv_rn(1.0f, w);
                 // A warp takes 8 neighbouring alpha1 of 4 neighbouring ratios at a time: lanes of similar alpha1 have about as
                 // many midpoints below max|x|, a lane keeps its own sums, and the points of a ratio are read by 8 lanes at once.
@@ -627,10 +630,9 @@ __global__ void __launch_bounds__(kDualBoundThreads, BLOCKS) dual_bound_kernel(c
                         const double unit = 2.0 * w_true * w_true * (double)s;
                         const double est = es - unit * (acc - (double)lin);
                         const double off = unit * (double)wid * 1.00001 + margin0 + 1e-5 * fabs(est);
-                        float low = ok ? (float)((est - off) * (1.0 - (est > off ? 1e-7 : -1e-7))) : INFINITY;
-                        if (extreme && ok) low = 0.f;                // every pair is re-scored
-                        curve[c * a.n_cand2 + d] = low;
-                        const double up = extreme ? 1e300 : est + off;
+                        // (kept as a share of sum x^2, which may lie outside binary32)
+                        curve[c * a.n_cand2 + d] = ok ? (float)((est - off) * inv_es * (1.0 - (est > off ? 1e-7 : -1e-7))) : INFINITY;
+                        const double up = est + off < 3e38 ? est + off : 1e300;
                         if (ok && (up < bv || (up == bv && c * a.n_cand2 + d < bi))) {
                             bv = up;
                             bi = c * a.n_cand2 + d;
@@ -647,7 +649,7 @@ __global__ void __launch_bounds__(kDualBoundThreads, BLOCKS) dual_bound_kernel(c
             float alpha1 = 0.f, alpha2 = 0.f;
             int best_pair = -1;
             if (!degenerate) {
-                const float top = extreme ? FLT_MAX : (float)(bv * (1.0 + 1e-7));
+                const float top = (float)fmin(bv * inv_es * (1.0 + 1e-7), (double)FLT_MAX);
                 auto rescore_all = [&](int begin, int end) -> int {  // lists the survivors of [begin, end); returns their number
                     __syncthreads();
                     if (tid == 0) s_n = 0;
@@ -665,7 +667,7 @@ __global__ void __launch_bounds__(kDualBoundThreads, BLOCKS) dual_bound_kernel(c
                 auto rescore = [&](int p) {                          // the codes of the reference arithmetic, fp64 sum
                     float a1, a2;
                     dual_scales(m, a, p / a.n_cand2, p % a.n_cand2, a1, a2);
-                    dc.set(a1, a2, a, extreme);
+                    dc.set(a1, a2, a, every);
                     double ss = 0.0;
                     long long zero = 0;
                     for (int i = tid; i < k; i += nthr) {
@@ -699,7 +701,7 @@ __global__ void __launch_bounds__(kDualBoundThreads, BLOCKS) dual_bound_kernel(c
             }
 
             // ---- final codes, squared error, emission: one output byte pair per thread
-            dc.set(alpha1, alpha2, a, extreme);
+            dc.set(alpha1, alpha2, a, every);
             double ss = 0.0;
             const int o = (int)(row_base & 1);
             const int n_pairs = (k + o + 1) >> 1;

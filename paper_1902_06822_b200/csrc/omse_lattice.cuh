@@ -59,7 +59,8 @@ struct TeamScratch {
 };
 
 __device__ __forceinline__ unsigned int warp_umax(unsigned int v) { return __reduce_max_sync(0xffffffffu, v); }
-__device__ __forceinline__ float warp_allsum(float v) {
+template <class V>
+__device__ __forceinline__ V warp_allsum(V v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;

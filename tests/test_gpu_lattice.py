@@ -234,3 +234,19 @@ def test_residual_rows_by_every_search(s, k, bits, n_cand, hi_frac, scale):
     if pk is not None:
         for j in range(2):
             assert np.array_equal(pk[j], orc.pack_int4(q[j]))
+
+
+@pytest.mark.parametrize("bits1,bits2,signed,exponent", [
+    (4, 4, True, -48), (4, 4, True, -56), (3, 4, False, -64), (4, 4, True, -68), (4, 4, True, -72), (2, 2, True, -76),    # squares below binary32
+    (4, 4, True, 58), (4, 4, True, 62), (2, 4, False, 64), (4, 4, True, 66), (4, 4, True, 70),                            # ... and above
+])
+def test_dual_search_at_the_ends_of_binary32(bits1, bits2, signed, exponent):
+    """The reference squares errors in binary32: equal squares take the lowest first code, infinite ones none."""
+    import gpu_util
+    from oracle import omse_oracle as orc
+    t = synth.student_t3(3 * 600, seed=84, tensor_id=exponent % 97).reshape(3, 600) * np.float32(2.0 ** exponent)
+    alpha, sse, idx, q, _ = gpu_util.dual_quantize(t, bits1, bits2, signed, 8, 8, 1.0, 0.25, True, False)
+    ref = orc.dual_rows(t, bits1, bits2, signed, 8, 8, 1.0, 0.25)
+    assert np.array_equal(idx, ref.best_idx) and np.array_equal(alpha, ref.alpha)
+    assert np.array_equal(q.reshape(2, 3, 600), ref.codes)
+    np.testing.assert_allclose(sse, ref.sse.astype(np.float32), rtol=1e-5, atol=1e-37)
