@@ -66,7 +66,7 @@ struct omse_ctx {
     omse::RowTensor* d_tensors;   // device, OMSE_MAX_BATCH descriptors of a batched launch
     // per-context launch bookkeeping (a context is used by one host thread at a time, so no lock)
     bool attr_rows[5], attr_dual[3];   // opt-in shared-memory attribute set, per kernel
-    LaunchShape seen[16];                           // blocks per SM of the row-kernel launch shapes met so far
+    LaunchShape seen[16];                           // blocks per SM of the launch shapes met so far
     int n_seen, next_seen;
     TensorLaunches tensor;                          // the same for the per-tensor kernels
     unsigned long long n_launches;                  // kernels launched since the last omse_read_launches
@@ -111,26 +111,31 @@ void bounds(int bits, int is_signed, int* lo, int* hi) {
 // Kernels of the row searches, by path (how rows are mapped to threads) and by what a launch needs.
 enum RowPath { kPathShort, kPathBlock, kPaths };     // short rows: a warp or some of its lanes per row
 
+// Blocks per SM of a launch shape, remembered: the query costs more than a small launch.  0: the query failed, or none fits.
+int blocks_per_sm(omse_ctx* ctx, int id, const void* kernel, int threads, size_t smem) {
+    for (int i = 0; i < ctx->n_seen; ++i)
+        if (ctx->seen[i].kernel == id && ctx->seen[i].threads == threads && ctx->seen[i].smem == smem) return ctx->seen[i].occ;
+    int occ = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, smem) != cudaSuccess || occ < 1) return 0;
+    ctx->seen[ctx->next_seen] = LaunchShape{id, threads, smem, occ};   // round robin once the table is full
+    ctx->next_seen = (ctx->next_seen + 1) % 16;
+    if (ctx->n_seen < 16) ++ctx->n_seen;
+    return occ;
+}
+constexpr int kRowKernels = 5;       // ids of launch shapes: the row kernels, then the dual search's
+
 int launch_rows_kernel(omse_ctx* ctx, const omse::RowArgs& a, int path, bool ext, int threads, size_t smem) {
     typedef void (*Kernel)(const omse::RowArgs);
-    const Kernel kernels[5] = {omse::rows_kernel<false, false>, omse::rows_kernel<true, false>, omse::rows_kernel<false, true>,
-                               omse::rows_short_kernel<false>, omse::rows_short_kernel<true>};
+    const Kernel kernels[kRowKernels] = {omse::rows_kernel<false, false>, omse::rows_kernel<true, false>, omse::rows_kernel<false, true>,
+                                         omse::rows_short_kernel<false>, omse::rows_short_kernel<true>};
     const int id = path == kPathShort ? (a.short_direct ? 4 : 3) : ext ? 1 : a.packed_counts ? 2 : 0;
     const Kernel kernel = kernels[id];
     if (!ctx->attr_rows[id]) {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess) return OMSE_ECUDA;
         ctx->attr_rows[id] = true;
     }
-    // blocks per SM for this launch shape (remembered: the query costs more than a small launch)
-    int occ = 0;
-    for (int i = 0; i < ctx->n_seen; ++i)
-        if (ctx->seen[i].kernel == id && ctx->seen[i].threads == threads && ctx->seen[i].smem == smem) occ = ctx->seen[i].occ;
-    if (occ == 0) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, smem) != cudaSuccess || occ < 1) return OMSE_ECUDA;
-        ctx->seen[ctx->next_seen] = LaunchShape{id, threads, smem, occ};   // round robin once the table is full
-        ctx->next_seen = (ctx->next_seen + 1) % 16;
-        if (ctx->n_seen < 16) ++ctx->n_seen;
-    }
+    const int occ = blocks_per_sm(ctx, id, (const void*)kernel, threads, smem);
+    if (occ == 0) return OMSE_ECUDA;
     long long grid = (long long)ctx->n_sm * occ;
     const long long teams = path == kPathShort ? (a.n_units + threads / 32 - 1) / (threads / 32) : a.n_units;
     if (grid > teams) grid = teams;
@@ -1015,8 +1020,8 @@ int omse_dual_quantize(omse_ctx* ctx, const float* d_t, int64_t n_kernels, int64
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess) return OMSE_ECUDA;
         ctx->attr_dual[id] = true;
     }
-    int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, smem) != cudaSuccess || occ < 1) return OMSE_ECUDA;
+    const int occ = blocks_per_sm(ctx, kRowKernels + id, kernel, threads, smem);
+    if (occ == 0) return OMSE_ECUDA;
     long long blocks = (long long)ctx->n_sm * occ;
     if (blocks > n_units) blocks = n_units;
     // the context workspace holds the sorted points of every alpha2, then each block's grid values of its current row
