@@ -197,9 +197,9 @@ int launch_rows(omse_ctx* ctx, omse::RowArgs& a, long long max_k, int path) {
     // Rows that are shorter than this evaluate candidates instead of making a histogram.  In a small launch a row's chain of steps
     // counts, in a large one the barriers: 32 threads per row then.  (Two tensors of 4 bits, 1024 candidates, histogram and candidates:
     // 38,836 rows of 27 values 993 us and 326, 16,384 of 64 429 and 203, 10,485 of 100 283 and 161, 7133 of 147 205 and 163; 64
-    // rows of 27 22.8 us and 18.7, of 64 22.7 and 18.7, of 100 22.7 and 23.)
+    // rows of 27 22.8 us and 18.5, of 64 22.7 and 18.5, of 100 22.6 and 19.0, of 147 with 200 candidates 20.5 and 21.3.)
     const bool many = a.n_units >= 8ll * ctx->n_sm;
-    if (max_k <= (many ? 160 : 64)) {
+    if (max_k <= (many ? 160 : 128)) {
         ext = true;
         a.direct = k4 >= 32 ? 2 : k4 >= 16 ? 1 : 0;
         smem = fixed + (size_t)((a.n_cand + 3) & ~3) * 4;

@@ -212,6 +212,7 @@ def test_dual_search_by_bounds(s, k, bits1, bits2, signed, c1, c2, hf1, hf2, sca
     (1201, 127, 4, 1, 1.0, 1.0), (1201, 128, 4, 2, 1.0, 1.0),       # ... four; one and two candidates
     (1201, 160, 4, 4096, 1.0, 1.0), (1201, 161, 4, 4096, 1.0, 1.0), # one value more: by histogram
     (9, 27, 8, 1024, 1.0, 1.0), (9, 36, 4, 17, 0.3, 1.0), (9, 64, 4, 1024, 1.0, 1.0),     # small launches: 64 and 128 threads
+    (9, 128, 4, 1024, 1.0, 1.0), (9, 129, 8, 1024, 1.0, 1.0),                             # ... the last row, by histogram
     (1201, 31, 4, 300, 1.0, 2.0 ** -112), (9, 40, 2, 300, 0.5, 2.0 ** 59),                # squares outside binary32
     (40, 700, 4, 4096, 0.1, 1.0), (40, 700, 8, 4096, 0.01, 2.0 ** -100),                  # by splits: bins do not fit
     (3, 12_287, 4, 4096, 0.1, 1.0), (3, 12_289, 4, 4096, 0.25, 1.0),                      # the last row by splits, windows
