@@ -141,7 +141,8 @@ int omse_quantize_weights_batched(omse_ctx* ctx, const omse_weight_tensor* tenso
  * Per-tensor MMSE scale for an activation tensor (Section 3.7, first equation): one scale for
  * all n elements of d_x.  Outputs: d_alpha[1], d_sse[1] (float), d_best_idx[1] (nullable),
  * d_sse_curve[n_cand] (nullable, double): the squared error at every candidate, i.e. the curve of
- * Figure 1, accumulated in binary32 blocks of 128 elements folded into binary64.
+ * Figure 1, from an exact integer histogram and binary64 sums: within 2e-6 of the error that the codes give, up to what
+ * values within 2^-23 of a rounding threshold contribute (they may be counted with either neighbouring code).
  * n >= 0 (0 is treated as a degenerate tensor).  d_x must be 16-byte aligned (128-bit loads).
  */
 int omse_activation_scale(omse_ctx* ctx, const float* d_x, int64_t n, int bits, int is_signed,
@@ -372,7 +373,8 @@ int omse_pack_int4(omse_ctx* ctx, const int8_t* d_codes, int64_t n, int is_signe
  * Sharing: all calls on a device use the same array.  Each call re-initialises what must start
  * at zero, so calls that follow one another on one stream are independent; calls that can overlap
  * on the GPU (different streams, different threads) race on the array and give wrong results.
- * Results equal omse_activation_scale's up to the grouping of partial sums (same tolerances).
+ * Results equal omse_activation_scale's within the same tolerances; a tensor that the context call searches in one kernel, on
+ * chip, goes through a sequence of launches here, so sums are grouped differently.
  */
 #define OMSE_STATIC_MAX_CANDIDATES 2048
 #define OMSE_STATIC_SCRATCH_BYTES (4u * 1024u * 1024u + 32u * 1024u)
@@ -387,8 +389,9 @@ int omse_last_device_status(omse_ctx* ctx, uint32_t* host_out);
 /* Instrumentation (no counterpart in the paper): synchronises the stream and returns in *host_out how many element
  * evaluations the search kernels of this context executed since the last read, then clears the counter.  Placing an
  * element of a row on the grid counts as one, re-scoring a row at one candidate as one per element; where candidates are
- * evaluated one by one (rows of up to 1024 elements) every (element, candidate) evaluation counts.  For
- * omse_dual_quantize the unit is (element, pair, first code).  omse_activation_scale_static does not count. */
+ * evaluated one by one (rows of up to 1024 elements, grids that end far below max|x|) every (element, candidate)
+ * evaluation counts.  For omse_dual_quantize the unit is (element, pair, first code); rows whose pairs are decided by bounds
+ * count once per element and re-scored pair.  omse_activation_scale_static does not count. */
 int omse_read_evaluations(omse_ctx* ctx, uint64_t* host_out);
 
 /* Instrumentation (no counterpart in the paper): the number of kernels the calls on this context have launched since

@@ -1,5 +1,5 @@
 // Host side of the C interface declared in include/omse.h: argument checks, launch shapes, context.
-// Every step of the method runs in the kernels of omse_rows.cuh / omse_tensor.cuh; there is no
+// Every step of the method runs in the kernels of omse_rows*.cuh, omse_tensor.cuh and omse_dual.cuh; there is no
 // host arithmetic on tensor data and no CPU fallback.
 #include "../../include/omse.h"
 
@@ -10,22 +10,16 @@
 #include <new>
 #include <vector>
 
-#ifndef OMSE_SMALL_K
-#define OMSE_SMALL_K 1024           /* rows up to this length are searched in the registers of a warp or of some of its lanes:
-                                       40,000 rows of 1000 values 517 us against 843 by blocks */
-#endif
-
-#ifndef OMSE_DUAL_BOUND_K
-#define OMSE_DUAL_BOUND_K 256       /* dual search: rows at least this long go by histogram and bounds (16 rows of 256 values
-                                       58 us against 100 by the sweep, of 128 values 55 by the sweep, whose time is proportional to the length) */
-#endif
-
 #include "omse_rows.cuh"
 #include "omse_tensor.cuh"
 #include "omse_dual.cuh"
 
 namespace {
 
+constexpr long long kSmallK = 1024;           // rows up to this length are searched in the registers of a warp or of some of its lanes:
+                                              // 40,000 rows of 1000 values 517 us against 843 by blocks
+constexpr long long kDualBoundK = 256;        // dual search: rows at least this long go by histogram and bounds (16 rows of 256 values 58 us
+                                              // against 100 by the sweep, of 128 values 55 by the sweep, whose time is proportional to the length)
 constexpr size_t kPartialBytes = 16u << 20;   // per-block partial sums of the per-tensor search
 constexpr size_t kSmSmem = 233472;            // shared memory of an SM, and what a block of the row kernels takes beside the dynamic part:
 constexpr size_t kBlockSmem = 1024 + 1232;    // 1 KB for the system, static
@@ -459,8 +453,8 @@ struct ListMode {
 };
 
 // Launch for a list of weight tensors (bounds already set by the caller).
-int quantize_list(omse_ctx* ctx, std::vector<omse::RowTensor>& list, long long max_k, int bits, int is_signed,
-                  const omse_grid* grid, const ListMode& mode = ListMode()) {
+int quantize_list(omse_ctx* ctx, std::vector<omse::RowTensor>& list, int bits, int is_signed, const omse_grid* grid,
+                  const ListMode& mode = ListMode()) {
     if (list.empty()) return OMSE_OK;
     DeviceScope dev(ctx->device);
     if (!dev.ok()) return OMSE_ECUDA;
@@ -487,12 +481,12 @@ int quantize_list(omse_ctx* ctx, std::vector<omse::RowTensor>& list, long long m
     const bool plain = mode.solver == 0 && mode.n_delta == 0;   // the block path implements everything else
     long long short_rows = 0, short_elements = 0, short_warps = 0;
     for (const auto& t : list)
-        if (t.K <= OMSE_SMALL_K) {
+        if (t.K <= kSmallK) {
             short_rows += t.S;
             short_elements += t.S * t.K;
             short_warps += (t.S << omse::short_lanes(t.K)) / 32;
         }
-    const long long short_k = short_rows >= 8ll * ctx->n_sm ? OMSE_SMALL_K : 160;
+    const long long short_k = short_rows >= 8ll * ctx->n_sm ? kSmallK : 160;
     a.short_direct = short_rows < (a.hi[0] > 63 ? 96ll : 48ll) * ctx->n_sm && short_elements < 5120ll * ctx->n_sm;
     int spread = 0;                                             // more lanes per row where the warps do not fill the GPU
     while (spread < 5 && (short_warps << (spread + 1)) <= 16ll * ctx->n_sm) ++spread;
@@ -773,7 +767,6 @@ int omse_quantize_weights_batched(omse_ctx* ctx, const omse_weight_tensor* tenso
         return OMSE_EINVAL;
     std::vector<omse::RowTensor> list;
     list.reserve((size_t)n_tensors);
-    long long max_k = 0;
     for (int i = 0; i < n_tensors; ++i) {
         const omse_weight_tensor& u = tensors[i];
         if (u.n_kernels < 0 || u.kernel_len < 1 || u.kernel_len > OMSE_MAX_KERNEL_LEN || u.n_kernels > (int64_t)1 << 40)
@@ -786,9 +779,8 @@ int omse_quantize_weights_batched(omse_ctx* ctx, const omse_weight_tensor* tenso
         omse::RowTensor t;
         fill_tensor(t, u.d_w, u.n_kernels, u.kernel_len, u.d_alpha, u.d_sse, u.d_best_idx, u.d_codes, u.d_packed);
         list.push_back(t);
-        if (u.kernel_len > max_k) max_k = u.kernel_len;
     }
-    return quantize_list(ctx, list, max_k, bits, is_signed, grid);
+    return quantize_list(ctx, list, bits, is_signed, grid);
 }
 
 int omse_quantize_weights_offset(omse_ctx* ctx, const float* d_w, int64_t n_kernels, int64_t kernel_len, int bits,
@@ -804,7 +796,7 @@ int omse_quantize_weights_offset(omse_ctx* ctx, const float* d_w, int64_t n_kern
     std::vector<omse::RowTensor> list(1);
     fill_tensor(list[0], d_w, n_kernels, kernel_len, d_alpha, d_sse, d_best_idx, d_codes, d_packed);
     list[0].delta = d_delta;
-    return quantize_list(ctx, list, kernel_len, bits, /*is_signed=*/0, grid);
+    return quantize_list(ctx, list, bits, /*is_signed=*/0, grid);
 }
 
 int omse_residual_quantize(omse_ctx* ctx, const float* d_t, int64_t n_kernels, int64_t kernel_len, const int* bits,
@@ -888,7 +880,7 @@ int omse_quantize_weights_solver(omse_ctx* ctx, const float* d_w, int64_t n_kern
     ListMode mode;
     mode.solver = solver;
     mode.solver_iters = n_iter;
-    return quantize_list(ctx, list, kernel_len, bits, is_signed, grid, mode);
+    return quantize_list(ctx, list, bits, is_signed, grid, mode);
 }
 
 int omse_quantize_weights_affine(omse_ctx* ctx, const float* d_w, int64_t n_kernels, int64_t kernel_len, int bits,
@@ -909,7 +901,7 @@ int omse_quantize_weights_affine(omse_ctx* ctx, const float* d_w, int64_t n_kern
     ListMode mode;
     mode.n_delta = offsets->n_delta;
     mode.off_frac = offsets->off_frac;
-    return quantize_list(ctx, list, kernel_len, bits, /*is_signed=*/0, grid, mode);
+    return quantize_list(ctx, list, bits, /*is_signed=*/0, grid, mode);
 }
 
 int omse_quantize_key_layers(omse_ctx* ctx, const omse_key_layer* layers, int n_layers, int bits, int is_signed,
@@ -940,16 +932,14 @@ int omse_quantize_key_layers(omse_ctx* ctx, const omse_key_layer* layers, int n_
     // 3. one launch over all layers for the second tensor: blocks skip the layers whose flag is 0, so the host
     //    never reads the flags; each row's residual is rebuilt on chip from the first scale
     std::vector<omse::RowTensor> list((size_t)n_layers);
-    long long max_k = 0;
     for (int l = 0; l < n_layers; ++l) {
         const omse_key_layer& L = layers[l];
         fill_tensor(list[l], L.first.d_w, L.first.n_kernels, L.first.kernel_len, L.d_alpha2, L.d_sse2, nullptr,
                     L.d_codes2, L.d_packed2);
         list[l].prior_alpha = L.first.d_alpha;
         list[l].gate = d_is_key + l;
-        if (L.first.kernel_len > max_k) max_k = L.first.kernel_len;
     }
-    rc = quantize_list(ctx, list, max_k, bits, is_signed, grid);
+    rc = quantize_list(ctx, list, bits, is_signed, grid);
     if (rc != OMSE_OK) return rc;
     // 4. compression ratio of the result (one or two quantized tensors per layer)
     if (d_cr) {
@@ -1006,7 +996,7 @@ int omse_dual_quantize(omse_ctx* ctx, const float* d_t, int64_t n_kernels, int64
     a.rows_per_unit = (d_packed && (kernel_len & 1)) ? 2 : 1;
     // Which of the two kernels: see dual_bound_kernel.  Where alpha1 comes near the last place of max|x| (2^-23 of it) binary32 cannot
     // tell neighbouring first codes apart and the reference takes the lowest one, which only the full enumeration finds.
-    const bool bound = kernel_len >= OMSE_DUAL_BOUND_K && bits1 + bits2 <= 8 && grid->hi_frac2 <= 1.0f &&
+    const bool bound = kernel_len >= kDualBoundK && bits1 + bits2 <= 8 && grid->hi_frac2 <= 1.0f &&
                        (double)grid->hi_frac1 * 1048576.0 >= (double)grid->n_cand1;
     const long long n_units = (n_kernels + a.rows_per_unit - 1) / a.rows_per_unit;
     const bool few = n_units <= 3ll * ctx->n_sm;

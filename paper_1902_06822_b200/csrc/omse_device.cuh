@@ -140,6 +140,18 @@ __device__ __forceinline__ void block_sum2(double& d, long long& q, double* scra
     }
 }
 
+__device__ __forceinline__ void block_max(float& a, double* scratch) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = (blockDim.x + 31) >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a = fmaxf(a, __shfl_down_sync(0xffffffffu, a, o));
+    float* fs = reinterpret_cast<float*>(scratch);
+    __syncthreads();
+    if (lane == 0) fs[warp] = a;
+    __syncthreads();
+    a = fs[0];
+    for (int w = 1; w < nwarp; ++w) a = fmaxf(a, fs[w]);
+}
+
 __device__ __forceinline__ void block_max2(float& a, float& b, double* scratch) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = (blockDim.x + 31) >> 5;
 #pragma unroll

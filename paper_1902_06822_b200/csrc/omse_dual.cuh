@@ -11,9 +11,9 @@
 // the distance from x/alpha1 up to the asymmetry of Z_p2, which can only move the winner to the other
 // neighbour of x/alpha1.  So the codes within (max|Z_p2| + 1/2)*alpha2/alpha1 + 1/2 of round(x/alpha1),
 // and at least the two neighbours, hold the minimum (codes beyond Z_p1 collapse onto its ends).
-// Grid values are compared in fp32 (blocks of 64 elements folded
-// into fp64); pairs within the fp32 noise band of the minimum are re-scored with the full
-// enumeration in the reference arithmetic, and the final codes always use the full enumeration.
+// Grid values are compared in fp32 (blocks of 64 elements folded into fp64); pairs within the fp32 noise band of the minimum
+// are re-scored in the reference arithmetic.  dual_kernel does that, and the final codes, with the full enumeration,
+// dual_bound_kernel below with the window, except for rows at the ends of binary32, where equal squares decide.
 #pragma once
 #include "omse_rows.cuh"
 
@@ -103,8 +103,7 @@ __global__ void __launch_bounds__(kDualThreads) dual_kernel(const DualArgs a) {
                 else bad = true;
             }
             if (bad) st |= 1u;
-            float dummy = 0.f;
-            block_max2(mx, dummy, scratch);
+            block_max(mx, scratch);
             const float m = mx;
             float a1_last, a2_last;
             dual_scales(m, a, a.n_cand1 - 1, a.n_cand2 - 1, a1_last, a2_last);
@@ -470,8 +469,7 @@ __global__ void __launch_bounds__(kDualBoundThreads, BLOCKS) dual_bound_kernel(c
             for (int i = tid; i < 2 * kDualBins; i += nthr) reinterpret_cast<uint4*>(bins)[i] = make_uint4(0u, 0u, 0u, 0u);
             if (bad) st |= 1u;
             const bool any_bad = __syncthreads_or(bad) != 0;
-            float l1b = l1;
-            block_max2(mx, l1b, scratch);                            // (l1b: a maximum nobody needs)
+            block_max(mx, scratch);
             const float m = mx;
             float a1_last, a2_last;
             dual_scales(m, a, a.n_cand1 - 1, a.n_cand2 - 1, a1_last, a2_last);

@@ -1,4 +1,4 @@
-// Short kernels (up to 896 weights, e.g. 3x3x3 or 64x3x3): a group of G = 1, 2, 4, ... 32 lanes of a warp owns a row, which
+// Short kernels (up to 1024 weights, e.g. 3x3x3 or 64x3x3): a group of G = 1, 2, 4, ... 32 lanes of a warp owns a row, which
 // sits in their registers, and looks for the best candidate by evaluating a few of them, one after the other.
 //
 // W(alpha) = sum_i sum_j (|x_i| - (j - 1/2)*alpha)_+ is convex, and the error is E - 2*alpha*W, so the errors at two
@@ -25,15 +25,10 @@
 
 namespace omse {
 
-#ifndef OMSE_SHORT_BLOCKS
-#define OMSE_SHORT_BLOCKS 5
-#endif
-
 constexpr int kShortThreads = 128;       // blocks of four warps: five per SM at 96 registers, against four at 128 and six at 80
-                                         // (rows of 147 values 492 us, 503 and 514; of 27 values 1148, 1172 and 1267)
+constexpr int kShortBlocks = 5;          // (rows of 147 values 492 us, 503 and 514; of 27 values 1148, 1172 and 1267)
 constexpr int kShortMinQuads = 3;
 constexpr int kShortQuads = 10;          // float4s of a row per lane, at most
-constexpr int kShortMaxK = 32 * 4 * kShortQuads;
 
 // Lanes per row (log2) for rows of k values.
 inline int short_lanes(long long k) {
@@ -145,7 +140,7 @@ __device__ __forceinline__ ShortResult short_search(const ShortSmem& sm, const S
     const float sat_alpha = r.search ? fmaxf(__fdividef(r.mpos, r.fhi + 0.5f), __fdividef(r.mneg, 0.5f - r.flo)) * 1.00002f : 0.f;
     const u64 M2 = pack2(kMagic, kMagic), NM2 = pack2(-kMagic, -kMagic);
     const float clo = kMagic + r.flo, chi = kMagic + r.fhi;
-    // squared error of the row at candidate a1 - 1
+    // squared error of the row at candidate a1 - 1; the reciprocal by one step of Newton's method from the quick one
     auto error_at = [&](float a1) -> float {
         const float ac = __fmul_rn(a1, r.step);
         const float al = ac * r.sc, rough = quick_reciprocal(al), inv = fmaf(fmaf(-al, rough, 1.0f), rough, rough);
@@ -680,7 +675,7 @@ __device__ __forceinline__ void short_step(const RowArgs& a, const RowTensor& T,
 
 // DIRECT: all lanes on one row, a candidate each (lanes = 5).
 template <bool DIRECT>
-__global__ void __launch_bounds__(kShortThreads, DIRECT ? 6 : OMSE_SHORT_BLOCKS) rows_short_kernel(const RowArgs a) {
+__global__ void __launch_bounds__(kShortThreads, DIRECT ? 6 : kShortBlocks) rows_short_kernel(const RowArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     ShortSmem sm;

@@ -13,8 +13,8 @@
 //   to re-score -> re-score -> polish x R -> final error.
 // Grid-wide sums there use "the last block to arrive reduces" (a ticket from atomicAdd, no waiting).
 // Measured on one B200 against a sweep of the candidates over the values each does not code as 0: 51,380,224 post-ReLU
-// values with 2048 candidates 697 -> 364 us, 25,088 with 50 candidates 53 -> 24 us, 1,605,633 values of both signs with
-// offset and 500 candidates 230 -> 50 us.
+// values with 2048 candidates 655 -> 364 us, 25,088 with 50 candidates 53 -> 21 us, 1,605,633 values of both signs with
+// offset and 500 candidates 229 -> 50 us.
 #pragma once
 #include "omse_lattice.cuh"
 

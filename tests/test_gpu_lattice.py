@@ -25,14 +25,14 @@ pytestmark = pytest.mark.gpu
     (6, 500, 3, True, 64, 1.0, 2.0 ** 59),          # the sum of squares overflows binary32
     (7, 1, 4, True, 1, 1.0, 1.0),
     (9, 33, 8, True, 7, 1.0, 1.0),
-    (2500, 33, 4, True, 1000, 1.0, 1.0),            # warp per row: shortest, longest; one more: block per row
+    (2500, 33, 4, True, 1000, 1.0, 1.0),            # lanes per row: two; long rows of the same path
     (2500, 896, 4, True, 1024, 1.0, 1.0),
     (2500, 897, 4, True, 1024, 1.0, 1.0),
-    (2500, 193, 4, True, 1024, 1.0, 2.0 ** -112),   # warp per row: values scaled, squares would underflow ...
+    (2500, 193, 4, True, 1024, 1.0, 2.0 ** -112),   # values scaled, squares would underflow ...
     (2500, 191, 2, True, 300, 0.5, 2.0 ** 59),      # ... or overflow
     (2500, 100, 3, True, 4096, 2.0, 1.0),           # coarse candidates beyond max|x|, wide neighbourhood of the minimum
     (2500, 70, 2, True, 4096, 1.0, 1.0),            # ... of more candidates than are kept
-    (151_600, 9, 4, True, 1024, 1.0, 1.0),          # thread per row: every register class, even and odd lengths,
+    (151_600, 9, 4, True, 1024, 1.0, 1.0),          # one lane per row: even and odd lengths,
     (151_600, 17, 4, False, 300, 1.0, 1.0),         # a last unit that is not full
     (151_553, 32, 8, True, 64, 1.0, 1.0),
     (2500, 147, 3, True, 1300, 1.0 / 3, 1.0),

@@ -42,8 +42,8 @@ def _divisors(limit):
 
 @pytest.mark.parametrize("s,k", [(5, 2048), (3, 9000), (2500, 256), (2500, 64), (9700, 27), (6, 300)])
 def test_exact_ties_beyond_any_list_on_every_row_path(gpu, s, k):
-    """34 candidates with error exactly 0 on every row; long regrouped rows, element groups, batched short
-    rows (with and without regrouping), thread-per-row and plain block-per-row paths."""
+    """34 candidates with error exactly 0 on every row; long rows, short rows by several lanes
+    and by one, and rows by a block."""
     assert len(_divisors(127)) == 34
     w = _tie_rows(s, k, seed=k)
     rows = None if s <= 10 else np.unique(np.concatenate([np.arange(0, s, 41), [s - 1]]))

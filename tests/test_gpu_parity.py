@@ -361,7 +361,7 @@ def test_algorithm_1_history_and_mixed_signedness_match_oracle(gpu):
     assert torch.equal(hist[-1], sse)
 
 
-# ---------------------------------------------------------------- very short rows in large numbers: a thread per row
+# ---------------------------------------------------------------- very short rows in large numbers: one lane of a warp each
 @pytest.mark.parametrize("k,bits,signed", [(1, 4, True), (2, 4, True), (3, 2, True), (9, 4, False), (17, 3, True),
                                            (27, 4, True), (27, 2, True), (28, 8, True), (32, 4, True), (31, 4, False)])
 def test_very_short_rows_thread_per_row_path(gpu, k, bits, signed):
@@ -384,7 +384,7 @@ def test_very_short_rows_thread_per_row_path(gpu, k, bits, signed):
 
 def test_non_finite_and_zero_rows_on_every_launch_path(gpu):
     """NaN / Inf / all-zero / denormal rows never fault and never disturb their neighbours, whichever path
-    (long regrouped rows, batched short rows, thread-per-row) the launch takes."""
+    (long rows, short rows by several lanes or by one) the launch takes."""
     for s, k in [(12, 3000), (2600, 256), (9700, 27)]:
         w = synth.laplace(s * k, 0.02, seed=950 + k).reshape(s, k).copy()
         w[1] = 0.0

@@ -249,7 +249,7 @@ def test_launch_counter_counts_one_launch_per_row_path():
     x = torch.from_numpy(synth.relu_activations(100_000, seed=3)).cuda()
     a, e = torch.empty(1, device="cuda"), torch.empty(1, device="cuda")
     ctx.omse_activation_scale(x, x.numel(), 4, False, 2048, 1.0, 3, a, e)
-    assert ctx.omse_read_launches() == 11          # init, maxima, two sweeps, curve, argmin, re-score, 3 polish steps, final
+    assert ctx.omse_read_launches() == 11          # init, maxima, histogram, scan, levels, argmin, re-score, 3 polish steps, final
     torch.cuda.synchronize()
 
 
