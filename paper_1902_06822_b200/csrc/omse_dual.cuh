@@ -103,7 +103,8 @@ __global__ void __launch_bounds__(kDualThreads) dual_kernel(const DualArgs a) {
                 else bad = true;
             }
             if (bad) st |= 1u;
-            block_max(mx, scratch);
+            float dummy = 0.f;
+            block_max2(mx, dummy, scratch);
             const float m = mx;
             float a1_last, a2_last;
             dual_scales(m, a, a.n_cand1 - 1, a.n_cand2 - 1, a1_last, a2_last);

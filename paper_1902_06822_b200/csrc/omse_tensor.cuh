@@ -65,7 +65,7 @@ struct TensorArgs {
     double* chunks;         // [n_chunks][3] sums of the chunks of a window
     int n_chunks;
     double* block_sums;     // [grid][kBlockSums]: sum x^2, number and excess of the values above the bins, the same for the coarse
-                            // ones, sum of the bins of the values next to an edge
+                            // ones, sum of the bins of the values next to an edge (the bits of an integer)
     int n_blocks;           // blocks of the histogram launch
     double* levels;         // [2][n_cand] <x,q>/h and <q,q>
     double* partials;       // passes: [blocks][listed candidates] doubles + [blocks] int64
@@ -466,7 +466,7 @@ __global__ void __launch_bounds__(kHistThreads, 2) tensor_hist_kernel(const Tens
             long long near = j == 0 ? s.near : 0ll;
             block_sum2(v[j], near, dscratch);
             if (tid == 0) a.block_sums[kBlockSums * blockIdx.x + j] = v[j];
-            if (tid == 0 && j == 0) a.block_sums[kBlockSums * blockIdx.x + 5] = (double)near;
+            if (tid == 0 && j == 0) a.block_sums[kBlockSums * blockIdx.x + 5] = __longlong_as_double(near);
         }
     }
 }
@@ -596,17 +596,22 @@ __global__ void __launch_bounds__(256) tensor_levels_kernel(const TensorArgs a) 
 // What the histogram's blocks left beside the bins, by one block: sum x^2, the sum of the values next to an edge, the state of the
 // scan above the topmost window, N and P of the coarse bins.
 __device__ __forceinline__ void tensor_scan_begin(const TensorArgs& a, double unit, double (*part)[3], double* scratch) {
-    double t[kBlockSums];
+    double t[kBlockSums - 1];
+    long long near = 0;
 #pragma unroll
-    for (int j = 0; j < kBlockSums; ++j) {                 // the blocks' sums, in a fixed order
-        long long zero = 0;
+    for (int j = 0; j < kBlockSums - 1; ++j) {             // the blocks' sums, in a fixed order
         t[j] = 0.0;
-        for (int b = threadIdx.x; b < a.n_blocks; b += kScanThreads) t[j] += __ldcg(a.block_sums + kBlockSums * b + j);
-        if (j == 0 || j == 5 || a.clipped) block_sum2(t[j], zero, scratch);
+        for (int b = threadIdx.x; b < a.n_blocks; b += kScanThreads) {
+            t[j] += __ldcg(a.block_sums + kBlockSums * b + j);
+            if (j == 0) near += __double_as_longlong(__ldcg(a.block_sums + kBlockSums * b + 5));
+        }
+        long long zero = 0;
+        if (j == 0) block_sum2(t[0], near, scratch);
+        else if (a.clipped) block_sum2(t[j], zero, scratch);
     }
     if (threadIdx.x == 0) {
         a.st->sum_sq = t[0];
-        a.st->near = t[5];
+        a.st->near = (double)near;
         a.st->scan[a.which] = TensorState::Scan{a.clipped ? t[1] : 0.0, a.clipped ? t[2] : 0.0, 0.0, a.n_bins};
     }
     if (a.n_bins2 > 0) {
