@@ -25,6 +25,8 @@ constexpr size_t kSmSmem = 233472;            // shared memory of an SM, and wha
 constexpr size_t kBlockSmem = 1024 + 1232;    // 1 KB for the system, static
 constexpr int kMaxSmem = 229376;              // dynamic shared memory per block: the 227 KB opt-in limit of sm_100 less 3 KB for static use
 
+constexpr int kNearValues = 1 << 18;          // (51M values less their minimum, 2048 candidates: some 70,000 next to an edge of a bin)
+
 struct Workspace {
     unsigned int status;
     unsigned int pad_[3];
@@ -34,6 +36,7 @@ struct Workspace {
     omse::TensorState tstate;
     double curve[OMSE_MAX_CANDIDATES];
     int list[OMSE_MAX_CANDIDATES];  // candidates of the per-tensor search that are re-scored in fp64
+    float near[kNearValues];        // its values next to an edge of a bin
     omse::ResidentExchange exchange;
 };
 
@@ -293,7 +296,7 @@ int launch_hist(const TensorEnv& env, const omse::TensorArgs& a, bool full, int*
     const size_t smem = (size_t)a.shared_win * 20 + 8 * omse::kHotWords + (size_t)a.n_bins2 * 12;
     if (!env.seen->attr_hist) {
         for (const auto k : kernels)
-            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess) return OMSE_ECUDA;
+            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem - 4096) != cudaSuccess) return OMSE_ECUDA;   // (static: 4.6 KB)
         env.seen->attr_hist = true;
     }
     const int id = (full ? 2 : 0) + (a.lo < 0 ? 1 : 0);
@@ -333,6 +336,7 @@ int enqueue_tensor_search(const TensorEnv& env, omse::TensorArgs& a, int refine_
     cudaStream_t s = env.stream;
     const long long n = a.n;
     tensor_bins(a);
+    a.refine_iters = refine_iters;
     // the workspace until the passes take it over: the blocks' sums, <x,q> and <q,q>, then the histogram and N and P.  The blocks keep
     // up to kHistWindow bins in shared memory, and one block scans them; up to twice as many are two such windows, each with a
     // look at the tensor.  More bins (a grid that ends far below max|x|) are one window too where the workspace holds
@@ -391,7 +395,10 @@ int enqueue_tensor_search(const TensorEnv& env, omse::TensorArgs& a, int refine_
     omse::tensor_finish_kernel<<<1, 1024, 0, s>>>(a);
     omse::tensor_pass_kernel<0><<<(unsigned)pass_grid<0>(env, n), 256, 0, s>>>(a);
     const int g1 = pass_grid<1>(env, n);
-    for (int it = 0; it < refine_iters; ++it) omse::tensor_pass_kernel<1><<<(unsigned)g1, 256, 0, s>>>(a);
+    for (int it = 0; it < refine_iters; ++it) {
+        a.first_pass = it == 0 ? 1 : 0;
+        omse::tensor_pass_kernel<1><<<(unsigned)g1, 256, 0, s>>>(a);
+    }
     omse::tensor_pass_kernel<2><<<(unsigned)pass_grid<2>(env, n), 256, 0, s>>>(a);
     *env.launches += 3 + (unsigned long long)refine_iters;   // argmin, re-score, polish steps, final
     return cudaGetLastError() == cudaSuccess ? OMSE_OK : OMSE_ECUDA;
@@ -1111,6 +1118,8 @@ static int activation_impl(omse_ctx* ctx, const float* d_x, int64_t n, int bits,
     a.partials = ctx->partials;
     a.partial_doubles = (long long)(kPartialBytes / 8);
     a.list = ctx->ws->list;
+    a.near = ctx->ws->near;
+    a.near_cap = kNearValues;
     a.curve = ctx->ws->curve;
     a.curve_out = d_sse_curve;
     a.alpha_out = d_alpha;
@@ -1154,6 +1163,7 @@ int omse_pack_int4(omse_ctx* ctx, const int8_t* d_codes, int64_t n, int is_signe
 namespace {
 
 constexpr size_t kStaticPartialDoubles = 1u << 19;   // 4 MiB of per-block partial sums
+constexpr int kStaticNear = 1024;                    // values next to an edge of a bin; more, and the polish starts with a look at the tensor
 
 struct StaticScratch {
     unsigned int status;
@@ -1161,6 +1171,7 @@ struct StaticScratch {
     omse::TensorState tstate;
     double curve[OMSE_STATIC_MAX_CANDIDATES];
     int list[OMSE_STATIC_MAX_CANDIDATES];
+    float near[kStaticNear];
     double partials[kStaticPartialDoubles];
 };
 static_assert(sizeof(StaticScratch) <= OMSE_STATIC_SCRATCH_BYTES, "static scratch larger than documented");
@@ -1225,6 +1236,8 @@ extern "C" int omse_activation_scale_static(int device, void* cuda_stream, const
     a.partials = sc->partials;
     a.partial_doubles = (long long)kStaticPartialDoubles;
     a.list = sc->list;
+    a.near = sc->near;
+    a.near_cap = kStaticNear;
     a.curve = sc->curve;
     a.curve_out = d_sse_curve;
     a.alpha_out = d_alpha;

@@ -13,9 +13,11 @@
 //   to re-score -> re-score -> polish x R -> final error.
 // Grid-wide sums there use "the last block to arrive reduces" (a ticket from atomicAdd, no waiting).
 // Measured on one B200 against a sweep of the candidates over the values each does not code as 0: 51,380,224 post-ReLU
-// values with 2048 candidates 655 -> 364 us, 25,088 with 50 candidates 53 -> 21 us, 1,605,633 values of both signs with
-// offset and 500 candidates 229 -> 50 us.
+// values with 2048 candidates 655 -> 322 us, 25,088 with 50 candidates 53 -> 19 us, 1,605,633 values of both signs with
+// offset and 500 candidates 229 -> 33 us.
 #pragma once
+#include <type_traits>
+
 #include "omse_lattice.cuh"
 
 namespace omse {
@@ -34,6 +36,8 @@ struct TensorState {          // lives in the context workspace
     float alpha;
     float step;
     int n_list;                      // candidates to re-score in fp64 (0: the winner of the curve needs none)
+    unsigned int n_near;             // values next to an edge of a bin, listed (more than TensorArgs::near_cap: not all of them)
+    int first_done;                  // the first polish step came out of the histogram
     int polish_done;                 // set when a polish step stops or reaches a fixed point: later steps return at once
     int key_min, key_max;                // offset mode: order-preserving integer keys of min and max of the tensor
     float delta;                         // offset subtracted from every element (0 without offset)
@@ -71,6 +75,10 @@ struct TensorArgs {
     double* partials;       // passes: [blocks][listed candidates] doubles + [blocks] int64
     long long partial_doubles;   // capacity of `partials`
     int* list;              // [n_cand] candidates to re-score (workspace)
+    float* near;            // [near_cap] values next to an edge of a bin, less the offset and times HistGeometry::pre (workspace)
+    int near_cap;
+    int refine_iters;
+    int first_pass;         // polish pass 0, which the histogram may have made unnecessary
     double* curve;          // [n_cand] error per candidate (workspace)
     double* curve_out;      // user copy, nullable
     float* alpha_out;
@@ -91,6 +99,8 @@ __device__ __forceinline__ void tensor_state_init(TensorState* st) {
     st->alpha = 0.f;
     st->step = 0.f;
     st->n_list = 0;
+    st->n_near = 0u;
+    st->first_done = 0;
     st->polish_done = 0;
     st->key_min = 0x7fffffff;
     st->key_max = (int)0x80000000;
@@ -246,8 +256,32 @@ struct HistSums {
     long long near;
 };
 constexpr int kBlockSums = 6;
+// Values next to an edge of a bin, on their way to the list of the tensor.  The count is looked at before it is added to: a tensor
+// whose values all lie on edges would queue for it.
+template <unsigned int CAP>
+struct NearList {
+    unsigned int n;
+    float v[CAP];
+    __device__ __forceinline__ void add(float x) {
+        if (*(volatile unsigned int*)&n > CAP) return;
+        const unsigned int at = atomicAdd(&n, 1u);
+        if (at < CAP) v[at] = x;
+    }
+    // the block's values to the tensor's list, by all threads, between barriers
+    __device__ __forceinline__ void flush(unsigned int* n_all, float* all, unsigned int cap, unsigned int& s_at) {
+        const unsigned int mine = n;
+        if (mine == 0u) return;                             // (the same in all threads)
+        if (threadIdx.x == 0) s_at = atomicAdd(n_all, mine > CAP ? cap + 1u : mine);
+        __syncthreads();
+        const unsigned int at = s_at;
+        if (mine <= CAP && at <= cap && mine <= cap - at)
+            for (unsigned int i = threadIdx.x; i < mine; i += blockDim.x) all[at + i] = v[i];
+    }
+};
 // Words of a block's histograms.
+constexpr unsigned int kHistNear = 1024;
 struct HistWords {
+    NearList<kHistNear>* near;
     unsigned int *w1, *w2;            // fine window, hot copies first (two-word form)
     unsigned int *c2, *lo2, *hi2;     // coarse histogram (three-word form)
 };
@@ -292,6 +326,7 @@ __device__ __forceinline__ void hist_insert4(const float (&x)[4], const HistGeom
             int m = magic_int(u[j]), k = (int)r[j];
             if (m >= 1 && hist_near(k, m)) {
                 s.near += m;
+                w.near->add(x[j]);
                 hist_correct(k, m, g.hk);
                 u[j] = kMagic + (float)m;
                 r[j] = (float)k;
@@ -351,10 +386,14 @@ template <bool FULL, bool SIGNED>
 __global__ void __launch_bounds__(kHistThreads, 2) tensor_hist_kernel(const TensorArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double dscratch[64];
+    __shared__ NearList<kHistNear> s_near;
+    __shared__ unsigned int s_near_at;
     TensorState* st = a.st;
     const int tid = threadIdx.x, swin = a.shared_win, words = kHotWords + swin;         // swin is a multiple of 4
     unsigned long long* acc_f = reinterpret_cast<unsigned long long*>(smem_raw);       // [swin]
     HistWords w;
+    w.near = &s_near;
+    if (tid == 0) s_near.n = FULL ? 0u : kHistNear + 1u;           // (not listed by windows)
     w.w1 = reinterpret_cast<unsigned int*>(acc_f + swin);
     w.w2 = w.w1 + words;
     w.c2 = w.w2 + words;
@@ -457,6 +496,7 @@ __global__ void __launch_bounds__(kHistThreads, 2) tensor_hist_kernel(const Tens
                     atomicAdd(a.hist + 2 * a.win + a.n_bins2 + b, ((unsigned long long)w.hi2[b] << 16) + w.lo2[b]);
                 }
         s.sq *= 1.0 / ((double)g.pre * (double)g.pre);
+        if (first) s_near.flush(&st->n_near, a.near, (unsigned)a.near_cap, s_near_at);
         if (blockIdx.x == 0 && tid == 0 && a.evals && first) atomicAdd(a.evals, (unsigned long long)a.n);
     }
     if (a.first_window) {
@@ -474,37 +514,52 @@ __global__ void __launch_bounds__(kHistThreads, 2) tensor_hist_kernel(const Tens
 // Suffix scan of bins 0 .. n-1 of (count, fractional sum) by a block of kScanThreads threads: above_n[i] = N, above_p[i] = P at
 // the position of bin i, in units of h.  (cn, cs, cf): the state N, S, F at the position `gap` bins above bin 0, replaced by
 // the state at bin 0's position.  `unit` turns fractional sums into units of h.  part: exchange words.
+constexpr int kScanHeld = 8;
 __device__ __forceinline__ void tensor_scan(const unsigned long long* hn, const unsigned long long* hf, int n, double unit,
                                             double& cn, double& cs, double& cf, double gap, double* above_n, double* above_p,
                                             double (*part)[3]) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int run = (n + kScanThreads - 1) / kScanThreads, first = tid * run;
-    double pn = 0.0, ps = 0.0, pf = 0.0;
-    for (int i0 = (run - 1) & ~7; i0 >= 0; i0 -= 8) {       // eight bins' loads in flight
-        unsigned long long c[8], f[8];
+    // Runs of up to kScanHeld bins are loaded once and stay in registers (4096 bins; a second trip to L2 is 1500 cycles).
+    double hc[kScanHeld], hf8[kScanHeld];
+    auto load = [&](int i0) {                               // eight bins' loads in flight
+        unsigned long long c[kScanHeld], f[kScanHeld];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < kScanHeld; ++j) {
             const bool in = i0 + j < run && first + i0 + j < n;
             c[j] = in ? __ldcg(hn + first + i0 + j) : 0ull;
             f[j] = in ? __ldcg(hf + first + i0 + j) : 0ull;
         }
 #pragma unroll
-        for (int j = 7; j >= 0; --j) {
-            if (i0 + j < run) ps += pn;
-            pn += (double)c[j];
-            pf += (double)f[j];
+        for (int j = 0; j < kScanHeld; ++j) {
+            hc[j] = (double)c[j];
+            hf8[j] = (double)f[j];
         }
-    }
+    };
+    double pn = 0.0, ps = 0.0, pf = 0.0;
+    for (int i0 = (run - 1) & ~(kScanHeld - 1); i0 >= 0; i0 -= kScanHeld) {
+        load(i0);
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const double n2 = __shfl_down_sync(0xffffffffu, pn, o), s2 = __shfl_down_sync(0xffffffffu, ps, o),
-                     f2 = __shfl_down_sync(0xffffffffu, pf, o);
-        if (lane + o < 32) {
-            ps += s2 + (double)(o * run) * n2;
-            pn += n2;
-            pf += f2;
+        for (int j = kScanHeld - 1; j >= 0; --j) {
+            if (i0 + j < run) ps += pn;
+            pn += hc[j];
+            pf += hf8[j];
         }
     }
+    // suffix sums over the lanes' runs, then over the warps' (each warp for itself)
+    auto suffix = [](double& vn, double& vs, double& vf, int l, int items, int width) {
+#pragma unroll
+        for (int o = 1; o < items; o <<= 1) {
+            const double n2 = __shfl_down_sync(0xffffffffu, vn, o), s2 = __shfl_down_sync(0xffffffffu, vs, o),
+                         f2 = __shfl_down_sync(0xffffffffu, vf, o);
+            if (l + o < items) {
+                vs += s2 + (double)(o * width) * n2;
+                vn += n2;
+                vf += f2;
+            }
+        }
+    };
+    suffix(pn, ps, pf, lane, 32, run);
     __syncthreads();                                        // exchange words free
     if (lane == 0) {
         part[warp][0] = pn;
@@ -514,36 +569,33 @@ __device__ __forceinline__ void tensor_scan(const unsigned long long* hn, const 
     double xn = __shfl_down_sync(0xffffffffu, pn, 1), xs = __shfl_down_sync(0xffffffffu, ps, 1), xf = __shfl_down_sync(0xffffffffu, pf, 1);
     if (lane == 31) xn = xs = xf = 0.0;
     __syncthreads();
-    // the state moved to the end of the last thread's run (a sum of T - position is linear in the position)
-    double an = cn, as = cs - ((double)run * kScanThreads - gap) * cn, af = cf, mn = 0.0, ms = 0.0, mf = 0.0;
-    for (int w = kScanThreads / 32 - 1; w >= 0; --w) {
-        if (w == warp) {
-            mn = an;
-            ms = as;
-            mf = af;
-        }
-        as += part[w][1] + (double)(32 * run) * an;
-        an += part[w][0];
-        af += part[w][2];
+    constexpr int nwarp = kScanThreads / 32;
+    double wn = 0.0, ws = 0.0, wf = 0.0;
+    if (lane < nwarp) {
+        wn = part[lane][0];
+        ws = part[lane][1];
+        wf = part[lane][2];
     }
-    cn = an;
-    cs = as;
-    cf = af;
+    suffix(wn, ws, wf, lane, nwarp, 32 * run);
+    // the state above moved to the end of this warp's last run, and to bin 0 (a sum of T - position is linear in the position)
+    const int behind = (warp + 1) & 31;                     // (lane 16 and above hold zeros)
+    double mn = __shfl_sync(0xffffffffu, wn, behind), ms = __shfl_sync(0xffffffffu, ws, behind), mf = __shfl_sync(0xffffffffu, wf, behind);
+    if (warp == nwarp - 1) mn = ms = mf = 0.0;
+    ms += cs + ((double)(nwarp - 1 - warp) * (32 * run) - ((double)run * kScanThreads - gap)) * cn;
+    mn += cn;
+    mf += cf;
+    cs += __shfl_sync(0xffffffffu, ws, 0) + gap * cn;
+    cn += __shfl_sync(0xffffffffu, wn, 0);
+    cf += __shfl_sync(0xffffffffu, wf, 0);
     double dn = xn + mn, ds = xs + ms + (double)((31 - lane) * run) * mn, df = xf + mf;
-    for (int i0 = (run - 1) & ~7; i0 >= 0; i0 -= 8) {
-        unsigned long long c[8], f[8];
+    for (int i0 = (run - 1) & ~(kScanHeld - 1); i0 >= 0; i0 -= kScanHeld) {
+        if (run > kScanHeld) load(i0);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const bool in = i0 + j < run && first + i0 + j < n;
-            c[j] = in ? __ldcg(hn + first + i0 + j) : 0ull;
-            f[j] = in ? __ldcg(hf + first + i0 + j) : 0ull;
-        }
-#pragma unroll
-        for (int j = 7; j >= 0; --j) {
+        for (int j = kScanHeld - 1; j >= 0; --j) {
             if (i0 + j >= run) continue;
             ds += dn;
-            dn += (double)c[j];
-            df += (double)f[j];
+            dn += hc[j];
+            df += hf8[j];
             if (first + i0 + j < n) {
                 above_n[first + i0 + j] = dn;
                 above_p[first + i0 + j] = fma(df, unit, ds);
@@ -555,13 +607,14 @@ __device__ __forceinline__ void tensor_scan(const unsigned long long* hn, const 
 // <x,q>/h and <q,q> of candidate c from the window [base, base+win) of N and P, shared by `stride` threads.
 __device__ __forceinline__ void tensor_levels(const double* above_n, const double* above_p, int base, int top, int a1, int levels,
                                               int first, int stride, double& sx, double& sq) {
-    int j = (base + a1) / (2 * a1) + first;                 // (2j+1)*a1 > base
-    for (; j < levels; j += stride) {
-        const long long m = (long long)(2 * j + 1) * a1;
-        if (m > top) break;
+    int j = base > 0 ? (base + a1) / (2 * a1) + first : first;      // (2j+1)*a1 > base
+    const int end = min(levels, (top / a1 + 1) >> 1);               // (2j+1)*a1 <= top
+#pragma unroll 4
+    for (; j < end; j += stride) {
+        const int m = (2 * j + 1) * a1;                     // (below 2^21)
         const double nn = above_n[m - 1 - base];
-        sx += above_p[m - 1 - base] + (double)m * nn;
-        sq += (double)(2 * j + 1) * nn;
+        sx += fma((double)m, nn, above_p[m - 1 - base]);
+        sq = fma((double)(2 * j + 1), nn, sq);
     }
 }
 // Eight threads per candidate; i: this thread among all of them.  Later windows add to what earlier ones left.
@@ -719,6 +772,45 @@ __device__ __forceinline__ double tensor_band(double bv, double sum_sq) {
     return bv * (1.0 + kRescoreBand) + 1e-13 * sum_sq;
 }
 
+// The first polish step, alpha <- <x,q>/<q,q> at candidate c, needs no look at the tensor: at a scale of the grid the thresholds are
+// edges of bins, and <x,q>, <q,q> are the sums that the curve was made of, exact integers but for a last rounding in binary64.  Only
+// the values next to an edge may be coded differently by the IEEE quotient; they are listed, and here is what such a value
+// changes.  (51,380,224 values: a step less is 47 us of 366; 1,605,633 in one kernel: an exchange and a pass, 4 us of 37.)  y: the value times HistGeometry::pre; hi, d: levels and spacing of the extra negative level as in HistGeometry.
+__device__ __forceinline__ void near_correction(float y, const HistGeometry& g, int c, int hi, float alpha, float inv, float flo, float fhi, float thr,
+                                                double& dx, long long& dq) {
+    const float s = y * g.scale, v = g.sgn ? fabsf(s) : s, u = __fmaf_rd(v, g.inv_up, kMagic);
+    int m = magic_int(u), k = __float2int_rz(fmaf(-(u - kMagic), g.h, v));
+    if (hist_near(k, m)) hist_correct(k, m, g.hk);
+    int counted = min(hi, (min(m, g.n_bins) / (c + 1) + 1) >> 1);
+    if (y < 0.f && g.d > 0 && min(m / g.d, g.n_bins2) >= c + 1) ++counted;
+    const float x = y * __fdiv_rn(1.0f, g.pre);
+    const int coded = abs(exact_code(x, alpha, inv, flo, fhi, thr));
+    dx += (double)fabsf(x) * (double)(coded - counted);
+    dq += coded * coded - counted * counted;
+}
+// The step by one block at candidate c (same in all threads): sx, sq are <x,q>/h and <q,q> there as the bins have it.
+__device__ __forceinline__ void tensor_first_step(const TensorArgs& a, float step, int c, double* scratch) {
+    TensorState* st = a.st;
+    const unsigned int n_near = __ldcg(&st->n_near);
+    if (a.refine_iters < 1 || n_near > (unsigned)a.near_cap) return;
+    const HistGeometry g = hist_geometry(step, a);
+    const float alpha = __fmul_rn((float)(c + 1), step), inv = __fdiv_rn(1.0f, alpha), flo = (float)a.lo, fhi = (float)a.hi,
+                thr = ambiguity_threshold(flo, fhi);
+    double dx = 0.0;
+    long long dq = 0;
+    for (unsigned int i = threadIdx.x; i < n_near; i += blockDim.x)
+        near_correction(__ldcg(a.near + i), g, c, a.hi, alpha, inv, flo, fhi, thr, dx, dq);
+    block_sum2(dx, dq, scratch);
+    if (threadIdx.x == 0) {
+        const double sxq = fma(0.5 * (double)step, __ldcg(a.levels + c), dx);
+        const long long sqq = (long long)__ldcg(a.levels + a.n_cand + c) + dq;
+        const float a_new = sqq != 0 ? (float)(sxq / (double)sqq) : 0.f;
+        if (a_new >= FLT_MIN && a_new <= FLT_MAX && a_new != alpha) st->alpha = a_new;
+        else st->polish_done = 1;                           // as a polish pass would
+        st->first_done = 1;
+    }
+}
+
 // One block: the curve, its minimum and the list of candidates to re-score.
 __global__ void __launch_bounds__(1024) tensor_finish_kernel(const TensorArgs a) {
     __shared__ double scratch[64];
@@ -763,6 +855,7 @@ __global__ void __launch_bounds__(1024) tensor_finish_kernel(const TensorArgs a)
         st->alpha = __fmul_rn((float)(bi + 1), g.step);
         st->n_list = cnt > 1 || bv < tiny ? cnt : 0;   // a single candidate in the band needs no re-scoring
     }
+    if (!(cnt > 1 || bv < tiny)) tensor_first_step(a, g.step, bi, scratch);
 }
 
 // Grid-wide pass over the tensor; sums in fp64, codes equal to those of the IEEE division (see magic_code).
@@ -783,13 +876,14 @@ __global__ void __launch_bounds__(256) tensor_pass_kernel(const TensorArgs a) {
     if (MODE == 0 && n_list == 0) return;
     const float alpha_now = st->alpha;
     const float delta = st->delta;
-    if (MODE == 1 && (!(alpha_now > 0.f) || st->polish_done)) return;
+    if (MODE == 1 && (!(alpha_now > 0.f) || st->polish_done || (a.first_pass && st->first_done))) return;
     const int slot = MODE == 0 ? ((n_list + 3) & ~3) : 1;                  // doubles per block
-    const long long fit = a.partial_doubles / (slot + 1);
+    double* const room = MODE == 0 ? a.levels + 2 * a.n_cand : a.partials;   // (the first polish step still needs <x,q> and <q,q>)
+    const long long fit = (a.partial_doubles - (room - a.partials)) / (slot + 1);
     const unsigned int nblk = (long long)gridDim.x < fit ? gridDim.x : (unsigned int)fit;
     if (blockIdx.x >= nblk) return;
-    double* part_d = a.partials;                                           // [nblk][slot]
-    long long* part_q = reinterpret_cast<long long*>(a.partials + (size_t)nblk * slot);   // [nblk]
+    double* part_d = room;                                                 // [nblk][slot]
+    long long* part_q = reinterpret_cast<long long*>(room + (size_t)nblk * slot);   // [nblk]
     const long long stride = (long long)nblk * blockDim.x;
     const long long tid0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long n4 = a.n >> 2;
@@ -917,6 +1011,10 @@ __global__ void __launch_bounds__(256) tensor_pass_kernel(const TensorArgs a) {
             if (a.status_out) *a.status_out = *a.status;
         }
     }
+    if (MODE == 0) {
+        __syncthreads();                                    // best_idx and alpha before the step replaces alpha
+        tensor_first_step(a, st->step, best, scratch);
+    }
 }
 
 // -------------------------------------------------------------------------------------------------
@@ -930,16 +1028,19 @@ __global__ void __launch_bounds__(256) tensor_pass_kernel(const TensorArgs a) {
 constexpr int kResidentBlocks = 160;     // blocks the exchange area has room for
 constexpr int kResidentBins = 4096;      // bins of the histogram in the exchange area (and as many coarse ones)
 constexpr int kResidentCands = 1024;
+constexpr int kResidentNear = 512;       // values next to an edge of a bin in the list, a thread's each
 constexpr unsigned int kSpinLimit = 1u << 22;   // polls of a slot before a block gives up (seconds), by default
 
-struct __align__(16) ResidentSlot {      // one block's contribution to an exchange: 64 bits, and 40 bits under a 24-bit tag
-    unsigned long long a, b;
+struct __align__(128) ResidentSlot {     // one block's contribution to an exchange: 64 bits, and 40 bits under a 24-bit tag
+    unsigned long long a, b;             // (a line of its own: see below)
 };
 struct ResidentExchange {                // in the context workspace; all zero between calls
     ResidentSlot slot[2][kResidentBlocks];
     unsigned int ticket;
-    unsigned int pad_[3];
+    unsigned int n_near;                 // as TensorState::n_near
+    unsigned int pad_[2];
     double fin[kResidentBlocks];
+    float near[kResidentNear];
     unsigned long long hist[4 * kResidentBins];
 };
 
@@ -950,15 +1051,22 @@ struct ResidentArgs {
     unsigned int spin_limit;             // polls of a slot before a block gives up
 };
 
-// An exchange between the blocks: every block publishes a slot, data and tag in one 16-byte store, and thread b of every
-// block polls the slot of block b.  No counter that all blocks would have to add to one after the other, no fence between
-// data and flag, and one trip to L2 each way.  Slots alternate between two sets: a block can only be one exchange ahead,
-// since it waits for everybody's slot of this one.  Tags count the exchanges of a call from 1; the last block of a call
-// clears the slots.  Slots are stored and loaded with relaxed order.  Where an exchange stands for more than its slots (DATA: the
-// histogram, the errors of the re-scored candidates), thread 0 fences between the barrier behind which the block's writes lie
-// and its slot, and the polls are acquiring loads, before the barrier that lets the block read (with fences of the polling threads
-// instead 601,676 values and 63 candidates take 28.3 us against 26.5).  A block that does not see a slot within the limit
-// of polls sets s_bad, goes on to the end without further exchanges, and reports it.
+// An exchange between the blocks: every block publishes a slot, data and tag in one 16-byte store, and the first warp of every
+// block polls all of them, up to five slots a lane.  No counter that all blocks would have to add to one after the other, no fence
+// between data and flag, and one trip to L2 each way.  One warp polls and not a thread for each slot, and every slot has a
+// line of L2 to itself: the polls of all blocks queue at the lines that slots share, and the slots of the last blocks to arrive
+// wait behind them (148 blocks that arrive within 0.75 us: 148 threads of each poll 5.4 us, a warp 3.7, a warp and a line per slot
+// 2.2).  The warp has the sums in its lanes, so that a barrier on either side of it is all that the block waits for.  Slots
+// alternate between two sets: a block can only be one exchange ahead, since it waits for everybody's slot of this one.  Tags count
+// the exchanges of a call from 1; the last block of a call clears the slots.  Slots are stored and loaded with relaxed order.  Where
+// an exchange stands for more than its slots (DATA: the histogram, the errors of the re-scored candidates), thread 0 fences between
+// the barrier behind which the block's writes lie and its slot, and the polling warp fences between its polls and the barrier that
+// lets the block read.  A block that does not see a slot within the limit of polls sets s_bad, goes on to the end without further
+// exchanges, and reports it.
+struct ResidentPart {                // shared words of a block's part in an exchange
+    double d[kResidentThreads / 32], d_all;
+    long long q[kResidentThreads / 32], q_all;
+};
 struct ResidentTeam {
     ResidentExchange* ex;
     unsigned int step;               // exchanges so far
@@ -968,54 +1076,119 @@ struct ResidentTeam {
 __device__ __forceinline__ void slot_store(ResidentSlot* p, unsigned long long a, unsigned long long b) {
     asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(p), "l"(a), "l"(b) : "memory");
 }
-template <bool ACQUIRE>
 __device__ __forceinline__ void slot_load(const ResidentSlot* p, unsigned long long& a, unsigned long long& b) {
-    if (ACQUIRE) asm volatile("{\n\t.reg .b128 t;\n\tld.acquire.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}" : "=l"(a), "=l"(b) : "l"(p) : "memory");
-    else asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+    asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}" : "=l"(a), "=l"(b) : "l"(p) : "memory");
 }
 __device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
-// publishes (thread 0 of the block, after a barrier)
-template <bool DATA>
-__device__ __forceinline__ void resident_publish(ResidentTeam& t, unsigned long long a, unsigned long long b40) {
-    ++t.step;
-    if (threadIdx.x == 0) {
+// The first warp publishes the block's slot (a, b40: the same in all lanes, known after a barrier) and polls; use(a, b40) is called
+// for every block's slot, the slots lane, lane + 32, ... by a lane in increasing order.
+template <bool DATA, class F>
+__device__ __forceinline__ void resident_gather(const ResidentTeam& t, unsigned long long a, unsigned long long b40, F use) {
+    const int lane = threadIdx.x & 31, nblk = gridDim.x;
+    ResidentSlot* set = t.ex->slot[t.step & 1];
+    if (lane == 0) {
         if (DATA) fence_gpu();
-        slot_store(&t.ex->slot[t.step & 1][blockIdx.x], a, ((unsigned long long)t.step << 40) | b40);
+        slot_store(set + blockIdx.x, a, ((unsigned long long)t.step << 40) | b40);
     }
-}
-// thread b < gridDim.x gets block b's slot; others get `none`.  A barrier has to follow before the block reads what came with them.
-template <bool DATA>
-__device__ __forceinline__ void resident_collect(ResidentTeam& t, unsigned long long& a, unsigned long long& b40,
-                                                 unsigned long long none_a) {
-    a = none_a;
-    b40 = 0ull;
-    if (threadIdx.x < gridDim.x) {
-        const ResidentSlot* p = &t.ex->slot[t.step & 1][threadIdx.x];
-        unsigned long long va = 0ull, vb = 0ull;
-        bool there = false;
-        for (unsigned int polls = 0u; !there && polls < t.spin_limit; ++polls) {
-            slot_load<DATA>(p, va, vb);
-            there = (unsigned int)(vb >> 40) == t.step;
-        }
-        if (there) {
-            a = va;
-            b40 = vb & 0xffffffffffull;
-        } else {
-            *t.s_bad = 1;
-        }
+    constexpr int per = (kResidentBlocks + 31) / 32;
+    unsigned long long va[per], vb[per];
+    unsigned int open = 0u;
+#pragma unroll
+    for (int j = 0; j < per; ++j) {
+        va[j] = vb[j] = 0ull;
+        if (lane + 32 * j < nblk) open |= 1u << j;
     }
+    for (unsigned int polls = 0u; open && polls < t.spin_limit; ++polls) {
+#pragma unroll
+        for (int j = 0; j < per; ++j)
+            if (open >> j & 1u) slot_load(set + lane + 32 * j, va[j], vb[j]);
+#pragma unroll
+        for (int j = 0; j < per; ++j)
+            if ((unsigned int)(vb[j] >> 40) == t.step) open &= ~(1u << j);
+    }
+    if (open) *t.s_bad = 1;
+    if (DATA) fence_gpu();
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < per; ++j)
+        if ((unsigned int)(vb[j] >> 40) == t.step) use(va[j], vb[j] & 0xffffffffffull);
 }
 // Sum of a double and of a non-negative integer below 2^40 over all threads of all blocks, in a fixed order; every thread
-// gets it.  False: see above.
+// gets it.  False: see above.  The words of `part` are for this function and resident_extremes() alone: their barriers order its uses.
 template <bool DATA>
-__device__ __forceinline__ bool resident_sum(ResidentTeam& t, double& d, long long& q, double* scratch) {
-    block_sum2(d, q, scratch);
-    resident_publish<DATA>(t, (unsigned long long)__double_as_longlong(d), (unsigned long long)q);
-    unsigned long long ua, ub;
-    resident_collect<DATA>(t, ua, ub, 0ull);
-    d = __longlong_as_double((long long)ua);
-    q = (long long)ub;
-    block_sum2(d, q, scratch);
+__device__ __forceinline__ bool resident_sum(ResidentTeam& t, double& d, long long& q, ResidentPart* part) {
+    constexpr int nwarp = kResidentThreads / 32;
+    const int lane = threadIdx.x & 31;
+    d = warp_sum(d);
+    q = warp_sum(q);
+    if (lane == 0) {
+        part->d[threadIdx.x >> 5] = d;
+        part->q[threadIdx.x >> 5] = q;
+    }
+    __syncthreads();
+    ++t.step;
+    if (threadIdx.x < 32) {
+        d = part->d[lane & (nwarp - 1)];
+        q = part->q[lane & (nwarp - 1)];
+#pragma unroll
+        for (int o = 1; o < nwarp; o <<= 1) {      // (all lanes end with the same bits: a + b == b + a)
+            d += __shfl_xor_sync(0xffffffffu, d, o);
+            q += __shfl_xor_sync(0xffffffffu, q, o);
+        }
+        double dt = 0.0;
+        long long qt = 0;
+        resident_gather<DATA>(t, (unsigned long long)__double_as_longlong(d), (unsigned long long)q, [&](unsigned long long va, unsigned long long vb) {
+            dt += __longlong_as_double((long long)va);
+            qt += (long long)vb;
+        });
+        dt = warp_allsum(dt);
+        qt = warp_allsum(qt);
+        if (lane == 0) {
+            part->d_all = dt;
+            part->q_all = qt;
+        }
+    }
+    __syncthreads();
+    d = part->d_all;
+    q = part->q_all;
+    return *t.s_bad == 0;
+}
+// Smallest key, largest key and the union of flags over all threads of all blocks; every thread gets them.
+__device__ __forceinline__ bool resident_extremes(ResidentTeam& t, int& kmin, int& kmax, unsigned int& flags, ResidentPart* part) {
+    constexpr int nwarp = kResidentThreads / 32;
+    const int lane = threadIdx.x & 31;
+    const auto both = [](int hi, int lo) { return (long long)(((unsigned long long)(unsigned)hi << 32) | (unsigned)lo); };
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
+    flags = __reduce_or_sync(0xffffffffu, flags);
+    if (lane == 0) {
+        part->q[threadIdx.x >> 5] = both(kmax, kmin);
+        part->d[threadIdx.x >> 5] = (double)flags;
+    }
+    __syncthreads();
+    ++t.step;
+    if (threadIdx.x < 32) {
+        const long long k = part->q[lane & (nwarp - 1)];
+        kmin = __reduce_min_sync(0xffffffffu, (int)(unsigned)k);
+        kmax = __reduce_max_sync(0xffffffffu, (int)(k >> 32));
+        flags = __reduce_or_sync(0xffffffffu, (unsigned)part->d[lane & (nwarp - 1)]);
+        resident_gather<false>(t, (unsigned long long)both(kmax, kmin), flags, [&](unsigned long long va, unsigned long long vb) {
+            kmin = min(kmin, (int)(unsigned)va);
+            kmax = max(kmax, (int)(unsigned)(va >> 32));
+            flags |= (unsigned)vb;
+        });
+        kmin = __reduce_min_sync(0xffffffffu, kmin);
+        kmax = __reduce_max_sync(0xffffffffu, kmax);
+        flags = __reduce_or_sync(0xffffffffu, flags);
+        if (lane == 0) {
+            part->q_all = both(kmax, kmin);
+            part->d_all = (double)flags;
+        }
+    }
+    __syncthreads();
+    kmin = (int)(unsigned)part->q_all;
+    kmax = (int)(part->q_all >> 32);
+    flags = (unsigned)part->d_all;
     return *t.s_bad == 0;
 }
 
@@ -1023,6 +1196,9 @@ __global__ void __launch_bounds__(kResidentThreads) tensor_resident_kernel(const
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double scratch[64];
     __shared__ double part[32][3];
+    __shared__ ResidentPart exchanged;
+    __shared__ NearList<256> s_near;
+    __shared__ unsigned int s_near_at;
     __shared__ int s_bad, s_last, s_count[33];
     ResidentExchange* ex = r.ex;
     ResidentTeam team = {ex, 0u, &s_bad, r.spin_limit};
@@ -1035,7 +1211,10 @@ __global__ void __launch_bounds__(kResidentThreads) tensor_resident_kernel(const
     double* curve = above2 + 2 * a.n_bins2;
     int* list = reinterpret_cast<int*>(curve + a.n_cand);
     bool ok = true;
-    if (tid == 0) s_bad = 0;
+    if (tid == 0) {
+        s_bad = 0;
+        s_near.n = 0u;
+    }
     // ---- the slice, its extremes
     const float4* x4 = reinterpret_cast<const float4*>(a.x);
     const long long n4 = a.n >> 2, begin = (long long)blockIdx.x * r.slice4;
@@ -1081,34 +1260,7 @@ __global__ void __launch_bounds__(kResidentThreads) tensor_resident_kernel(const
     // ---- extremes of the tensor, in every block
     int kmin = lo <= hi ? float_key(lo) : 0x7fffffff, kmax = lo <= hi ? float_key(hi) : (int)0x80000000;
     unsigned int nonfinite = bad ? 1u : 0u;
-    int* s_key = reinterpret_cast<int*>(scratch);                   // [3][32]
-    auto block_extremes = [&]() {
-        kmin = __reduce_min_sync(0xffffffffu, kmin);
-        kmax = __reduce_max_sync(0xffffffffu, kmax);
-        nonfinite = __reduce_or_sync(0xffffffffu, nonfinite);
-        __syncthreads();
-        if (lane == 0) {
-            s_key[warp] = kmin;
-            s_key[32 + warp] = kmax;
-            s_key[64 + warp] = (int)nonfinite;
-        }
-        __syncthreads();
-        const int l = lane & (kResidentThreads / 32 - 1);
-        kmin = __reduce_min_sync(0xffffffffu, s_key[l]);
-        kmax = __reduce_max_sync(0xffffffffu, s_key[32 + l]);
-        nonfinite = __reduce_or_sync(0xffffffffu, (unsigned)s_key[64 + l]);
-    };
-    block_extremes();
-    {
-        resident_publish<false>(team, ((unsigned long long)(unsigned)kmax << 32) | (unsigned)kmin, nonfinite);
-        unsigned long long ua, ub;
-        resident_collect<false>(team, ua, ub, 0x800000007fffffffull);
-        kmin = (int)(unsigned)ua;
-        kmax = (int)(unsigned)(ua >> 32);
-        nonfinite = (unsigned)ub;
-        block_extremes();
-        ok = s_bad == 0;
-    }
+    ok = resident_extremes(team, kmin, kmax, nonfinite, &exchanged);
     const float vmin = kmin <= kmax ? key_float(kmin) : 0.f, vmax = kmin <= kmax ? key_float(kmax) : 0.f;
     float delta = 0.f, m = fmaxf(fmaxf(vmax, 0.f), fmaxf(-vmin, 0.f));
     if (a.delta_out && kmin <= kmax) {
@@ -1138,6 +1290,7 @@ __global__ void __launch_bounds__(kResidentThreads) tensor_resident_kernel(const
             int ks = __float2int_rz(fmaf(-(u - kMagic), g.h, v));
             if (hist_near(ks, mm)) {
                 near += mm;
+                s_near.add(x * g.pre);
                 hist_correct(ks, mm, g.hk);
                 if (mm < 1) return;
             }
@@ -1178,13 +1331,16 @@ __global__ void __launch_bounds__(kResidentThreads) tensor_resident_kernel(const
             atomicAdd(gh + (coarse ? 2 * kResidentBins : 0) + b, (unsigned long long)c);
             atomicAdd(gh + (coarse ? 3 * kResidentBins : kResidentBins) + b, f);
         }
+        s_near.flush(&ex->n_near, ex->near, kResidentNear, s_near_at);
         // With more than a few values per thread the additions take longer than the block's sums: every thread waits for its own
         // beside them, which leaves thread 0's fence little to wait for (601,676 values 27.5 -> 26.5 us; 11,552 values 15.1 and 16.0)
         if (r.slice4 > kResidentThreads) fence_gpu();
         long long none = 0;
         double sum_sq = sq;
-        ok = resident_sum<true>(team, sum_sq, near, scratch) && ok; // every block's additions are known after this (near < 2^29 per block)
+        ok = resident_sum<true>(team, sum_sq, near, &exchanged) && ok; // every block's additions are known after this (near < 2^29 per block)
         // ---- N, P and the curve, in every block
+        const unsigned int n_near = ok ? __ldcg(&ex->n_near) : kResidentNear + 1u;      // (for the polish; on their way meanwhile)
+        const float near_y = __ldcg(ex->near + tid);
         const double unit = hist_unit(gr.step);
         double cn = 0.0, cs = 0.0, cf = 0.0;
         if (a.n_bins2 > 0) {
@@ -1196,50 +1352,57 @@ __global__ void __launch_bounds__(kResidentThreads) tensor_resident_kernel(const
         __syncthreads();
         double bv = INFINITY;
         int bi = 0x7fffffff;
-        for (int i0 = 0; i0 < 8 * a.n_cand; i0 += kResidentThreads) {
-            const int c = (i0 + tid) >> 3, p = tid & 7;
-            double sx = 0.0, sn = 0.0;
-            if (c < a.n_cand) tensor_levels(above, above + bins, 0, a.n_bins, c + 1, a.hi, p, 8, sx, sn);
-            if (p == 0 && c < a.n_bins2) {
-                const double nn = above2[c], d = (double)g.d;
-                sx += d * (above2[a.n_bins2 + c] + (double)(c + 1) * nn);
-                sn += d * nn;
-            }
+        // The smallest scales have the most levels: a warp for each of 16 candidates, eight threads for each of the next 64, then
+        // a thread (500 candidates on 8 bits 11,600 cycles with eight threads for all of them, 5300 so).
+        auto candidates = [&](auto lanes_tag, int from, int to) {
+            constexpr int lanes = decltype(lanes_tag)::value;
+            for (int c0 = from; c0 < to; c0 += kResidentThreads / lanes) {
+                const int c = c0 + tid / lanes, p = tid & (lanes - 1);
+                double sx = 0.0, sn = 0.0;
+                if (c < to) tensor_levels(above, above + bins, 0, a.n_bins, c + 1, a.hi, p, lanes, sx, sn);
+                if (p == 0 && c < min(to, a.n_bins2)) {
+                    const double nn = above2[c], d = (double)g.d;
+                    sx += d * (above2[a.n_bins2 + c] + (double)(c + 1) * nn);
+                    sn += d * nn;
+                }
 #pragma unroll
-            for (int o = 1; o < 8; o <<= 1) {
-                sx += __shfl_xor_sync(0xffffffffu, sx, o);
-                sn += __shfl_xor_sync(0xffffffffu, sn, o);
-            }
-            if (p == 0 && c < a.n_cand) {
-                const double v = tensor_error(gr.step, c, sum_sq, sx, sn);
-                curve[c] = v;
-                if (a.curve_out && blockIdx.x == 0) a.curve_out[c] = v;
-                if (v < bv) {
-                    bv = v;
-                    bi = c;
+                for (int o = 1; o < lanes; o <<= 1) {
+                    sx += __shfl_xor_sync(0xffffffffu, sx, o);
+                    sn += __shfl_xor_sync(0xffffffffu, sn, o);
+                }
+                if (p == 0 && c < to) {
+                    const double v = tensor_error(gr.step, c, sum_sq, sx, sn);
+                    curve[c] = v;
+                    if (a.curve_out && blockIdx.x == 0) a.curve_out[c] = v;
+                    if (v < bv) {
+                        bv = v;
+                        bi = c;
+                    }
                 }
             }
-        }
-        block_argmin(bv, bi, scratch);
-        __syncthreads();
+        };
+        candidates(std::integral_constant<int, 32>(), 0, min(16, a.n_cand));
+        candidates(std::integral_constant<int, 8>(), 16, min(80, a.n_cand));
+        candidates(std::integral_constant<int, 1>(), 80, a.n_cand);
+        block_argmin_error(bv, bi, scratch);
         best = bi;
         const double near_sum = (double)near, tiny = a.curve_out ? kTinyShare * sum_sq : 0.0;
         const double band = tensor_band(bv + tensor_noise(gr.step, bi, near_sum), sum_sq);
         // ---- candidates to re-score, in increasing order: thread t looks at candidates 2t and 2t+1
+        static_assert(kResidentNear == kResidentThreads, "a listed value per thread");
         static_assert(kResidentCands <= 2 * kResidentThreads, "two candidates per thread");
         auto wanted = [&](int c) { return c < a.n_cand && (curve[c] - tensor_noise(gr.step, c, near_sum) <= band || curve[c] < tiny); };
         const bool in0 = wanted(2 * tid), in1 = wanted(2 * tid + 1);
         const unsigned int b0 = __ballot_sync(0xffffffffu, in0), b1 = __ballot_sync(0xffffffffu, in1), below = (1u << lane) - 1u;
         if (lane == 0) s_count[warp] = __popc(b0) + __popc(b1);
         __syncthreads();
-        int at = __popc(b0 & below) + __popc(b1 & below), n_list = 0;
-        for (int w = 0; w < kResidentThreads / 32; ++w) {
-            if (w < warp) at += s_count[w];
-            n_list += s_count[w];
+        const int listed = s_count[lane & (kResidentThreads / 32 - 1)], n_list = (int)__reduce_add_sync(0xffffffffu, (unsigned)listed) / (1024 / kResidentThreads);
+        if (n_list > 1 || bv < tiny) {
+            int at = __popc(b0 & below) + __popc(b1 & below) + (int)__reduce_add_sync(0xffffffffu, lane < warp ? (unsigned)listed : 0u);
+            if (in0) list[at++] = 2 * tid;
+            if (in1) list[at] = 2 * tid + 1;
+            __syncthreads();
         }
-        if (in0) list[at++] = 2 * tid;
-        if (in1) list[at] = 2 * tid + 1;
-        __syncthreads();
         auto slice_error = [&](float al) -> double {                // squared error of the slice at one scale, exact codes
             const float inv = __fdiv_rn(1.0f, al);
             const double ad = (double)al;
@@ -1267,7 +1430,7 @@ __global__ void __launch_bounds__(kResidentThreads) tensor_resident_kernel(const
             }
             double nothing = 0.0;
             none = 0;
-            ok = resident_sum<true>(team, nothing, none, scratch) && ok;     // (only its waiting is wanted)
+            ok = resident_sum<true>(team, nothing, none, &exchanged) && ok;     // (only its waiting is wanted)
             double best_sse = INFINITY;
             int bc = 0x7fffffff;
             for (int l = warp; l < n_list; l += kResidentThreads / 32) {
@@ -1287,8 +1450,31 @@ __global__ void __launch_bounds__(kResidentThreads) tensor_resident_kernel(const
         }
         if (best == 0x7fffffff) best = -1;
         if (best >= 0) alpha = __fmul_rn((float)(best + 1), gr.step);
-        // ---- polish: alpha <- <x,q>/<q,q>
-        for (int it = 0; ok && best >= 0 && it < refine_iters; ++it) {
+        // ---- polish: alpha <- <x,q>/<q,q>.  The first step from the bins (see tensor_first_step), the others by a look at the slice.
+        int from = 0;
+        if (best >= 0 && refine_iters > 0 && n_near <= kResidentNear) {
+            double sx = 0.0, sn = 0.0, dx = 0.0;
+            long long dq = 0;
+            tensor_levels(above, above + bins, 0, a.n_bins, best + 1, a.hi, lane, 32, sx, sn);
+            sx = warp_allsum(sx);
+            sn = warp_allsum(sn);
+            if (best < a.n_bins2) {
+                const double nn = above2[best], d = (double)g.d;
+                sx += d * (above2[a.n_bins2 + best] + (double)(best + 1) * nn);
+                sn += d * nn;
+            }
+            if (tid < (int)n_near)
+                near_correction(near_y, g, best, a.hi, alpha, __fdiv_rn(1.0f, alpha), flo, fhi, thr, dx, dq);
+            if (__syncthreads_or(dq != 0)) block_sum2(dx, dq, scratch);
+            else dx = 0.0;
+            const double sxq = fma(0.5 * (double)gr.step, sx, dx);
+            const long long sqq = (long long)sn + dq;
+            const float a_new = sqq != 0 ? (float)(sxq / (double)sqq) : 0.f;
+            const bool moved = a_new >= FLT_MIN && a_new <= FLT_MAX && a_new != alpha;
+            if (moved) alpha = a_new;
+            from = moved ? 1 : refine_iters;
+        }
+        for (int it = from; ok && best >= 0 && it < refine_iters; ++it) {
             const float inv = __fdiv_rn(1.0f, alpha);
             double sxq = 0.0;
             long long sqq = 0;
@@ -1309,7 +1495,7 @@ __global__ void __launch_bounds__(kResidentThreads) tensor_resident_kernel(const
             }
             if (tid < tail) one(tailp[tid]);
             sqq += s32;
-            ok = resident_sum<false>(team, sxq, sqq, scratch) && ok;
+            ok = resident_sum<false>(team, sxq, sqq, &exchanged) && ok;
             if (sqq == 0) break;
             const float a_new = (float)(sxq / (double)sqq);
             if (!(a_new >= FLT_MIN) || !(a_new <= FLT_MAX) || a_new == alpha) break;
@@ -1367,8 +1553,11 @@ __global__ void __launch_bounds__(kResidentThreads) tensor_resident_kernel(const
     // the exchange area as the next call expects it
     for (int j = tid; j < bins; j += kResidentThreads) ex->hist[j] = ex->hist[kResidentBins + j] = 0ull;
     for (int j = tid; j < a.n_bins2; j += kResidentThreads) ex->hist[2 * kResidentBins + j] = ex->hist[3 * kResidentBins + j] = 0ull;
-    if (tid < kResidentBlocks) ex->slot[0][tid] = ex->slot[1][tid] = ResidentSlot{0ull, 0ull};
-    if (tid == 0) ex->ticket = 0u;
+    if (tid < kResidentBlocks) {
+        slot_store(&ex->slot[0][tid], 0ull, 0ull);
+        slot_store(&ex->slot[1][tid], 0ull, 0ull);
+    }
+    if (tid == 0) ex->ticket = ex->n_near = 0u;
 }
 
 // Key layers (Section 3.5): MSE of each layer = sum of its kernels' squared errors / elements, compared

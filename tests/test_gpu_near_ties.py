@@ -111,3 +111,29 @@ def test_natural_near_ties_rows_and_per_tensor(gpu, zero_prob, seed, hi_frac):
         assert abs(ref.sse_curve[i1] - ref.sse_curve[ref.best_idx]) <= 1e-6 * ref.sse_curve[ref.best_idx]
         ref = orc.phi(x, 2, True, 4096, hi_frac, 3, start_idx=i1, want_codes=False)
     assert a1 == pytest.approx(ref.alpha, rel=RTOL) and s1 == pytest.approx(ref.sse, rel=RTOL)
+
+
+@pytest.mark.parametrize("n,bits,signed,n_cand,on_edges", [
+    (5, 4, False, 50, 1), (4093, 4, True, 64, 40), (25_088, 8, False, 50, 300), (25_088, 4, True, 500, 2000),
+    (300_001, 8, True, 1024, 400), (300_001, 4, True, 1500, 900), (2_000_003, 4, False, 2000, 5000), (2_000_003, 8, True, 2048, 400_000)])
+def test_first_polish_step_with_values_on_thresholds(gpu, n, bits, signed, n_cand, on_edges):
+    """One polish step from the sums of the histogram: values within a few ulp of the thresholds of the chosen scale are coded by the
+    IEEE quotient, few of them (listed) and more than the lists hold, in one kernel (up to 1024 candidates) and by launches."""
+    x = synth.student_t3(n, seed=n + n_cand)
+    if not signed:
+        x = np.abs(x)
+    rng = np.random.default_rng(n)
+    a0 = np.float32(orc.activation_scale(x, bits, signed, n_cand, 1.0, 0).alpha)
+    top = (1 << (bits - 1)) - 1 if signed else (1 << bits) - 1
+    at = rng.choice(n, on_edges, replace=False)
+    at = at[at != np.argmax(np.abs(x))]
+    edges = ((rng.integers(1, top + 1, at.size) - 0.5) * a0).astype(np.float32)
+    for _ in range(2):                                   # up to two ulp to either side
+        edges = np.nextafter(edges, edges + rng.integers(-1, 2, at.size).astype(np.float32))
+    x[at] = np.where(edges < np.abs(x).max(), edges, x[at]) * (rng.choice([-1, 1], at.size) if signed else 1)
+    for refine in (1, 2):
+        ref = orc.activation_scale(x, bits, signed, n_cand, 1.0, refine)
+        alpha, sse, idx, _ = gpu.activation_scale(x, bits, signed, n_cand, 1.0, refine, want_curve=False)
+        assert idx == ref.best_idx
+        assert np.float32(alpha) == np.float32(ref.alpha)        # binary64 sums in another order: 1e-15 before the last rounding
+        assert sse == pytest.approx(ref.sse, rel=RTOL)
