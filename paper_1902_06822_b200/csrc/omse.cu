@@ -16,8 +16,13 @@
 
 namespace {
 
-constexpr long long kSmallK = 1024;           // rows up to this length are searched in the registers of a warp or of some of its lanes:
-                                              // 40,000 rows of 1000 values 517 us against 843 by blocks
+constexpr long long kSmallK = 1280;           // rows up to this length are searched in the registers of a warp or of some of its lanes:
+                                              // 58,254 rows of 1152 values 754 us against 1097 by blocks
+// Rows by a histogram of their warp, from 4 bits on (fewer leave too many candidates open).  Splits, or blocks beyond kSmallK, and
+// histogram, 67M Laplace values: 1024 candidates on 4 bits, 400 values a row 1034 us and 1005, 512 886 and 782, 1024 829 and 603, 1600
+// 887 and 600, 2304 698 and 538; on 8 bits, 640 values 999 and 991 (Student-t 867 and 975), 800 1211 and 969, 1024 998 and 772, 2304
+// 783 and 563.  Beyond 2304 values the rows leave an SM fewer than twelve warps.
+constexpr long long kHistK4 = 400, kHistK8 = 700, kHistMaxK = 2304;
 constexpr long long kDualBoundK = 256;        // dual search: rows at least this long go by histogram and bounds (16 rows of 256 values 58 us
                                               // against 100 by the sweep, of 128 values 55 by the sweep, whose time is proportional to the length)
 constexpr size_t kPartialBytes = 16u << 20;   // per-block partial sums of the per-tensor search
@@ -27,11 +32,13 @@ constexpr int kMaxSmem = 229376;              // dynamic shared memory per block
 
 constexpr int kNearValues = 1 << 18;          // (51M values less their minimum, 2048 candidates: some 70,000 next to an edge of a bin)
 
+constexpr int kSides = 2;          // side streams of a context
+
 struct Workspace {
     unsigned int status;
     unsigned int pad_[3];
-    unsigned long long ticket[4];   // work-unit dispensers of the row kernels (self-resetting): a pair for launches on the
-                                    // context's stream, a pair for the launch that runs beside them on the side stream
+    unsigned long long ticket[2 + 2 * kSides];      // work-unit dispensers of the row kernels (self-resetting): a pair for launches on
+                                    // the context's stream, a pair for each launch that runs beside them on a side stream
     unsigned long long evals;       // executed evaluations since the last omse_read_evaluations
     omse::TensorState tstate;
     double curve[OMSE_MAX_CANDIDATES];
@@ -54,15 +61,15 @@ struct LaunchShape { int kernel, threads; size_t smem; int occ; };
 struct omse_ctx {
     int device;
     cudaStream_t stream;
-    cudaStream_t side;                 // second launch of a batched call runs here, beside the first (fork and join by events)
-    cudaEvent_t ev_fork, ev_join;
+    cudaStream_t side[kSides];         // launches of a batched call run here, beside the last one (fork and join by events)
+    cudaEvent_t ev_fork, ev_join[kSides];
     int ticket_pair;                   // which dispenser pair the next row launch uses
     int n_sm;
     Workspace* ws;       // device
     double* partials;    // device, kPartialBytes
     omse::RowTensor* d_tensors;   // device, OMSE_MAX_BATCH descriptors of a batched launch
     // per-context launch bookkeeping (a context is used by one host thread at a time, so no lock)
-    bool attr_rows[5], attr_dual[3];   // opt-in shared-memory attribute set, per kernel
+    bool attr_rows[6], attr_dual[3];   // opt-in shared-memory attribute set, per kernel
     LaunchShape seen[16];                           // blocks per SM of the launch shapes met so far
     int n_seen, next_seen;
     TensorLaunches tensor;                          // the same for the per-tensor kernels
@@ -106,7 +113,8 @@ void bounds(int bits, int is_signed, int* lo, int* hi) {
 }
 
 // Kernels of the row searches, by path (how rows are mapped to threads) and by what a launch needs.
-enum RowPath { kPathShort, kPathBlock, kPaths };     // short rows: a warp or some of its lanes per row
+enum RowPath { kPathShort, kPathHist, kPathBlock, kPaths };     // short rows: a warp or some of its lanes per row; a histogram per warp
+static_assert(kPaths - 1 <= kSides, "a side stream for every path but the last");
 
 // Blocks per SM of a launch shape, remembered: the query costs more than a small launch.  0: the query failed, or none fits.
 int blocks_per_sm(omse_ctx* ctx, int id, const void* kernel, int threads, size_t smem) {
@@ -119,13 +127,14 @@ int blocks_per_sm(omse_ctx* ctx, int id, const void* kernel, int threads, size_t
     if (ctx->n_seen < 16) ++ctx->n_seen;
     return occ;
 }
-constexpr int kRowKernels = 5;       // ids of launch shapes: the row kernels, then the dual search's
+constexpr int kRowKernels = 6;       // ids of launch shapes: the row kernels, then the dual search's
 
 int launch_rows_kernel(omse_ctx* ctx, const omse::RowArgs& a, int path, bool ext, int threads, size_t smem) {
     typedef void (*Kernel)(const omse::RowArgs);
     const Kernel kernels[kRowKernels] = {omse::rows_kernel<false, false>, omse::rows_kernel<true, false>, omse::rows_kernel<false, true>,
-                                         omse::rows_short_kernel<false>, omse::rows_short_kernel<true>};
-    const int id = path == kPathShort ? (a.short_direct ? 4 : 3) : ext ? 1 : a.packed_counts ? 2 : 0;
+                                         omse::rows_short_kernel<omse::kBySplits>, omse::rows_short_kernel<omse::kByLanes>,
+                                         omse::rows_short_kernel<omse::kByHistogram>};
+    const int id = path == kPathHist ? 5 : path == kPathShort ? (a.short_direct ? 4 : 3) : ext ? 1 : a.packed_counts ? 2 : 0;
     const Kernel kernel = kernels[id];
     if (!ctx->attr_rows[id]) {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess) return OMSE_ECUDA;
@@ -134,7 +143,7 @@ int launch_rows_kernel(omse_ctx* ctx, const omse::RowArgs& a, int path, bool ext
     const int occ = blocks_per_sm(ctx, id, (const void*)kernel, threads, smem);
     if (occ == 0) return OMSE_ECUDA;
     long long grid = (long long)ctx->n_sm * occ;
-    const long long teams = path == kPathShort ? (a.n_units + threads / 32 - 1) / (threads / 32) : a.n_units;
+    const long long teams = path != kPathBlock ? (a.n_units + threads / 32 - 1) / (threads / 32) : a.n_units;
     if (grid > teams) grid = teams;
     kernel<<<(unsigned)grid, threads, smem, ctx->stream>>>(a);
     ++ctx->n_launches;
@@ -184,7 +193,7 @@ int launch_rows(omse_ctx* ctx, omse::RowArgs& a, long long max_k, int path) {
     if (a.tensors == nullptr) ext = ext || a.one.gate || a.one.prior_alpha;
     else ext = ext || a.ext_tensors;
     const int bins = all_bins(a.n_cand, a.hi_frac);
-    if (path == kPathShort)
+    if (path != kPathBlock)
         return launch_rows_kernel(ctx, a, path, ext, omse::kShortThreads, (size_t)(omse::kShortThreads / 32) * a.short_bytes);
     const size_t fixed = (size_t)(a.keep_x0 ? 2 : 1) * k4 * 16 + omse::kScratchDoubles * 8 + 8 * 4;
     a.direct = -1;
@@ -263,6 +272,16 @@ void fill_tensor(omse::RowTensor& t, const float* w, int64_t S, int64_t K, float
     t.unit_begin = 0;
     t.rows_per_unit = (packed && (K & 1)) ? 2 : 1;
     t.lanes = 5;
+    t.hist_fbits = t.hist_cshift = 0;
+}
+
+// The context's side streams and events, those that exist.
+void release_launches(omse_ctx* ctx) {
+    if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
+    for (int i = 0; i < kSides; ++i) {
+        if (ctx->ev_join[i]) cudaEventDestroy(ctx->ev_join[i]);
+        if (ctx->side[i]) cudaStreamDestroy(ctx->side[i]);
+    }
 }
 
 bool misaligned4(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 3) != 0; }
@@ -498,81 +517,109 @@ int quantize_list(omse_ctx* ctx, std::vector<omse::RowTensor>& list, int bits, i
     int spread = 0;                                             // more lanes per row where the warps do not fill the GPU
     while (spread < 5 && (short_warps << (spread + 1)) <= 16ll * ctx->n_sm) ++spread;
     std::vector<int> path_of(list.size(), kPathBlock);
-    // One launch per row path present in the list (short rows, block per row): each launch
-    // then runs the kernel instantiation that holds only its path.  Longest rows first inside a launch: the dispenser
-    // hands out work in decreasing size and the tail is short.
+    // Rows by a histogram of their warp; beyond kSmallK values where there are a few for every warp of the GPU.
+    a.n_bins = all_bins(a.n_cand, a.hi_frac);
+    a.hist_lb = 4;
+    while (a.hist_lb < 6 && (32 << a.hist_lb) < a.n_bins) ++a.hist_lb;
+    const int hist_words = 32 << a.hist_lb;
+    // (the largest |x|/h, rounded up to a fraction, lies in a bin)
+    const bool hist_fits = plain && a.hi[0] >= 7 && a.n_bins > 0 &&
+                           2.0 * a.n_cand / (double)a.hi_frac * (1.0 + 4e-7) + 1.0 / 64 < (double)hist_words + 1.0;
+    const long long hist_k = a.hi[0] > 15 ? kHistK8 : kHistK4;
+    long long long_rows = 0;
+    for (const auto& t : list)
+        if (t.K > kSmallK && t.K <= kHistMaxK) long_rows += t.S;
+    const bool hist_long = hist_fits && long_rows + short_rows >= 16ll * ctx->n_sm && (short_rows == 0 || !a.short_direct);
+    if (hist_long && short_rows == 0) a.short_direct = 0;
+    // One launch per row path present in the list: each launch then runs the kernel instantiation that holds only its path.
+    // Longest rows first inside a launch: the dispenser hands out work in decreasing size and the tail is short.
     std::stable_sort(list.begin(), list.end(), [](const omse::RowTensor& x, const omse::RowTensor& y) { return x.K > y.K; });
     bool present[kPaths] = {};
-    int rows4 = 0, groups_most = 0, codes_most = 0;
     for (size_t i = 0; i < list.size(); ++i) {
         omse::RowTensor& t = list[i];
-        if (plain && t.K <= short_k) {
+        if (hist_fits && !a.short_direct && t.K >= hist_k && t.K <= (hist_long ? kHistMaxK : short_k)) {
+            // count and fractions of all values in one word, bin and fraction in 23 bits
+            int count = 1, frac = 1;
+            while ((1ll << count) <= t.K) ++count;
+            while (frac < 12 && (t.K << (frac + 1)) <= (1ll << (32 - count)) && ((long long)hist_words << (frac + 1)) <= (1ll << 23)) ++frac;
+            path_of[i] = kPathHist;
+            t.hist_fbits = frac;
+            t.hist_cshift = 32 - count;
+        } else if (plain && t.K <= short_k) {
             path_of[i] = kPathShort;
             t.lanes = a.short_direct ? 5 : omse::short_lanes(t.K);
             for (int s = 0; s < spread && t.lanes < 5 && (4ll << t.lanes) < t.K; ++s) ++t.lanes;
+        }
+        if (path_of[i] != kPathBlock) {
             // several steps of a warp per unit, so that the dispenser is not the limit, where every warp of the GPU still
             // gets a few units; an even number of rows, for the packed nibbles
             const long long groups = 32 >> t.lanes, many = t.S / (groups * 128 * ctx->n_sm);
             t.rows_per_unit = (int)std::max((long long)t.rows_per_unit, groups * (many >= 2 ? std::min(many, 16ll) & ~1ll : 1));
-            rows4 = std::max(rows4, (int)groups * omse::short_stride4((int)((t.K + 3) >> 2), t.lanes));
-            groups_most = std::max(groups_most, (int)groups);
-            codes_most = std::max(codes_most, (int)(groups * t.K));
         }
         present[path_of[i]] = true;
     }
-    a.short_rows4 = rows4;
-    a.short_slots = a.short_direct ? (omse::kMaxCoarse + omse::kHullValues) / 2 : groups_most * omse::short_slots(a.n_cand);
-    a.short_codes = (a.short_rows4 * 16 + a.short_slots * 8 + omse::kShortClose * groups_most * 2 + 15) & ~15;
-    a.short_bytes = (a.short_codes + codes_most + 16 + 15) & ~15;
-    // With both long and short rows in the list, the launch of the short rows goes first, on the side stream (forked
-    // from and joined to the context's stream by events, with its own work dispenser), and the long rows' launch runs
-    // beside it: the blocks of the second fill the SMs as the blocks of the first run out of work, so only one tail
-    // is left.  The two launches touch different tensors.
-    const bool beside = present[kPathShort] && std::count(present, present + kPaths, true) > 1;
-    bool forked = false;
-    size_t desc_used = 0;
-    int rc_all = OMSE_OK;
-    for (int path = 0; path < kPaths && rc_all == OMSE_OK; ++path) {
-        if (!present[path]) continue;
-        std::vector<omse::RowTensor> sub;
-        long long sub_max_k = 0;
+    // The tensors of each path, one after the other; one copy for all descriptors.
+    std::vector<omse::RowTensor> sorted;
+    int first_of[kPaths + 1] = {}, last = 0;
+    for (int path = 0; path < kPaths; ++path) {
+        long long units = 0;
         for (size_t i = 0; i < list.size(); ++i) {
             if (path_of[i] != path) continue;
-            sub.push_back(list[i]);
-            if (list[i].K > sub_max_k) sub_max_k = list[i].K;
+            list[i].unit_begin = units;
+            units += (list[i].S + list[i].rows_per_unit - 1) / list[i].rows_per_unit;
+            sorted.push_back(list[i]);
         }
-        long long units = 0;
-        for (auto& t : sub) {
-            t.unit_begin = units;
-            units += (t.S + t.rows_per_unit - 1) / t.rows_per_unit;
-        }
-        a.n_launch_tensors = (int)sub.size();
-        a.n_units = units;
+        first_of[path + 1] = (int)sorted.size();
+        if (present[path]) last = path;
+    }
+    if (sorted.size() > 1 && cudaMemcpyAsync(ctx->d_tensors, sorted.data(), sizeof(omse::RowTensor) * sorted.size(), cudaMemcpyHostToDevice,
+                                             ctx->stream) != cudaSuccess)
+        return OMSE_ECUDA;
+    // With rows of several paths in the list, the launches of the shorter rows go first, on side streams (forked from and joined to
+    // the context's stream by events, with work dispensers of their own), and the longest rows' launch runs beside them: the blocks
+    // of the next one fill the SMs as the blocks of the first run out of work, so only one tail is left.  The launches touch
+    // different tensors.
+    bool forked[kSides] = {};
+    int rc_all = OMSE_OK;
+    for (int path = 0; path <= last && rc_all == OMSE_OK; ++path) {
+        if (!present[path]) continue;
+        const omse::RowTensor* sub = sorted.data() + first_of[path];
+        a.n_launch_tensors = first_of[path + 1] - first_of[path];
         a.ext_tensors = 0;
-        for (const auto& t : sub) a.ext_tensors |= (t.gate || t.prior_alpha) ? 1 : 0;
-        if (sub.size() == 1) {
-            a.tensors = nullptr;
-            a.one = sub[0];
-        } else {
-            omse::RowTensor* d_sub = ctx->d_tensors + desc_used;
-            if (cudaMemcpyAsync(d_sub, sub.data(), sizeof(omse::RowTensor) * sub.size(), cudaMemcpyHostToDevice,
-                                ctx->stream) != cudaSuccess) {
-                rc_all = OMSE_ECUDA;
-                break;
-            }
-            a.tensors = d_sub;
-            desc_used += sub.size();
+        int rows4 = 0, groups_most = 0, codes_most = 0;
+        long long sub_max_k = 0;
+        for (int i = 0; i < a.n_launch_tensors; ++i) {
+            const omse::RowTensor& t = sub[i];
+            const int groups = 32 >> t.lanes;
+            a.ext_tensors |= (t.gate || t.prior_alpha) ? 1 : 0;
+            sub_max_k = std::max(sub_max_k, t.K);
+            if (path == kPathBlock) continue;
+            rows4 = std::max(rows4, groups * omse::short_stride4((int)((t.K + 3) >> 2), t.lanes));
+            groups_most = std::max(groups_most, groups);
+            codes_most = std::max(codes_most, (int)(groups * t.K));
         }
-        const bool on_side = beside && path == kPathShort;
+        const omse::RowTensor& end = sub[a.n_launch_tensors - 1];
+        a.n_units = end.unit_begin + (end.S + end.rows_per_unit - 1) / end.rows_per_unit;
+        if (path != kPathBlock) {
+            const int by_lanes = (omse::kMaxCoarse + omse::kHullValues) / 2;
+            a.short_rows4 = rows4;
+            a.short_slots = path == kPathHist ? std::max((hist_words + omse::kMaxCoarse) / 2, by_lanes)      // (rows of extreme values go by lanes)
+                            : a.short_direct  ? by_lanes : groups_most * omse::short_slots(a.n_cand);
+            a.short_codes = a.short_rows4 * 16;    // the codes come where the search's stack has been
+            a.short_bytes = (a.short_codes + std::max(a.short_slots * 8 + omse::kShortClose * groups_most * 2, codes_most + 16) + 15) & ~15;
+        }
+        a.tensors = a.n_launch_tensors > 1 ? ctx->d_tensors + first_of[path] : nullptr;
+        a.one = sub[0];
+        const bool on_side = path != last;
         cudaStream_t own = ctx->stream;
         if (on_side) {
-            if (cudaEventRecord(ctx->ev_fork, own) != cudaSuccess || cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0) != cudaSuccess) {
+            if (cudaEventRecord(ctx->ev_fork, own) != cudaSuccess || cudaStreamWaitEvent(ctx->side[path], ctx->ev_fork, 0) != cudaSuccess) {
                 rc_all = OMSE_ECUDA;
                 break;
             }
-            forked = true;
-            ctx->stream = ctx->side;
-            ctx->ticket_pair = 1;
+            forked[path] = true;
+            ctx->stream = ctx->side[path];
+            ctx->ticket_pair = 1 + path;
         }
         rc_all = launch_rows(ctx, a, sub_max_k, path);
         if (on_side) {
@@ -580,10 +627,10 @@ int quantize_list(omse_ctx* ctx, std::vector<omse::RowTensor>& list, int bits, i
             ctx->ticket_pair = 0;
         }
     }
-    if (forked) {   // the side stream always rejoins, also after an error
-        if (cudaEventRecord(ctx->ev_join, ctx->side) != cudaSuccess || cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0) != cudaSuccess)
+    for (int i = 0; i < kSides; ++i)   // a side stream always rejoins, also after an error
+        if (forked[i] && (cudaEventRecord(ctx->ev_join[i], ctx->side[i]) != cudaSuccess ||
+                          cudaStreamWaitEvent(ctx->stream, ctx->ev_join[i], 0) != cudaSuccess))
             rc_all = rc_all == OMSE_OK ? OMSE_ECUDA : rc_all;
-    }
     return rc_all;
 }
 
@@ -634,12 +681,13 @@ int omse_create(omse_ctx** out, int device, void* cuda_stream) {
         cudaGetLastError();
         return OMSE_ENOMEM;
     }
-    if (cudaMemsetAsync(c->ws, 0, sizeof(Workspace), c->stream) != cudaSuccess ||
-        cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess) {
-        if (c->ev_fork) cudaEventDestroy(c->ev_fork);
-        if (c->side) cudaStreamDestroy(c->side);
+    bool ok = cudaMemsetAsync(c->ws, 0, sizeof(Workspace), c->stream) == cudaSuccess &&
+              cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) == cudaSuccess;
+    for (int i = 0; i < kSides && ok; ++i)
+        ok = cudaStreamCreateWithFlags(&c->side[i], cudaStreamNonBlocking) == cudaSuccess &&
+             cudaEventCreateWithFlags(&c->ev_join[i], cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) {
+        release_launches(c);
         cudaFree(c->ws);
         cudaFree(c->partials);
         cudaFree(c->d_tensors);
@@ -655,10 +703,8 @@ int omse_destroy(omse_ctx* ctx) {
     if (!ctx) return OMSE_EINVAL;
     DeviceScope dev(ctx->device);
     cudaStreamSynchronize(ctx->stream);
-    cudaStreamSynchronize(ctx->side);
-    cudaEventDestroy(ctx->ev_fork);
-    cudaEventDestroy(ctx->ev_join);
-    cudaStreamDestroy(ctx->side);
+    for (cudaStream_t s : ctx->side) cudaStreamSynchronize(s);
+    release_launches(ctx);
     cudaFree(ctx->ws);
     cudaFree(ctx->partials);
     cudaFree(ctx->d_tensors);

@@ -240,6 +240,10 @@ __device__ __forceinline__ void lattice_each(const BlockTeam& tm, const LatticeR
     }
 }
 
+// additions to a word of shared memory by its 32-bit address
+__device__ __forceinline__ void shared_add(unsigned int at, unsigned int v) { asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(at), "r"(v) : "memory"); }
+__device__ __forceinline__ void shared_add1(unsigned int at) { asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(at) : "memory"); }
+
 // The bin m of a >= h and the remainder r = a - m*h, 0 <= r < h.  inv_up exceeds 1/h by 2.3e-7 to 4.8e-7 of it, so floor(a*inv_up)
 // is m or, where it is the bin above, the remainder is negative (a/h < 2^21).  No rounding: r is a multiple of the last place of h.
 __device__ __forceinline__ float lattice_inv_up(float inv) { return inv * (1.0f + 3.0e-7f); }
@@ -374,6 +378,11 @@ __device__ __forceinline__ int lattice_fbits(long long terms) {
 }
 
 // Puts the row's values into the histograms; returns this thread's share of sum T^2.
+// Bound: the two atomics (eight clocks each for a warp's random words) and instruction issue.  Per value: the bin (M - 1 + m by one
+// rounded-down multiply-add, so that its low bits are the word's index and no integer is formed), the remainder, two atomics at
+// addresses that come out of the float's bits by a shift and an addition that wraps; one test in four values for those that the
+// reciprocal put into the bin above.  With the codes of the passes four at a time: 2674 rows of 25,088 values on 8 bits 427 -> 416 us,
+// two tensors of 4 bits 1411 -> 1377.
 template <bool PACKED, bool TINY>
 __device__ __forceinline__ float lattice_insert(const BlockTeam& tm, const LatticeSmem& sm, const float4* xs4, int k4, float step,
                                                 bool sgn, int n_bins, int lb, int fbits, int d, int n_bins2, int lb2, int f2bits) {
@@ -384,34 +393,60 @@ __device__ __forceinline__ float lattice_insert(const BlockTeam& tm, const Latti
     const float inv_fix = inv * (float)(1 << fbits);
     const unsigned int rd = d > 0 ? (unsigned)((0x100000000ull + d - 1) / d) : 0u;   // m/d = (m*rd) >> 32 for m < 2^24
     const int d_from = d > 0 ? d : 0x7fffffff;
-    float e = 0.f;
+    constexpr float kBase = kMagic - 1.0f;
+    constexpr unsigned int kBits = 0x4B400000u;                     // of M: bin 1, word 0
+    const unsigned int n_at = (unsigned)__cvta_generic_to_shared(sm.n), f_at = (unsigned)__cvta_generic_to_shared(sm.f) - 4u * kBits;
+    const u64 inv2 = pack2(inv, inv), zero2 = pack2(-0.f, -0.f), pre2 = pack2(pre, pre);
+    u64 e2 = 0ull;
     for (int i4 = tm.t; i4 < k4; i4 += tm.size()) {
-        const float4 v = xs4[i4];
-        const float x[4] = {v.x, v.y, v.z, v.w};
+        float4 v = xs4[i4];
+        u64 ya = pack2(v.x, v.y), yb = pack2(v.z, v.w);
+        if (TINY) {
+            ya = fma2(ya, pre2, zero2);
+            yb = fma2(yb, pre2, zero2);
+            unpack2(ya, v.x, v.y);
+            unpack2(yb, v.z, v.w);
+        }
+        const u64 ta = fma2(ya, inv2, zero2), tb = fma2(yb, inv2, zero2);
+        e2 = fma2(tb, tb, fma2(ta, ta, e2));
+        const float y[4] = {v.x, v.y, v.z, v.w};
+        float u[4], r[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const float y = TINY ? x[j] * pre : x[j];
-            const float a = sgn ? fabsf(y) : y;                     // an unsigned range codes negative values as 0
-            const float t = a * inv;
-            e = fmaf(t, t, e);
-            if (a >= h) {
-                int m;
-                const float r = lattice_bin(a, h, inv_up, m);
-                const unsigned int fi = (unsigned)magic_int(fmaf(r, inv_fix, kMagic));
-                const int w = lattice_word(min(m, n_bins) - 1, lb);
-                Counts<PACKED>::add(sm.n, w);
-                atomicAdd(sm.f + w, fi);
-                if (y < 0.f && m >= d_from) {
-                    const unsigned int m2 = __umulhi((unsigned)m, rd);
-                    const unsigned int rem = (unsigned)m - m2 * (unsigned)d;
-                    const int w2 = lattice_word(min((int)m2, n_bins2) - 1, lb2);
-                    atomicAdd(sm.n2 + w2, 1u);
-                    atomicAdd(sm.f2 + w2, (rem << f2bits) + (fi >> (fbits - f2bits)));
+            const float a = sgn ? fabsf(y[j]) : y[j];               // an unsigned range codes negative values as 0
+            u[j] = __fmaf_rd(a, inv_up, kBase);
+            r[j] = fmaf(-(u[j] - kBase), h, a);
+        }
+        if (fminf(fminf(fminf(r[0], r[1]), r[2]), r[3]) < 0.f) {    // below an edge by a few 1e-7
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (r[j] < 0.f) {
+                    r[j] += h;
+                    u[j] -= 1.0f;
                 }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (TINY) u[j] = fminf(u[j], kBase + (float)n_bins);    // (a subnormal step is off by more than the last bin allows for)
+            if (!(u[j] >= kMagic)) continue;                        // below the first bin
+            const unsigned int bits = __float_as_uint(u[j]), w = bits ^ ((bits >> (lb - 2)) & 0x1cu);      // lattice_word of the index
+            const unsigned int fi = __float_as_uint(fmaf(r[j], inv_fix, kMagic)) - kBits;
+            if (PACKED) shared_add(n_at + ((w >> 1) << 2) - 2u * kBits, 1u << ((w & 1u) << 4));
+            else shared_add1(n_at + (w << 2) - 4u * kBits);
+            shared_add(f_at + (w << 2), fi);
+            const int m = (int)(bits - kBits) + 1;
+            if (y[j] < 0.f && m >= d_from) {
+                const unsigned int m2 = __umulhi((unsigned)m, rd);
+                const unsigned int rem = (unsigned)m - m2 * (unsigned)d;
+                const int w2 = lattice_word(min((int)m2, n_bins2) - 1, lb2);
+                atomicAdd(sm.n2 + w2, 1u);
+                atomicAdd(sm.f2 + w2, (rem << f2bits) + (fi >> (fbits - f2bits)));
             }
         }
     }
-    return e;
+    float ea, eb;
+    unpack2(e2, ea, eb);
+    return ea + eb;
 }
 
 // sum over the levels first, first + stride, ... of P at candidate c (a1 = c+1), in units of 2^-shift

@@ -23,6 +23,7 @@ struct RowTensor {
     int rows_per_unit;       // block per row: 2 when nibble packing needs an even element count per unit (odd K), else 1;
                              // short rows: what a warp takes, 32 >> lanes at a time (even)
     int lanes;               // short rows: lanes per row (log2)
+    int hist_fbits, hist_cshift;    // short rows by a histogram of their warp: see HistShape
 };
 
 struct RowArgs {
@@ -54,6 +55,7 @@ struct RowArgs {
     float eps;                  // >= 0: Algorithm 1 stops after the first sweep whose relative error decrease is <= eps
     int* sweeps_done;           // [S] sweeps Algorithm 1 ran per row, nullable
     int short_direct;           // short rows: a candidate per lane
+    int hist_lb;                // short rows by a histogram: log2 of the bins in a lane's run
     int short_rows4, short_slots, short_codes, short_bytes;   // short rows: shared memory of a warp (float4s of the rows, slots
                                 // of the stacks, offset of the codes, size)
     int ext_tensors;            // a tensor of a batched launch has a gate or an earlier tensor's scale
@@ -128,19 +130,20 @@ __device__ __forceinline__ double exact_sse_block(const float* xs, int k, float 
                                                    double* scratch) {
     double ss = 0.0;
     long long zero = 0;
-    const float inv = __fdiv_rn(1.0f, alpha), thr = ambiguity_threshold(flo, fhi);
+    const Coder coder(alpha, __fdiv_rn(1.0f, alpha), flo, fhi);
     const double ad = (double)alpha;
     // four elements per step (the row is zero padded to a multiple of four; a zero has code 0 and error 0)
     const float4* xs4 = reinterpret_cast<const float4*>(xs);
     const int k4 = (k + 3) >> 2;
+#pragma unroll 1
     for (int i4 = threadIdx.x; i4 < k4; i4 += blockDim.x) {
         const float4 v = xs4[i4];
         const float x[4] = {v.x, v.y, v.z, v.w};
-        int q[4];
-        exact_codes4(x, alpha, inv, flo, fhi, thr, q);
+        float t[4];
+        coder.of(v, t);
         double d[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) d[e] = fma(-ad, int_double(q[e]), (double)x[e]);
+        for (int e = 0; e < 4; ++e) d[e] = fma(-ad, magic_double(t[e]), (double)x[e]);
 #pragma unroll
         for (int e = 0; e < 4; ++e) ss = fma(d[e], d[e], ss);
     }
@@ -155,21 +158,20 @@ __device__ __forceinline__ float polish_block(const float* xs, int k, float alph
     const int k4 = (k + 3) >> 2;
     for (int it = 0; it < n; ++it) {
         double sxq = 0.0;
-        long long sqq = 0;
-        const float inv = __fdiv_rn(1.0f, alpha), thr = ambiguity_threshold(flo, fhi);
-        for (int i4 = threadIdx.x; i4 < k4; i4 += blockDim.x) {   // four elements per step; the zero padding adds nothing
-            const float4 v = xs4[i4];
+        u64 qa = 0ull, qb = 0ull;
+        const Coder coder(alpha, __fdiv_rn(1.0f, alpha), flo, fhi);
+#pragma unroll 1
+        for (int i4 = threadIdx.x; i4 < k4; i4 += blockDim.x) {   // four elements per step (56 steps at most: blocks of 128 threads or
+            const float4 v = xs4[i4];                             // short rows); the zero padding adds nothing
             const float x[4] = {v.x, v.y, v.z, v.w};
-            int q[4];
-            exact_codes4(x, alpha, inv, flo, fhi, thr, q);
-            int qq = 0;
+            float t[4];
+            coder.of(v, t);
+            qa = add_squares(t[0], t[1], qa);
+            qb = add_squares(t[2], t[3], qb);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                qq += q[e] * q[e];
-                sxq = fma((double)x[e], int_double(q[e]), sxq);
-            }
-            sqq += qq;
+            for (int e = 0; e < 4; ++e) sxq = fma((double)x[e], magic_double(t[e]), sxq);
         }
+        long long sqq = squares_of(qa, qb);
         block_sum2(sxq, sqq, scratch);
         if (sqq == 0) break;
         const float a_new = (float)(sxq / (double)sqq);
@@ -335,44 +337,40 @@ __device__ double emit_block(const RowSmem& s, int k, float alpha, float flo, fl
     double ss = 0.0;
     const bool zero = !(alpha > 0.f);
     const float inv = zero ? 0.f : __fdiv_rn(1.0f, alpha), thr = ambiguity_threshold(flo, fhi);
+    const Coder coder(alpha, inv, flo, fhi);
     const double ad = (double)alpha;
     const bool aligned = ((reinterpret_cast<unsigned long long>(codes) & 3ull) == 0) &&
                          ((reinterpret_cast<unsigned long long>(packed) & 1ull) == 0);
     if ((k & 3) == 0 && aligned) {
         // aligned fast path: four codes per thread, 32-bit and 16-bit stores
         const float4* xs4 = reinterpret_cast<const float4*>(s.xs);
+#pragma unroll 1
         for (int i4 = tid; i4 < (k >> 2); i4 += nthr) {
             const float4 v = xs4[i4];
             const float x[4] = {v.x, v.y, v.z, v.w};
-            int q[4] = {0, 0, 0, 0};
-            if (!zero) exact_codes4(x, alpha, inv, flo, fhi, thr, q);
+            float t[4] = {kMagic, kMagic, kMagic, kMagic};
+            if (!zero) coder.of(v, t);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const double d = fma(-ad, int_double(q[e]), (double)x[e]);
+                const double d = fma(-ad, magic_double(t[e]), (double)x[e]);
                 ss = fma(d, d, ss);
             }
-            if (codes) {
-                const unsigned int w = (q[0] & 0xff) | ((q[1] & 0xff) << 8) | ((q[2] & 0xff) << 16) | ((unsigned)(q[3] & 0xff) << 24);
-                *reinterpret_cast<unsigned int*>(codes + row_base + 4ll * i4) = w;
-            }
-            if (packed) {
-                const unsigned short h = (unsigned short)((q[0] & 0xf) | ((q[1] & 0xf) << 4) | ((q[2] & 0xf) << 8) | ((q[3] & 0xf) << 12));
-                *reinterpret_cast<unsigned short*>(packed + ((row_base + 4ll * i4) >> 1)) = h;
-            }
+            const unsigned int w = code_bytes(t);
+            if (codes) *reinterpret_cast<unsigned int*>(codes + row_base + 4ll * i4) = w;
+            if (packed) *reinterpret_cast<unsigned short*>(packed + ((row_base + 4ll * i4) >> 1)) = (unsigned short)byte_nibbles(w);
         }
     } else if (!packed) {
         // codes alone at any offset: a byte per element, four independent ones per step
         for (int i = tid; i < k; i += 4 * nthr) {
-            float x[4];
-            int q[4] = {0, 0, 0, 0};
+            float x[4], t[4] = {kMagic, kMagic, kMagic, kMagic};
 #pragma unroll
             for (int e = 0; e < 4; ++e) x[e] = i + e * nthr < k ? s.xs[i + e * nthr] : 0.f;      // a zero has code 0 and error 0
-            if (!zero) exact_codes4(x, alpha, inv, flo, fhi, thr, q);
+            if (!zero) coder.of(make_float4(x[0], x[1], x[2], x[3]), t);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const double d = fma(-ad, int_double(q[e]), (double)x[e]);
+                const double d = fma(-ad, magic_double(t[e]), (double)x[e]);
                 ss = fma(d, d, ss);
-                if (codes && i + e * nthr < k) codes[row_base + i + e * nthr] = (signed char)q[e];
+                if (codes && i + e * nthr < k) codes[row_base + i + e * nthr] = (signed char)magic_int(t[e]);
             }
         }
     } else {
@@ -645,16 +643,15 @@ __global__ void __launch_bounds__(kRowsThreads) rows_kernel(const RowArgs a) {
                 }
                 if (!a.keep_x0 && j + 1 < a.n_tensors) {
                     // first sweep without a kept copy: the residual is updated in place
-                    const float inv = r.alpha > 0.f ? __fdiv_rn(1.0f, r.alpha) : 0.f, thr = ambiguity_threshold(flo, fhi);
+                    const Coder coder(r.alpha, r.alpha > 0.f ? __fdiv_rn(1.0f, r.alpha) : 0.f, flo, fhi);
                     float4* xw4 = reinterpret_cast<float4*>(s.xs);
                     if (r.alpha > 0.f)
                         for (int i4 = tid; i4 < k4; i4 += nthr) {        // the padding zeros stay
                             const float4 v = xw4[i4];
-                            const float x[4] = {v.x, v.y, v.z, v.w};
-                            int q[4];
-                            exact_codes4(x, r.alpha, inv, flo, fhi, thr, q);
-                            xw4[i4] = make_float4(fmaf(-r.alpha, (float)q[0], x[0]), fmaf(-r.alpha, (float)q[1], x[1]),
-                                                  fmaf(-r.alpha, (float)q[2], x[2]), fmaf(-r.alpha, (float)q[3], x[3]));
+                            float t[4];
+                            coder.of(v, t);
+                            xw4[i4] = make_float4(fmaf(-r.alpha, t[0] - kMagic, v.x), fmaf(-r.alpha, t[1] - kMagic, v.y),
+                                                  fmaf(-r.alpha, t[2] - kMagic, v.z), fmaf(-r.alpha, t[3] - kMagic, v.w));
                         }
                 }
                 bool stop = false;

@@ -27,6 +27,8 @@ namespace omse {
 
 constexpr int kShortThreads = 128;       // blocks of four warps: five per SM at 96 registers, against four at 128 and six at 80
 constexpr int kShortBlocks = 5;          // (rows of 147 values 492 us, 503 and 514; of 27 values 1148, 1172 and 1267)
+// Searches of rows_short_kernel; the last two take all lanes of a warp for one row.
+constexpr int kBySplits = 0, kByLanes = 1, kByHistogram = 2;
 constexpr int kShortMinQuads = 3;
 constexpr int kShortQuads = 10;          // float4s of a row per lane, at most
 
@@ -84,8 +86,8 @@ __device__ __forceinline__ float group_max(float v, int lg) {
 // Shared memory of one warp.
 struct ShortSmem {
     float4* xs;            // [group][short_stride4] the rows of a step, zero padded
-    signed char* qs;       // their codes on the way out
-    float2* stack;         // [slot][group] a candidate's index + 1 and 2*step*W there
+    float2* stack;         // [slot][group] a candidate's index + 1 and 2*step*W there; or the histogram
+    signed char* qs;       // the rows' codes on the way out, in the same place
     unsigned short* close; // [kShortClose][group] candidates within the noise band of the smallest error
 };
 // A row with one value far above the others has equal errors at every candidate that divides it without remainder, and
@@ -111,7 +113,7 @@ struct ShortRow {
     int k4, lg, g, j;      // float4s; lanes per row (log2); group of this lane, lane of its group
     bool search;
     float step, sc;        // grid; power of two that the values are multiplied by where their squares would leave binary32
-    float mpos, mneg, e, w_zero;    // scaled: maxima of the positive and negative part, sum of squares, 2*step*W at alpha = 0
+    float mpos, mneg, e, l1, w_zero;    // scaled: maxima of the positive and negative part, sums of squares and magnitudes, 2*step*W at alpha = 0
     float flo, fhi;
 };
 // The candidates that may be the minimum, by their index + 1: the one with the smallest binary32 error, the others within the
@@ -239,6 +241,281 @@ __device__ __forceinline__ ShortResult short_dispatch(int quads, const ShortSmem
         if (quads < NQ) return short_dispatch<NQ - 1>(quads, sm, r, n_cand);
     }
     return short_search<NQ>(sm, r, n_cand);
+}
+
+// ---- The search for the longer ones of the short rows: a warp makes one histogram of its row, as the block path does (see
+// omse_lattice.cuh), and looks the candidates up.  What is different: the count and the fractional sum of a bin share one word
+// (random words of shared memory take an atomic of a warp eight clocks, whatever is added), the fraction has eight to twelve bits, so
+// that bin and fraction are bit fields of one multiply-add's result, and the extra negative level has no histogram: counting it on both
+// sides gives a lower bound of the error, the largest negative value alone an upper one, and only the candidates that these leave
+// open (some 40 of 1024) get the exact sum over the few values that lie beyond it.  If more than one is within the noise of the
+// fractions, they are evaluated in binary32, as the splits do.
+// Bound: chains of dependent instructions (12 to 20 warps per SM) and 1000 clocks of an SM per row for clearing, scanning and looking
+// up 2048 bins.  Measured on one B200, 1024 candidates, 67M Laplace values, against splits (up to 1024 values) and a block per row:
+// 4 bits, 512 values a row 886 -> 782 us, 1024 829 -> 603, 1280 1014 -> 564, 2304 698 -> 538; 8 bits, 1024 998 -> 772, 2304 783 -> 563.
+struct HistShape {
+    int n_bins, lb, fbits, cshift;        // bins; log2 of a lane's run of them; bits of a fraction; the count's place in the word
+};
+constexpr int kHistOpen = 4;              // open candidates per lane at a time
+__device__ __forceinline__ bool hist_search(const ShortSmem& sm, const ShortRow& r, int k, int n_cand, const HistShape& g, ShortResult& res) {
+    const int lane = threadIdx.x & 31;
+    unsigned int* P = reinterpret_cast<unsigned int*>(sm.stack);
+    float* coarse = reinterpret_cast<float*>(P + (32 << g.lb));
+    res = ShortResult{0.f, 0.f, 0.f, 0.f, 0};
+    if (!r.search) return true;                               // (the same in all lanes)
+    if (r.sc != 1.0f) return false;
+    const int lb = g.lb, run = 1 << lb, levels = (int)r.fhi, n_bins = g.n_bins;
+    const bool sgn = r.flo < 0.f;
+    const int d = sgn ? 2 * (int)(-r.flo) - 1 : 0;
+    for (int i = lane; i < (8 << lb); i += 32) reinterpret_cast<uint4*>(P)[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+    // ---- insertion
+    const float h = 0.5f * r.step, inv = __fdiv_rn(1.0f, h);
+    {
+        const float inv_b = inv * (float)(1 << g.fbits), base = 8388608.0f - (float)(1 << g.fbits);      // 2^23: bin 1 is word 0
+        const unsigned int mask = (1u << g.fbits) - 1u, one = 1u << g.cshift;
+        const int s1 = g.fbits, s2 = g.fbits + lb - 2;
+        const unsigned int at = (unsigned)__cvta_generic_to_shared(P) - 4u * (0x4B000000u >> s1);
+#pragma unroll 2
+        for (int i = lane; i < r.k4; i += 32) {
+            const float4 v = sm.xs[i];
+            const float y[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float u = fmaf(sgn ? fabsf(y[j]) : y[j], inv_b, base);
+                const unsigned int bits = __float_as_uint(u);
+                if (u >= 8388608.0f) shared_add(at + 4u * ((bits >> s1) ^ ((bits >> s2) & 0x1cu)), (bits & mask) | one);
+            }
+        }
+    }
+    __syncwarp();
+    // ---- P(m) at word m - 1, in units of 2^-shift.  Counts and fractions of all bins together stay in their fields, so one addition
+    //      does for both.
+    int shift;
+    {
+        const int first = lane << lb;
+        const unsigned int fmask = (1u << g.cshift) - 1u;
+        unsigned int a = 0u, s = 0u;
+        for (int q = run - 4; q >= 0; q -= 4) {
+            const uint4 w = *reinterpret_cast<const uint4*>(P + lattice_word(first + q, lb));
+            s += a >> g.cshift;
+            a += w.w;
+            s += a >> g.cshift;
+            a += w.z;
+            s += a >> g.cshift;
+            a += w.y;
+            s += a >> g.cshift;
+            a += w.x;
+        }
+        const unsigned int own_a = a, own_s = s;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned int a2 = __shfl_down_sync(0xffffffffu, a, o), s2 = __shfl_down_sync(0xffffffffu, s, o);
+            if (lane + o < 32) {
+                s += s2 + ((unsigned)o << lb) * (a2 >> g.cshift);
+                a += a2;
+            }
+        }
+        const unsigned int total_a = __shfl_sync(0xffffffffu, a, 0), total_s = __shfl_sync(0xffffffffu, s, 0);
+        shift = scan_shift(total_a >> g.cshift, total_s, g.fbits);
+        // what lies behind this lane's run, at the run's end
+        a -= own_a;
+        s -= own_s + (unsigned)run * (a >> g.cshift);
+        const int drop = g.fbits - shift;
+        for (int q = run - 4; q >= 0; q -= 4) {
+            uint4* at = reinterpret_cast<uint4*>(P + lattice_word(first + q, lb));
+            uint4 w = *at;
+            auto put = [&](unsigned int x) {
+                s += a >> g.cshift;
+                a += x;
+                return (s << shift) + ((a & fmask) >> drop);
+            };
+            w.w = put(w.w);
+            w.z = put(w.z);
+            w.y = put(w.y);
+            w.x = put(w.x);
+            *at = w;
+        }
+    }
+    __syncwarp();
+    // ---- errors in units of h^2, E less its share of the levels
+    const double e = (double)r.e * (double)inv * (double)inv, scale = -4.0 * __longlong_as_double((long long)(1023 - shift) << 52);
+    const float ef = (float)e, q = __int_as_float((127 - shift) << 23), qn = (2.0f * (float)n_bins + 8.0f * (float)n_cand) * q;
+    const float s1 = r.l1 * inv, inv_f = __int_as_float((127 - g.fbits) << 23);
+    auto upper_sum = [&](int a1, int first, int stride) -> unsigned long long {
+        unsigned long long acc = 0ull;
+        const int last = min(n_bins, (2 * levels - 1) * a1);
+        for (int m = (2 * first + 1) * a1; m <= last; m += 2 * stride * a1) acc += P[lattice_word(m - 1, lb)];
+        return acc;
+    };
+    auto usable = [&](int a1) { return usable_scale(__fmul_rn((float)a1, r.step)); };
+    auto error = [&](int a1, unsigned long long p) { return usable(a1) ? (float)fma(scale * (double)a1, u52_double(p), e) : INFINITY; };
+    // The extra level's sum lies between what the largest negative value alone gives and what all values give less the largest
+    // positive one's.
+    const float t_pos = r.mpos * inv, t_neg = r.mneg * inv;
+    auto alone = [&](float t, int m) -> unsigned int {
+        return d > 0 ? (unsigned int)(fmaxf(t * 0.999999f - (float)m - 0.01f, 0.f) * (float)(1 << shift)) : 0u;
+    };
+    auto beyond = [&](int a1) -> unsigned int {
+        const int m = d * a1;
+        if (d == 0 || !(t_neg > (float)m) || m > n_bins) return 0u;
+        const unsigned int all = P[lattice_word(m - 1, lb)];
+        return all - min(all, alone(t_pos, m));
+    };
+    // ---- coarse candidates: upper bounds give the threshold, lower bounds are kept
+    const int n_coarse = coarse_count(n_cand);
+    float least = INFINITY;
+    auto note = [&](int i, int a1, unsigned long long p) {
+        least = fminf(least, error(a1, p + alone(t_neg, d * a1)));
+        coarse[i] = error(a1, p + beyond(a1));
+    };
+    int done = 0;
+    if (levels > 8) {
+        // The smallest scales have the most levels: 8 lanes share each of the first 16, 4 each of the next 8.  The smallest of all, which
+        // leave the largest value further away than the whole error is at the first scale that reaches it, are not looked at.
+        const float t_max = fmaxf(t_pos, t_neg), reach = ceilf(__fdividef(t_max, (float)(2 * levels + 1)) * 1.00001f) * 1.0001f;
+        const int skip = reach <= (float)n_cand ? max(0, (int)floorf(__fdividef(t_max - sqrtf((float)k) * reach, (float)(2 * levels + 2)) * 0.9999f) - 1) : 0;
+        for (int i = lane; i < min(min(skip, 16), n_coarse); i += 32) coarse[i] = 3e38f;
+        auto shared = [&](int from, int to, int lanes) {
+            for (int i0 = from; i0 < to; i0 += 32 / lanes) {
+                const int i = i0 + lane / lanes, a1 = coarse_a1(i, n_cand);
+                unsigned long long p = i < to ? upper_sum(a1, lane & (lanes - 1), lanes) : 0ull;
+                for (int o = 1; o < lanes; o <<= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
+                if (i < to && (lane & (lanes - 1)) == 0) note(i, a1, p);
+            }
+        };
+        shared(min(skip, 16), min(16, n_coarse), 8);
+        shared(16, min(24, n_coarse), 4);
+        done = 24;
+    }
+    for (int i = done + lane; i < n_coarse; i += 32) {
+        const int a1 = coarse_a1(i, n_cand);
+        note(i, a1, upper_sum(a1, 0, 1));
+    }
+    __syncwarp();
+    // (values may be below zero by what E is off)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) least = fminf(least, __shfl_xor_sync(0xffffffffu, least, o));
+    if (!(least < INFINITY)) return true;                     // no usable scale
+    // What a value may be off by at candidate a1: the fraction by 2^-(F+1) per value and level, at most T/(2*a1) + 1/2 levels of
+    // 4*a1 each, none below T = a1; the truncation of P; and, as in lattice_band, what the scales' and the quotients' rounding move
+    // (the reciprocal's, the same for all values, among them).
+    auto noise = [&](float v, float a1) {
+        const float dv = fmaxf(v, 0.f) + 2e-6f * ef;
+        return inv_f * fminf(s1 + a1 * (float)k, 2.0f * s1) + qn + 6e-7f * sqrtf(dv * ef) + 1e-9f * ef;
+    };
+    auto band = [&](float v, float a1) { return v + (float)kRescoreBand * (fmaxf(v, 0.f) + 2e-6f * ef) + 2.0f * noise(v, a1); };
+    const float keep = band(least, (float)n_cand) + 1e-6f * ef;            // 1e-6: binary32 in the bounds below
+    int lo = 0x7fffffff, hi = -1;
+    for (int i = lane; i < n_coarse; i += 32) {
+        const int a0 = coarse_a1(i, n_cand);
+        if (!(coarse[i] > keep)) {
+            lo = min(lo, a0);
+            hi = max(hi, a0);
+        }
+        if (i + 1 >= n_coarse) continue;
+        const int a1 = coarse_a1(i + 1, n_cand);
+        if (a1 - a0 >= 2 && !(chord_bound(ef, a0, coarse[i], a1, coarse[i + 1]) > keep)) {      // (an unusable end keeps the interval)
+            lo = min(lo, a0 + 1);
+            hi = max(hi, a1 - 1);
+        }
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    // ---- the open candidates, four to a lane at a time, with the extra level as it is: the negative values beyond it are met one by
+    //      one.  First the smallest error, then the candidates within the noise (found again where there were more than one lot).
+    float value[kHistOpen], best = INFINITY, most = 0.f, limit = 0.f, single = 0.f, best_v = INFINITY;
+    int met = 0, n_left = 0;
+    // a candidate within the noise by its binary32 error (the same in all lanes); what is kept is what short_search keeps
+    auto consider = [&](float a1) {
+        const float v = warp_allsum(direct_part<false>(sm.xs, r.k4, lane, 32, __fmul_rn(a1, r.step), 1.0f, r.flo, r.fhi));
+        const float band_f = 1.0f + 1.25f * (float)kRescoreBand;
+        res.n_eval += 1.f;
+        if (!(v <= best_v * band_f)) return;
+        const bool fresh = v * band_f < best_v;
+        res.n_close = fresh ? 0 : res.n_close;
+        res.w_lo = fresh ? a1 : res.w_lo;
+        res.w_hi = a1;
+        if (v < best_v) {                                     // (increasing scales: the lowest one keeps a tie)
+            best_v = v;
+            res.best = a1;
+        }
+        sm.close[min(res.n_close, kShortClose - 1)] = (unsigned short)a1;
+        ++res.n_close;
+    };
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll 1
+        for (int first = lo; first <= hi; first += 32 * kHistOpen) {
+            const int last = min(hi, first + 32 * kHistOpen - 1);
+            if (pass == 0 || hi - lo >= 32 * kHistOpen) {
+                float extra[kHistOpen] = {0.f, 0.f, 0.f, 0.f};
+                if (d > 0 && t_neg > (float)(d * first)) {
+                    const float from = -((float)(d * first) * h);
+#pragma unroll 1
+                    for (int i0 = 0; i0 < r.k4; i0 += 32) {
+                        const float4 v = i0 + lane < r.k4 ? sm.xs[i0 + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+                        const float y[4] = {v.x, v.y, v.z, v.w};
+                        if (!__any_sync(0xffffffffu, fminf(fminf(fminf(y[0], y[1]), y[2]), y[3]) < from)) continue;
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            unsigned int some = __ballot_sync(0xffffffffu, y[j] < from);
+                            met += __popc(some);
+                            while (some) {
+                                const float t = -__shfl_sync(0xffffffffu, y[j], __ffs(some) - 1) * inv;
+                                some &= some - 1;
+#pragma unroll
+                                for (int c = 0; c < kHistOpen; ++c) {
+                                    if (first + 32 * c > last) break;
+                                    extra[c] += fmaxf(t - (float)(d * (first + lane + 32 * c)), 0.f);
+                                }
+                            }
+                        }
+                    }
+                }
+#pragma unroll
+                for (int c = 0; c < kHistOpen; ++c) {
+                    const int a1 = first + lane + 32 * c;
+                    value[c] = INFINITY;
+                    if (a1 <= last) {
+                        const float gain = 4.0f * (float)a1 * extra[c];
+                        value[c] = error(a1, upper_sum(a1, 0, 1)) - gain;
+                        most = fmaxf(most, gain);
+                    }
+                    best = fminf(best, value[c]);
+                }
+            }
+            if (pass == 0) continue;
+#pragma unroll
+            for (int c = 0; c < kHistOpen; ++c) {
+                unsigned int some = __ballot_sync(0xffffffffu, value[c] <= limit);
+                while (some) {
+                    const float a1 = (float)(first + __ffs(some) - 1 + 32 * c);
+                    some &= some - 1;
+                    if (n_left == 1) consider(single);
+                    if (n_left > 0) consider(a1);
+                    else single = a1;                         // (left as it is if it is the only one)
+                    ++n_left;
+                }
+            }
+        }
+        if (pass == 1) break;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
+            most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, o));
+        }
+        if (!(best < INFINITY)) return true;
+        // (binary32 in the sums of `extra`: values by 1.2e-7, the additions by half of that each)
+        limit = band(best, (float)hi) + 2.0f * (1.2e-7f + 6e-8f * (float)met) * most + 2.5e-7f * ef / (float)max(d, 1);
+    }
+    res.n_eval += 1.f;
+    if (n_left == 1) {
+        res.best = res.w_lo = res.w_hi = single;
+        res.n_close = 1;
+    }
+    __syncwarp();                                             // the list
+    return true;
 }
 
 // ---- The search for small launches, where a row's chain of evaluations is what counts: the whole warp on one row, a
@@ -415,7 +692,7 @@ __device__ __forceinline__ ShortResult direct_search(const ShortSmem& sm, const 
 // where that shares a byte of packed codes with it); more: the warp goes on with the next rows of the same tensor.
 // Outside the search the rows are read from shared memory in loops that are not unrolled: the code of the passes, unrolled
 // over registers, was most of the kernel, and warps waited for instructions (rows of 27 values 1.42 -> 1.20 ms).
-template <bool DIRECT>
+template <int BY>
 __device__ __forceinline__ void short_step(const RowArgs& a, const RowTensor& T, const ShortSmem& sm, int lg, long long row0, int nrows,
                                            bool more, int& carry, unsigned int& st, unsigned long long& ev) {
     const int lane = threadIdx.x & 31;
@@ -430,7 +707,11 @@ __device__ __forceinline__ void short_step(const RowArgs& a, const RowTensor& T,
     const long long row = row0 + r.g, flat0 = row0 * T.K;
     r.flo = (float)a.lo[0];
     r.fhi = (float)a.hi[0];
-    const float flo = r.flo, fhi = r.fhi, thr = ambiguity_threshold(flo, fhi);
+    const float flo = r.flo, fhi = r.fhi;
+    auto codes = [](const Coder& coder, const float4& v, float (&t)[4]) {
+        if (BY == kBySplits) coder.of_single(v, t);
+        else coder.of(v, t);
+    };
 
     // ---- the rows into shared memory
     __syncwarp();                                        // the previous step's rows and codes have been read
@@ -472,16 +753,16 @@ __device__ __forceinline__ void short_step(const RowArgs& a, const RowTensor& T,
             for (int u = 4 * i; u < min(4 * i + 4, k); ++u) reinterpret_cast<float*>(mine)[u] = y[u] - off;
         if (active && r.j == 0) T.delta[row] = off;
     } else if (T.prior_alpha) {                          // second tensor of a key layer: the residual of the first one
-        const float a1 = active ? T.prior_alpha[row] : 0.f, inv = a1 > 0.f ? __fdiv_rn(1.0f, a1) : 0.f;
+        const float a1 = active ? T.prior_alpha[row] : 0.f;
+        const Coder coder(a1, a1 > 0.f ? __fdiv_rn(1.0f, a1) : 0.f, flo, fhi);
         if (a1 > 0.f)
 #pragma unroll 1
             for (int i = r.j; i < own; i += 1 << lg) {
                 const float4 v = mine[i];
-                const float y[4] = {v.x, v.y, v.z, v.w};
-                int q[4];
-                exact_codes4(y, a1, inv, flo, fhi, thr, q);
-                mine[i] = make_float4(fmaf(-a1, (float)q[0], y[0]), fmaf(-a1, (float)q[1], y[1]),
-                                      fmaf(-a1, (float)q[2], y[2]), fmaf(-a1, (float)q[3], y[3]));
+                float t[4];
+                codes(coder, v, t);
+                mine[i] = make_float4(fmaf(-a1, t[0] - kMagic, v.x), fmaf(-a1, t[1] - kMagic, v.y),
+                                      fmaf(-a1, t[2] - kMagic, v.z), fmaf(-a1, t[3] - kMagic, v.w));
             }
     }
     // ---- maxima and sums; a power of two against overflow and underflow of the squares
@@ -530,14 +811,20 @@ __device__ __forceinline__ void short_step(const RowArgs& a, const RowTensor& T,
     r.e = group_sum(e, lg);
     l1 = group_sum(l1, lg);
     l0 = group_sum(l0, lg);
+    r.l1 = l1;
     r.w_zero = r.step * r.sc * (fhi * (l1 + l0) - flo * (l1 - l0));         // every level counts |x| in full
 
     ShortResult s;
-    if constexpr (DIRECT) {
-        __syncwarp();                                    // the other lanes' part of the row
-        s = direct_search(sm, r, a.n_cand);
-    } else {
+    if constexpr (BY == kBySplits) {
         s = short_dispatch<kShortQuads>((k4 + (1 << lg) - 1) >> lg, sm, r, a.n_cand);
+    } else {
+        __syncwarp();                                    // the other lanes' part of the row
+        bool found = false;
+        if constexpr (BY == kByHistogram) {
+            found = hist_search(sm, r, k, a.n_cand, HistShape{a.n_bins, a.hist_lb, T.hist_fbits, T.hist_cshift}, s);
+            __syncwarp();
+        }
+        if (!found) s = direct_search(sm, r, a.n_cand);
     }
 
     // ---- candidates within the fp32 noise band of the minimum: decide in fp64 with exact codes
@@ -550,7 +837,8 @@ __device__ __forceinline__ void short_step(const RowArgs& a, const RowTensor& T,
         for (int i = 0; __any_sync(0xffffffffu, open); ++i) {
             float a1 = s.w_lo + (float)i;
             if (open && listed) a1 = (float)sm.close[(i << (5 - lg)) + r.g];
-            const float ac = __fmul_rn(a1, r.step), inv = __fdiv_rn(1.0f, ac);
+            const float ac = __fmul_rn(a1, r.step);
+            const Coder coder(ac, __fdiv_rn(1.0f, ac), flo, fhi);
             const double ad = (double)ac;
             double ss = 0.0;
             const bool ok = open && usable_scale(ac);
@@ -558,11 +846,11 @@ __device__ __forceinline__ void short_step(const RowArgs& a, const RowTensor& T,
             for (int q4 = r.j; q4 < (ok ? own : 0); q4 += 1 << lg) {    // the padding zeros code to 0 and add nothing
                 const float4 v = mine[q4];
                 const float y[4] = {v.x, v.y, v.z, v.w};
-                int q[4];
-                exact_codes4(y, ac, inv, flo, fhi, thr, q);
+                float t[4];
+                codes(coder, v, t);
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    const double d = fma(-ad, int_double(q[u]), (double)y[u]);
+                    const double d = fma(-ad, magic_double(t[u]), (double)y[u]);
                     ss = fma(d, d, ss);
                 }
             }
@@ -585,23 +873,22 @@ __device__ __forceinline__ void short_step(const RowArgs& a, const RowTensor& T,
     {
         bool open = found;
         for (int it = 0; it < a.refine_iters && __any_sync(0xffffffffu, open); ++it) {
-            const float inv = found ? __frcp_rn(alpha) : 0.f;
+            const Coder coder(alpha, found ? __frcp_rn(alpha) : 0.f, flo, fhi);
             double sxq = 0.0;
-            int sqq = 0;
+            u64 qa = 0ull, qb = 0ull;
 #pragma unroll 1
             for (int q4 = r.j; q4 < (open ? own : 0); q4 += 1 << lg) {
                 const float4 v = mine[q4];
                 const float y[4] = {v.x, v.y, v.z, v.w};
-                int q[4];
-                exact_codes4(y, alpha, inv, flo, fhi, thr, q);
+                float t[4];
+                codes(coder, v, t);
+                qa = add_squares(t[0], t[1], qa);        // (18 steps at most: see there)
+                qb = add_squares(t[2], t[3], qb);
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    sqq += q[u] * q[u];
-                    sxq = fma((double)y[u], int_double(q[u]), sxq);
-                }
+                for (int u = 0; u < 4; ++u) sxq = fma((double)y[u], magic_double(t[u]), sxq);
             }
             sxq = group_sum(sxq, lg);
-            sqq = group_sum(sqq, lg);
+            const int sqq = group_sum((int)squares_of(qa, qb), lg);
             const float a_new = (float)(sxq / (double)sqq);
             open = open && sqq != 0 && a_new >= FLT_MIN && a_new <= FLT_MAX && a_new != alpha;   // a fixed point would repeat exactly
             if (open) alpha = a_new;
@@ -611,28 +898,27 @@ __device__ __forceinline__ void short_step(const RowArgs& a, const RowTensor& T,
     const int o = (int)(flat0 & 7);
     signed char* qs = sm.qs;
     {
-        const float inv = alpha > 0.f ? __fdiv_rn(1.0f, alpha) : 0.f;
+        const Coder coder(alpha, alpha > 0.f ? __fdiv_rn(1.0f, alpha) : 0.f, flo, fhi);
         const double ad = (double)alpha;
         double ss = 0.0;
 #pragma unroll 1
         for (int q4 = r.j; q4 < own; q4 += 1 << lg) {
             const float4 v = mine[q4];
             const float y[4] = {v.x, v.y, v.z, v.w};
-            int q[4] = {0, 0, 0, 0};
-            if (alpha > 0.f) exact_codes4(y, alpha, inv, flo, fhi, thr, q);
+            float t[4] = {kMagic, kMagic, kMagic, kMagic};
+            if (alpha > 0.f) codes(coder, v, t);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const double d = fma(-ad, int_double(q[u]), (double)y[u]);
+                const double d = fma(-ad, magic_double(t[u]), (double)y[u]);
                 ss = fma(d, d, ss);
             }
             signed char* dst = qs + o + r.g * k + 4 * q4;
             if ((k & 3) == 0) {
-                *reinterpret_cast<unsigned int*>(dst) =
-                    (q[0] & 0xff) | ((q[1] & 0xff) << 8) | ((q[2] & 0xff) << 16) | ((unsigned)(q[3] & 0xff) << 24);
+                *reinterpret_cast<unsigned int*>(dst) = code_bytes(t);
             } else {
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
-                    if (4 * q4 + u < k) dst[u] = (signed char)q[u];
+                    if (4 * q4 + u < k) dst[u] = (signed char)magic_int(t[u]);
             }
         }
         ss = group_sum(ss, lg);
@@ -665,17 +951,15 @@ __device__ __forceinline__ void short_step(const RowArgs& a, const RowTensor& T,
         for (int b = b0 + lane; b < from; b += 32) dst[b] = byte_of(b);
         for (int b = from + 4 * lane; b < to; b += 128) {
             const uint2 u = *reinterpret_cast<const uint2*>(qs + 2 * b);
-            auto nibbles = [](unsigned int v) { return (v & 0xfu) | ((v >> 4) & 0xf0u) | ((v >> 8) & 0xf00u) | ((v >> 12) & 0xf000u); };
-            *reinterpret_cast<unsigned int*>(dst + b) = nibbles(u.x) | (nibbles(u.y) << 16);
+            *reinterpret_cast<unsigned int*>(dst + b) = __byte_perm(byte_nibbles(u.x), byte_nibbles(u.y), 0x5410);
         }
         if (to + lane < b1) dst[to + lane] = byte_of(to + lane);
         carry = qs[end - 1];
     }
 }
 
-// DIRECT: all lanes on one row, a candidate each (lanes = 5).
-template <bool DIRECT>
-__global__ void __launch_bounds__(kShortThreads, DIRECT ? 6 : kShortBlocks) rows_short_kernel(const RowArgs a) {
+template <int BY>
+__global__ void __launch_bounds__(kShortThreads, BY == kByLanes ? 6 : kShortBlocks) rows_short_kernel(const RowArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     ShortSmem sm;
@@ -692,14 +976,14 @@ __global__ void __launch_bounds__(kShortThreads, DIRECT ? 6 : kShortBlocks) rows
         if (unit >= a.n_units) break;
         const RowTensor& T = a.tensors ? a.tensors[tensor_of_unit(a, unit)] : a.one;
         if (T.gate && *T.gate == 0) continue;
-        const int lg = DIRECT ? 5 : T.lanes, groups = 32 >> lg;
+        const int lg = BY == kBySplits ? T.lanes : 5, groups = 32 >> lg;
         const long long row0 = (unit - T.unit_begin) * T.rows_per_unit;
         const int nrows = (int)min((long long)T.rows_per_unit, T.S - row0);
         int carry = 0;
         for (int r = 0; r < nrows; r += groups) {
             const int now = min(groups, nrows - r);
             const bool more = r + groups < nrows;
-            short_step<DIRECT>(a, T, sm, lg, row0 + r, now, more, carry, st, ev);
+            short_step<BY>(a, T, sm, lg, row0 + r, now, more, carry, st, ev);
         }
     }
     rows_done(a, st, ev);

@@ -251,3 +251,38 @@ def test_dual_search_at_the_ends_of_binary32(bits1, bits2, signed, exponent):
     assert np.array_equal(idx, ref.best_idx) and np.array_equal(alpha, ref.alpha)
     assert np.array_equal(q.reshape(2, 3, 600), ref.codes)
     np.testing.assert_allclose(sse, ref.sse.astype(np.float32), rtol=1e-5, atol=1e-37)
+
+
+@pytest.mark.parametrize("s,k,bits,signed,n_cand,hi_frac,kind", [
+    (2101, 400, 4, True, 1024, 1.0, "student"),       # the shortest rows of that path, the finest fractions
+    (1501, 1023, 4, True, 1024, 1.0, "extremes"),     # ten bits for the count, eleven from here on
+    (1501, 1024, 4, False, 1000, 1.0, "student"),
+    (1301, 1280, 5, True, 256, 1.0, "extremes"),
+    (2401, 1281, 4, True, 500, 1.3, "student"),       # longer than a warp's registers hold; a grid beyond max|x|
+    (2401, 2047, 8, True, 1024, 1.0, "extremes"),
+    (2401, 2048, 4, True, 1024, 1.0, "extremes"),     # twelve bits for the count: the coarsest fractions
+    (2371, 2304, 4, True, 1023, 1.0, "repeats"),      # a whole row in a few bins
+    (2371, 2303, 8, False, 200, 1.0, "repeats"),
+    (2101, 700, 8, True, 17, 1.0, "student"),         # fewer candidates than are looked at first
+    (2101, 641, 4, True, 1024, 1.0, "scaled"),        # squares beyond binary32: a candidate per lane
+    (2101, 640, 3, False, 1024, 1.0, "repeats"),
+    (1301, 1280, 3, True, 1024, 1.0, "extremes"),     # fewer bits: by splits, and a block per row beyond
+    (1301, 1281, 3, True, 1024, 1.0, "extremes"),
+])
+def test_rows_by_a_histogram_of_their_warp(s, k, bits, signed, n_cand, hi_frac, kind):
+    import gpu_util
+    w = synth.student_t3(s * k, seed=78, tensor_id=k).reshape(s, k)
+    if kind == "extremes":                            # one value far above the others, of either sign: candidates all over the grid are open
+        at = np.arange(0, s, 2)
+        w[at, at % k] = np.where(at % 4 == 0, 1.0, -1.0).astype(np.float32) * np.float32(30.0) * (1.0 + at % 7).astype(np.float32)
+    elif kind == "repeats":                           # all values on a lattice: thresholds meet them exactly
+        w = np.clip(np.round(w * np.float32(2)), -9, 9).astype(np.float32) * np.float32(0.125)
+        w[::5] = np.sign(w[::5]) * np.float32(0.25)   # one magnitude (and zeros)
+    elif kind == "scaled":
+        w = w * np.float32(2.0 ** 60)
+    if not signed:
+        w = np.abs(w)
+    alpha, sse, idx, q, pk = gpu_util.quantize_weights(w, bits, signed, n_cand, hi_frac, 3, True, bits <= 4)
+    rows = np.unique(np.concatenate([np.arange(0, s, 41), np.arange(0, s, 130), [s - 2, s - 1]]))
+    st = check_rows(w, alpha, sse, idx, q, None, bits, signed, n_cand, hi_frac, 3, rows=rows)
+    assert st["idx_diff"] <= max(1, st["rows"] // 50) and st["alpha_bitwise"] >= 0.99, st
