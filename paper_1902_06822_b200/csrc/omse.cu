@@ -505,9 +505,11 @@ int quantize_list(omse_ctx* ctx, std::vector<omse::RowTensor>& list, int bits, i
     // 40 and 33; 2400 rows of 288 values 29 and 33, 10,000 75 and 70; 1200 rows of 576 values 34 and 31); 8 bits, whose
     // best scale lies where the splits have furthest to go, change over later (10,000 rows of 27 values 41 and 52).
     const bool plain = mode.solver == 0 && mode.n_delta == 0;   // the block path implements everything else
-    long long short_rows = 0, short_elements = 0, short_warps = 0;
+    long long short_rows = 0, short_elements = 0, short_warps = 0, long_rows = 0;
     for (const auto& t : list)
-        if (t.K <= kSmallK) {
+        if (t.K > kSmallK && t.K <= kHistMaxK) {
+            long_rows += t.S;
+        } else if (t.K <= kSmallK) {
             short_rows += t.S;
             short_elements += t.S * t.K;
             short_warps += (t.S << omse::short_lanes(t.K)) / 32;
@@ -517,7 +519,7 @@ int quantize_list(omse_ctx* ctx, std::vector<omse::RowTensor>& list, int bits, i
     int spread = 0;                                             // more lanes per row where the warps do not fill the GPU
     while (spread < 5 && (short_warps << (spread + 1)) <= 16ll * ctx->n_sm) ++spread;
     std::vector<int> path_of(list.size(), kPathBlock);
-    // Rows by a histogram of their warp; beyond kSmallK values where there are a few for every warp of the GPU.
+    // Rows by a histogram of their warp.
     a.n_bins = all_bins(a.n_cand, a.hi_frac);
     a.hist_lb = 4;
     while (a.hist_lb < 6 && (32 << a.hist_lb) < a.n_bins) ++a.hist_lb;
@@ -525,19 +527,21 @@ int quantize_list(omse_ctx* ctx, std::vector<omse::RowTensor>& list, int bits, i
     // (the largest |x|/h, rounded up to a fraction, lies in a bin)
     const bool hist_fits = plain && a.hi[0] >= 7 && a.n_bins > 0 &&
                            2.0 * a.n_cand / (double)a.hi_frac * (1.0 + 4e-7) + 1.0 / 64 < (double)hist_words + 1.0;
-    const long long hist_k = a.hi[0] > 15 ? kHistK8 : kHistK4;
-    long long long_rows = 0;
-    for (const auto& t : list)
-        if (t.K > kSmallK && t.K <= kHistMaxK) long_rows += t.S;
-    const bool hist_long = hist_fits && long_rows + short_rows >= 16ll * ctx->n_sm && (short_rows == 0 || !a.short_direct);
-    if (hist_long && short_rows == 0) a.short_direct = 0;
+    // A row takes a warp 15 to 30 us, a block a third of that: with fewer rows than this blocks are sooner done (600 rows of 576 values
+    // 22 us by blocks and 18.5, 300 rows 19 and 18.5; 600 of 1024 values 22 and 22.6, 1180 35 and 25; 600 of 2304 28 and 37, 1180 43
+    // and 40).  Beside rows of other paths the launch has to be worth its cost.
+    long long hist_from = a.hi[0] > 15 ? kHistK8 : kHistK4, hist_to = kHistMaxK, hist_elements = 0, other_elements = 0;
+    if (short_rows + long_rows < 7ll * ctx->n_sm) hist_to = 800;
+    if (!hist_fits || short_rows + long_rows < 4ll * ctx->n_sm) hist_to = 0;
+    for (const auto& t : list) (t.K >= hist_from && t.K <= hist_to ? hist_elements : other_elements) += t.S * t.K;
+    if (other_elements > 0 && hist_elements < 1 << 21) hist_to = 0;
     // One launch per row path present in the list: each launch then runs the kernel instantiation that holds only its path.
     // Longest rows first inside a launch: the dispenser hands out work in decreasing size and the tail is short.
     std::stable_sort(list.begin(), list.end(), [](const omse::RowTensor& x, const omse::RowTensor& y) { return x.K > y.K; });
     bool present[kPaths] = {};
     for (size_t i = 0; i < list.size(); ++i) {
         omse::RowTensor& t = list[i];
-        if (hist_fits && !a.short_direct && t.K >= hist_k && t.K <= (hist_long ? kHistMaxK : short_k)) {
+        if (t.K >= hist_from && t.K <= hist_to) {
             // count and fractions of all values in one word, bin and fraction in 23 bits
             int count = 1, frac = 1;
             while ((1ll << count) <= t.K) ++count;

@@ -78,6 +78,18 @@ __device__ __forceinline__ int exact_code(float x, float alpha, float inv, float
 __device__ __forceinline__ float ambiguity_threshold(float flo, float fhi) {
     return 0.5f - (fmaxf(fhi, -flo) + 2.0f) * 4.76837158203125e-7f;
 }
+// Four codes at once: one branch for the rare division instead of four.
+__device__ __forceinline__ void exact_codes4(const float (&x)[4], float alpha, float inv, float flo, float fhi, float amb_thr,
+                                             int (&q)[4]) {
+    bool amb[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) q[e] = magic_int(magic_code(x[e], inv, kMagic + flo, kMagic + fhi, amb_thr, amb[e]));
+    if (amb[0] || amb[1] || amb[2] || amb[3]) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (amb[e]) q[e] = code_of(x[e], alpha, flo, fhi);
+    }
+}
 // M + q (q an integer above -2^22) as a double that holds q: the bits are the low word of a double in [2^52, 2^53).
 __device__ __forceinline__ double magic_double(float tc) {
     return __hiloint2double(0x43300000, __float_as_int(tc)) - (4503599627370496.0 + 1262485504.0);   // 2^52 + the bits of M, exact
@@ -89,7 +101,7 @@ __device__ __forceinline__ float max3_nan(float a, float b, float c) {     // Na
 }
 // The codes of four values at a scale, as M + code: those of code_of, by the argument at magic_code, with one branch for the rare
 // divisions; in packed arithmetic and with one test (a pass over rows in shared memory, 24 warps per SM: 5.9 clocks per 32 values
-// with four separate codes, 4.8 so).
+// with exact_codes4, 4.8 so; in the rolled loops over a few values per lane that short rows have, it costs 1 % more than it saves).
 struct Coder {
     u64 inv2;
     float alpha, flo, fhi, thr;
@@ -111,21 +123,6 @@ struct Coder {
 #pragma unroll
             for (int e = 0; e < 4; ++e)
                 if (!(fabsf(d[e]) <= thr)) t[e] = kMagic + (float)code_of(x[e], alpha, flo, fhi);
-        }
-    }
-    // the same a value at a time: in the rolled loops over a few values per lane that short rows have, packing costs 1 % more than it
-    // saves (131,072 rows of 512 values on 8 bits 1130 us, 1147 packed)
-    __device__ __forceinline__ void of_single(const float4& v, float (&t)[4]) const {
-        const float x[4] = {v.x, v.y, v.z, v.w};
-        float inv, unused;
-        unpack2(inv2, inv, unused);
-        bool amb[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) t[e] = magic_code(x[e], inv, kMagic + flo, kMagic + fhi, thr, amb[e]);
-        if (amb[0] || amb[1] || amb[2] || amb[3]) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-                if (amb[e]) t[e] = kMagic + (float)code_of(x[e], alpha, flo, fhi);
         }
     }
 };

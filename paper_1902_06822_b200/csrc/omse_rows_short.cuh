@@ -707,11 +707,7 @@ __device__ __forceinline__ void short_step(const RowArgs& a, const RowTensor& T,
     const long long row = row0 + r.g, flat0 = row0 * T.K;
     r.flo = (float)a.lo[0];
     r.fhi = (float)a.hi[0];
-    const float flo = r.flo, fhi = r.fhi;
-    auto codes = [](const Coder& coder, const float4& v, float (&t)[4]) {
-        if (BY == kBySplits) coder.of_single(v, t);
-        else coder.of(v, t);
-    };
+    const float flo = r.flo, fhi = r.fhi, thr = ambiguity_threshold(flo, fhi);
 
     // ---- the rows into shared memory
     __syncwarp();                                        // the previous step's rows and codes have been read
@@ -753,16 +749,16 @@ __device__ __forceinline__ void short_step(const RowArgs& a, const RowTensor& T,
             for (int u = 4 * i; u < min(4 * i + 4, k); ++u) reinterpret_cast<float*>(mine)[u] = y[u] - off;
         if (active && r.j == 0) T.delta[row] = off;
     } else if (T.prior_alpha) {                          // second tensor of a key layer: the residual of the first one
-        const float a1 = active ? T.prior_alpha[row] : 0.f;
-        const Coder coder(a1, a1 > 0.f ? __fdiv_rn(1.0f, a1) : 0.f, flo, fhi);
+        const float a1 = active ? T.prior_alpha[row] : 0.f, inv = a1 > 0.f ? __fdiv_rn(1.0f, a1) : 0.f;
         if (a1 > 0.f)
 #pragma unroll 1
             for (int i = r.j; i < own; i += 1 << lg) {
                 const float4 v = mine[i];
-                float t[4];
-                codes(coder, v, t);
-                mine[i] = make_float4(fmaf(-a1, t[0] - kMagic, v.x), fmaf(-a1, t[1] - kMagic, v.y),
-                                      fmaf(-a1, t[2] - kMagic, v.z), fmaf(-a1, t[3] - kMagic, v.w));
+                const float y[4] = {v.x, v.y, v.z, v.w};
+                int q[4];
+                exact_codes4(y, a1, inv, flo, fhi, thr, q);
+                mine[i] = make_float4(fmaf(-a1, (float)q[0], y[0]), fmaf(-a1, (float)q[1], y[1]),
+                                      fmaf(-a1, (float)q[2], y[2]), fmaf(-a1, (float)q[3], y[3]));
             }
     }
     // ---- maxima and sums; a power of two against overflow and underflow of the squares
@@ -837,8 +833,7 @@ __device__ __forceinline__ void short_step(const RowArgs& a, const RowTensor& T,
         for (int i = 0; __any_sync(0xffffffffu, open); ++i) {
             float a1 = s.w_lo + (float)i;
             if (open && listed) a1 = (float)sm.close[(i << (5 - lg)) + r.g];
-            const float ac = __fmul_rn(a1, r.step);
-            const Coder coder(ac, __fdiv_rn(1.0f, ac), flo, fhi);
+            const float ac = __fmul_rn(a1, r.step), inv = __fdiv_rn(1.0f, ac);
             const double ad = (double)ac;
             double ss = 0.0;
             const bool ok = open && usable_scale(ac);
@@ -846,11 +841,11 @@ __device__ __forceinline__ void short_step(const RowArgs& a, const RowTensor& T,
             for (int q4 = r.j; q4 < (ok ? own : 0); q4 += 1 << lg) {    // the padding zeros code to 0 and add nothing
                 const float4 v = mine[q4];
                 const float y[4] = {v.x, v.y, v.z, v.w};
-                float t[4];
-                codes(coder, v, t);
+                int q[4];
+                exact_codes4(y, ac, inv, flo, fhi, thr, q);
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    const double d = fma(-ad, magic_double(t[u]), (double)y[u]);
+                    const double d = fma(-ad, int_double(q[u]), (double)y[u]);
                     ss = fma(d, d, ss);
                 }
             }
@@ -873,22 +868,23 @@ __device__ __forceinline__ void short_step(const RowArgs& a, const RowTensor& T,
     {
         bool open = found;
         for (int it = 0; it < a.refine_iters && __any_sync(0xffffffffu, open); ++it) {
-            const Coder coder(alpha, found ? __frcp_rn(alpha) : 0.f, flo, fhi);
+            const float inv = found ? __frcp_rn(alpha) : 0.f;
             double sxq = 0.0;
-            u64 qa = 0ull, qb = 0ull;
+            int sqq = 0;
 #pragma unroll 1
             for (int q4 = r.j; q4 < (open ? own : 0); q4 += 1 << lg) {
                 const float4 v = mine[q4];
                 const float y[4] = {v.x, v.y, v.z, v.w};
-                float t[4];
-                codes(coder, v, t);
-                qa = add_squares(t[0], t[1], qa);        // (18 steps at most: see there)
-                qb = add_squares(t[2], t[3], qb);
+                int q[4];
+                exact_codes4(y, alpha, inv, flo, fhi, thr, q);
 #pragma unroll
-                for (int u = 0; u < 4; ++u) sxq = fma((double)y[u], magic_double(t[u]), sxq);
+                for (int u = 0; u < 4; ++u) {
+                    sqq += q[u] * q[u];
+                    sxq = fma((double)y[u], int_double(q[u]), sxq);
+                }
             }
             sxq = group_sum(sxq, lg);
-            const int sqq = group_sum((int)squares_of(qa, qb), lg);
+            sqq = group_sum(sqq, lg);
             const float a_new = (float)(sxq / (double)sqq);
             open = open && sqq != 0 && a_new >= FLT_MIN && a_new <= FLT_MAX && a_new != alpha;   // a fixed point would repeat exactly
             if (open) alpha = a_new;
@@ -898,27 +894,28 @@ __device__ __forceinline__ void short_step(const RowArgs& a, const RowTensor& T,
     const int o = (int)(flat0 & 7);
     signed char* qs = sm.qs;
     {
-        const Coder coder(alpha, alpha > 0.f ? __fdiv_rn(1.0f, alpha) : 0.f, flo, fhi);
+        const float inv = alpha > 0.f ? __fdiv_rn(1.0f, alpha) : 0.f;
         const double ad = (double)alpha;
         double ss = 0.0;
 #pragma unroll 1
         for (int q4 = r.j; q4 < own; q4 += 1 << lg) {
             const float4 v = mine[q4];
             const float y[4] = {v.x, v.y, v.z, v.w};
-            float t[4] = {kMagic, kMagic, kMagic, kMagic};
-            if (alpha > 0.f) codes(coder, v, t);
+            int q[4] = {0, 0, 0, 0};
+            if (alpha > 0.f) exact_codes4(y, alpha, inv, flo, fhi, thr, q);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const double d = fma(-ad, magic_double(t[u]), (double)y[u]);
+                const double d = fma(-ad, int_double(q[u]), (double)y[u]);
                 ss = fma(d, d, ss);
             }
             signed char* dst = qs + o + r.g * k + 4 * q4;
             if ((k & 3) == 0) {
-                *reinterpret_cast<unsigned int*>(dst) = code_bytes(t);
+                *reinterpret_cast<unsigned int*>(dst) =
+                    (q[0] & 0xff) | ((q[1] & 0xff) << 8) | ((q[2] & 0xff) << 16) | ((unsigned)(q[3] & 0xff) << 24);
             } else {
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
-                    if (4 * q4 + u < k) dst[u] = (signed char)magic_int(t[u]);
+                    if (4 * q4 + u < k) dst[u] = (signed char)q[u];
             }
         }
         ss = group_sum(ss, lg);
@@ -951,7 +948,8 @@ __device__ __forceinline__ void short_step(const RowArgs& a, const RowTensor& T,
         for (int b = b0 + lane; b < from; b += 32) dst[b] = byte_of(b);
         for (int b = from + 4 * lane; b < to; b += 128) {
             const uint2 u = *reinterpret_cast<const uint2*>(qs + 2 * b);
-            *reinterpret_cast<unsigned int*>(dst + b) = __byte_perm(byte_nibbles(u.x), byte_nibbles(u.y), 0x5410);
+            auto nibbles = [](unsigned int v) { return (v & 0xfu) | ((v >> 4) & 0xf0u) | ((v >> 8) & 0xf00u) | ((v >> 12) & 0xf000u); };
+            *reinterpret_cast<unsigned int*>(dst + b) = nibbles(u.x) | (nibbles(u.y) << 16);
         }
         if (to + lane < b1) dst[to + lane] = byte_of(to + lane);
         carry = qs[end - 1];

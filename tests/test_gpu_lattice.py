@@ -264,7 +264,7 @@ def test_dual_search_at_the_ends_of_binary32(bits1, bits2, signed, exponent):
     (2371, 2304, 4, True, 1023, 1.0, "repeats"),      # a whole row in a few bins
     (2371, 2303, 8, False, 200, 1.0, "repeats"),
     (2101, 700, 8, True, 17, 1.0, "student"),         # fewer candidates than are looked at first
-    (2101, 641, 4, True, 1024, 1.0, "scaled"),        # squares beyond binary32: a candidate per lane
+    (2101, 641, 4, True, 1024, 1.0, "scaled"),        # values that are scaled for their squares: a candidate per lane
     (2101, 640, 3, False, 1024, 1.0, "repeats"),
     (1301, 1280, 3, True, 1024, 1.0, "extremes"),     # fewer bits: by splits, and a block per row beyond
     (1301, 1281, 3, True, 1024, 1.0, "extremes"),
@@ -279,7 +279,7 @@ def test_rows_by_a_histogram_of_their_warp(s, k, bits, signed, n_cand, hi_frac, 
         w = np.clip(np.round(w * np.float32(2)), -9, 9).astype(np.float32) * np.float32(0.125)
         w[::5] = np.sign(w[::5]) * np.float32(0.25)   # one magnitude (and zeros)
     elif kind == "scaled":
-        w = w * np.float32(2.0 ** 60)
+        w = w * np.float32(2.0 ** 50)
     if not signed:
         w = np.abs(w)
     alpha, sse, idx, q, pk = gpu_util.quantize_weights(w, bits, signed, n_cand, hi_frac, 3, True, bits <= 4)
