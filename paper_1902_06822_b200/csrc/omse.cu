@@ -1072,7 +1072,7 @@ int omse_dual_quantize(omse_ctx* ctx, const float* d_t, int64_t n_kernels, int64
     long long blocks = (long long)ctx->n_sm * occ;
     if (blocks > n_units) blocks = n_units;
     // the context workspace holds the sorted points of every alpha2, then each block's grid values of its current row
-    const size_t point_bytes = bound ? (size_t)grid->n_cand2 * (omse::kDualPoints * sizeof(omse::DualPoint) + 16) : 0;
+    const size_t point_bytes = bound ? (size_t)grid->n_cand2 * 2 * omse::kDualSide * sizeof(omse::DualPoint) : 0;
     const long long cap = (long long)((kPartialBytes - point_bytes) / ((size_t)grid->n_cand1 * grid->n_cand2 * 4));
     if (blocks > cap) blocks = cap;
     if (blocks < 1) return OMSE_EINVAL;
@@ -1080,10 +1080,9 @@ int omse_dual_quantize(omse_ctx* ctx, const float* d_t, int64_t n_kernels, int64
     a.evals = &ctx->ws->evals;
     if (bound) {
         omse::DualPoint* points = reinterpret_cast<omse::DualPoint*>(ctx->partials);
-        int* counts = reinterpret_cast<int*>(points + (size_t)grid->n_cand2 * omse::kDualPoints);
-        omse::dual_points_kernel<<<(unsigned)grid->n_cand2, omse::kDualPoints, 0, ctx->stream>>>(
-            points, counts, grid->n_cand2, grid->hi_frac2, a.lo1, a.hi1, a.lo2, a.hi2);
-        const omse::DualPoints pts = {points, counts};
+        omse::dual_points_kernel<<<(unsigned)grid->n_cand2, omse::kDualPoints, 0, ctx->stream>>>(points, grid->n_cand2, grid->hi_frac2, a.lo1,
+                                                                                                 a.hi1, a.lo2, a.hi2);
+        const omse::DualPoints pts = {points};
         if (few) omse::dual_bound_kernel<3><<<(unsigned)blocks, threads, smem, ctx->stream>>>(a, pts);
         else omse::dual_bound_kernel<4><<<(unsigned)blocks, threads, smem, ctx->stream>>>(a, pts);
         ctx->n_launches += 2;

@@ -323,66 +323,65 @@ __global__ void __launch_bounds__(kDualThreads) dual_kernel(const DualArgs a) {
 // within n*width*f*(1-f) below the chord, f being the position in the bin.  That gives an estimate of every pair's error and
 // a bound of its distance from the truth: pairs whose lower bound is above the smallest upper bound are out.  One or two
 // of 1024 pairs are left, and those are re-scored in the reference arithmetic if there is more than one.
-// Bound: instruction issue, some 60 warp instructions a pair whatever the row's length, where the sweep above takes
-// K*(first codes)/4 of them: this path is for rows of at least OMSE_DUAL_BOUND_K values, sorted point sets of at most
-// kDualPoints and rho <= 1.  512 rows of 4608 values, 4 bits twice, 32 x 32 pairs on one B200: 3.62 ms -> 187 us, 16 such
-// rows 1636 -> 78 us, 148 rows of 256 values 101 -> 57 us.
+// Bound: chains of look-ups, four points of a pair at a time, and in the re-scores and codes instruction issue.  The sweep above takes
+// K*(first codes)/4 warp instructions a pair, this whatever the row's length: it is for rows of at least OMSE_DUAL_BOUND_K values,
+// sorted point sets of at most kDualPoints and rho <= 1.  512 rows of 4608 values, 4 bits twice, 32 x 32 pairs on one B200: 3.62 ms ->
+// 164 us (191 with 16-byte points and bins in binary64, every lane's end tested, five first codes per value), 16 such rows 1636 -> 70
+// us, 16 rows of 300 values 57 -> 49.
 // -------------------------------------------------------------------------------------------------
 constexpr int kDualPoints = 256;
+constexpr int kDualSide = 264;         // entries of a side: at most 255 midpoints, then ends (four are read ahead)
 constexpr int kDualBins = 1024;        // per side; every value lies below bin kDualBins - 1
 constexpr int kDualBoundThreads = 256;
 
-struct __align__(16) DualPoint {       // one midpoint, in units of alpha1
-    double gap;
-    float mid, gap_f;
+struct DualPoint {                     // one midpoint and its gap, in units of alpha1
+    float mid, gap;
 };
 struct DualPoints {
-    const DualPoint* p;                // [n_cand2][kDualPoints], outwards from 0: positive side, then negative side
-    const int* n;                      // [n_cand2][2]
+    const DualPoint* p;                // [n_cand2][2][kDualSide], outwards from 0: positive side, then negative side
 };
 struct __align__(16) DualBin {
     union {
         struct { unsigned int n, f, pad0, pad1; } h;     // while inserting: values, sum of their fractional parts
-        struct { double r; float dr, half; } v;          // R at the lower edge, its fall over the bin, half of n
+        struct { float r, dr, half, pad; } v;            // R at the lower edge, its fall over the bin, half of n
     };
 };
 
-__global__ void __launch_bounds__(kDualPoints) dual_points_kernel(DualPoint* out, int* n_out, int n_cand2, float hi_frac2, int lo1,
-                                                                  int hi1, int lo2, int hi2) {
+__global__ void __launch_bounds__(kDualPoints) dual_points_kernel(DualPoint* out, int n_cand2, float hi_frac2, int lo1, int hi1, int lo2, int hi2) {
     __shared__ double pts[kDualPoints], sorted[kDualPoints];
     const int i = threadIdx.x, d = blockIdx.x, l2 = hi2 - lo2 + 1, n = (hi1 - lo1 + 1) * l2;
     const double rho = (double)(d + 1) * (double)hi_frac2 / (double)n_cand2;
     const double p = (double)(lo1 + i / l2) + rho * (double)(lo2 + i % l2);
     if (i < n) pts[i] = p;
     __syncthreads();
-    int below = 0;
     if (i < n) {
         int rank = 0;
         for (int j = 0; j < n; ++j) rank += pts[j] < p || (pts[j] == p && j < i);
         sorted[rank] = p;
     }
-    below = __syncthreads_count(i < n && p < 0.0);          // the first zero: t = q = 0 is always a point
+    const int below = __syncthreads_count(i < n && p < 0.0);          // the first zero: t = q = 0 is always a point
+    DualPoint* side[2] = {out + (size_t)2 * d * kDualSide, out + (size_t)(2 * d + 1) * kDualSide};
     if (i + 1 < n) {
         const bool neg = i < below;
-        DualPoint e;
-        e.gap = sorted[i + 1] - sorted[i];
-        e.mid = (float)(0.5 * (sorted[i] + sorted[i + 1]) * (neg ? -1.0 : 1.0));
-        e.gap_f = (float)e.gap;
-        out[(size_t)d * kDualPoints + (neg ? n - 2 - i : i - below)] = e;
+        const DualPoint e = {(float)(0.5 * (sorted[i] + sorted[i + 1]) * (neg ? -1.0 : 1.0)), (float)(sorted[i + 1] - sorted[i])};
+        side[neg][neg ? below - 1 - i : i - below] = e;
     }
-    if (i == 0) {
-        n_out[2 * d] = n - 1 - below;
-        n_out[2 * d + 1] = below;
-    }
+    for (int k = n - 1 - below + i; k < kDualSide; k += kDualPoints) side[0][k] = DualPoint{1e9f, 0.f};       // beyond every value
+    for (int k = below + i; k < kDualSide; k += kDualPoints) side[1][k] = DualPoint{1e9f, 0.f};
 }
 
 // The reference's codes of one element: the first codes that can win (see the window of dual_kernel), lowest first code on
 // equal binary32 errors, codes equal to those of the IEEE division.
+// Two first codes at a time in packed arithmetic.  Where some first code leaves a rest that does not saturate the second one, only
+// those can win (the others err by more than alpha2/2): their range is narrower than the window, 3 codes instead of 5 at alpha2 =
+// 0.19*alpha1 on 4 bits twice.
 struct DualCodes {
-    float a1, a2, inv1, inv2, w, flo1, fhi1, flo2, fhi2, thr;
-    __device__ __forceinline__ void set(float a1_, float a2_, const DualArgs& a, bool every) {
+    float a1, a2, inv1, inv2, w, flo1, fhi1, flo2, fhi2, thr, up, down;
+    bool every;
+    __device__ __forceinline__ void set(float a1_, float a2_, const DualArgs& a, bool every_) {
         a1 = a1_;
         a2 = a2_;
+        every = every_;
         inv1 = a1 > 0.f ? __fdiv_rn(1.0f, a1) : 0.f;
         inv2 = a2 > 0.f ? __fdiv_rn(1.0f, a2) : 0.f;
         flo1 = (float)a.lo1;
@@ -390,31 +389,61 @@ struct DualCodes {
         flo2 = (float)a.lo2;
         fhi2 = (float)a.hi2;
         thr = ambiguity_threshold(flo2, fhi2);
-        w = (float)max(1, (int)((fmaxf(fhi2, -flo2) + 0.5f) * fminf(a2 * inv1, 16.f) * 1.0001f + 0.501f));
-        if (every) w = 512.f;
+        const float ratio = fminf(a2 * inv1, 16.f);
+        w = (float)max(1, (int)((fmaxf(fhi2, -flo2) + 0.5f) * ratio * 1.0001f + 0.501f));
+        up = (0.5f - flo2) * ratio + 1e-3f;                  // rests from (lo2 - 1/2)*alpha2 to (hi2 + 1/2)*alpha2, and a margin that
+        down = (fhi2 + 0.5f) * ratio + 1e-3f;                // binary32 does not reach
     }
-    __device__ __forceinline__ void of(float x, int& t_out, int& q_out) const {
-        const float c = rintf(x * inv1);
-        const float t0 = fminf(fmaxf(c - w, flo1), fhi1), t1 = fminf(fmaxf(c + w, flo1), fhi1);
-        float best = INFINITY;
-        int bt = (int)flo1, bq = 0;
-        for (float t = t0; t <= t1; t += 1.0f) {
-            const float r = fmaf(-a1, t, x);
-            const int q = exact_code(r, a2, inv2, flo2, fhi2, thr);
-            const float e = fmaf(-a2, (float)q, r), ee = __fmul_rn(e, e);
-            if (ee < best) {
-                best = ee;
-                bt = (int)t;
-                bq = q;
+    // codes as M + code
+    __device__ __forceinline__ void of(float x, float& t_out, float& q_out) const {
+        const float c = x * inv1, near = rintf(c);
+        float t0 = fmaxf(ceilf(c - down), flo1), t1 = fminf(floorf(c + up), fhi1);
+        // (none, or none for sure: all rests may saturate)
+        if (!(fmaxf(ceilf(c - down + 2e-3f), flo1) <= fminf(floorf(c + up - 2e-3f), fhi1)) || !(fabsf(c) < 4096.f)) {
+            t0 = fminf(fmaxf(near - w, flo1), fhi1);
+            t1 = fminf(fmaxf(near + w, flo1), fhi1);
+        }
+        if (every) {
+            t0 = flo1;
+            t1 = fhi1;
+        }
+        float best = INFINITY, bt = flo1, bq = kMagic;
+        const u64 na1 = pack2(-a1, -a1), na2 = pack2(-a2, -a2), i2 = pack2(inv2, inv2), M2 = pack2(kMagic, kMagic), NM2 = pack2(-kMagic, -kMagic),
+                  minus = pack2(-1.f, -1.f), x2 = pack2(x, x), z2 = pack2(-0.f, -0.f);
+        const float clo = kMagic + flo2, chi = kMagic + fhi2;
+        for (float t = t0; t <= t1; t += 2.0f) {
+            const u64 r = fma2(na1, pack2(t, t + 1.0f), x2), u = fma2(r, i2, M2);
+            float d0, d1, q0, q1, e0, e1;
+            unpack2(fma2(r, i2, fma2(u, minus, M2)), d0, d1);
+            unpack2(u, q0, q1);
+            q0 = fminf(fmaxf(q0, clo), chi);
+            q1 = fminf(fmaxf(q1, clo), chi);
+            if (!(max3_nan(fabsf(d0), fabsf(d1), 0.f) <= thr)) {
+                float r0, r1;
+                unpack2(r, r0, r1);
+                if (!(fabsf(d0) <= thr)) q0 = kMagic + (float)code_of(r0, a2, flo2, fhi2);
+                if (!(fabsf(d1) <= thr)) q1 = kMagic + (float)code_of(r1, a2, flo2, fhi2);
+            }
+            const u64 e = fma2(na2, add2(pack2(q0, q1), NM2), r);
+            unpack2(fma2(e, e, z2), e0, e1);
+            if (e0 < best) {
+                best = e0;
+                bt = t;
+                bq = q0;
+            }
+            if (e1 < best && t + 1.0f <= t1) {
+                best = e1;
+                bt = t + 1.0f;
+                bq = q1;
             }
         }
-        t_out = bt;
+        t_out = kMagic + bt;
         q_out = bq;
     }
 };
 
 // BLOCKS: blocks per SM that the registers are cut for.  Four hide more latency where there are rows for them (512 rows of
-// 4608 values 190 us, 203 with three); with up to three rows per SM the wider schedule is faster (16 such rows 78 us, 98).
+// 4608 values 164 us); with up to three rows per SM the wider schedule is faster (16 such rows 70 us).
 template <int BLOCKS>
 __global__ void __launch_bounds__(kDualBoundThreads, BLOCKS) dual_bound_kernel(const DualArgs a, const DualPoints pts) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -423,7 +452,8 @@ __global__ void __launch_bounds__(kDualBoundThreads, BLOCKS) dual_bound_kernel(c
     __shared__ double scratch[64];
     __shared__ double s_sums[2][kDualBoundThreads / 32];
     __shared__ unsigned int s_part[3][kDualBoundThreads / 32];
-    __shared__ int s_list[kDualListCap], s_n, s_carry[2];
+    __shared__ int s_list[kDualListCap], s_n;
+    __shared__ float s_carry[2];
     const int tid = threadIdx.x, nthr = kDualBoundThreads, lane = tid & 31, warp = tid >> 5, nwarp = kDualBoundThreads / 32;
     const int k = (int)a.K;
     const long long n_total = a.S * a.K, packed_stride = (n_total + 1) >> 1, n_units = (a.S + a.rows_per_unit - 1) / a.rows_per_unit;
@@ -552,7 +582,7 @@ __global__ void __launch_bounds__(kDualBoundThreads, BLOCKS) dual_bound_kernel(c
                     x.n += hn[i];
                     x.f += hf[i];
                     const double r = fma((double)x.f, fq, (double)x.s);
-                    mine[i].v.r = r;
+                    mine[i].v.r = (float)r;
                     mine[i].v.dr = (float)(r - above);
                     mine[i].v.half = 0.5f * (float)hn[i];
                     above = r;
@@ -564,18 +594,20 @@ __global__ void __launch_bounds__(kDualBoundThreads, BLOCKS) dual_bound_kernel(c
                     ls += s_sums[1][v];
                 }
                 __syncthreads();
-                // ---- estimate and bounds of every pair.  What the fixed point (ls), binary32 in the bounds and the scales'
-                //      own rounding (es, the estimate) can add is in the margin.
+                // ---- estimate and bounds of every pair.  What the fixed point (ls) and binary32 in the sums and bounds, the midpoints and
+                //      the scales can add (es: 2*unit*acc is at most es, and each of its terms is off by six roundings) is in the margin.
                 const float scale_pre = pre;
                 const double w_true = (double)w / (double)scale_pre;
-                const double margin0 = 2e-7 * es + ls * w_true * fq + 3e-45 * (double)k;
+                const double margin0 = 1e-6 * es + ls * w_true * fq + 3e-45 * (double)k;
                 inv_es = 1.0 / es;
                 const float inv_w = __fdiv_rn(1.0f, w);
                 // A warp takes 8 neighbouring alpha1 of 4 neighbouring ratios at a time: lanes of similar alpha1 have about as
                 // many midpoints below max|x|, a lane keeps its own sums, and the points of a ratio are read by 8 lanes at once.
-                const int n_dq = (a.n_cand2 + 3) >> 2, n_task = n_dq * ((a.n_cand1 + 7) >> 3);
+                // The warps go through all alpha1 of a few ratios before the next ones: L1 holds the points of that many.
+                const int n_dq = (a.n_cand2 + 3) >> 2, n_cb = (a.n_cand1 + 7) >> 3, n_task = n_dq * n_cb;
                 for (int task = warp; task < n_task; task += nwarp) {
-                    const int cb = task / n_dq, d = 4 * (task - cb * n_dq) + (lane >> 3), c = 8 * cb + (lane & 7);
+                    // (small alpha1 have the most midpoints: which of them a warp takes changes from ratio to ratio)
+                    const int dq = task / n_cb, cb = (task + dq * n_cb / nwarp) % n_cb, d = 4 * dq + (lane >> 3), c = 8 * cb + (lane & 7);
                     const bool valid = d < a.n_cand2 && c < a.n_cand1;
                     const int dv = min(d, a.n_cand2 - 1);
                     float a1, a2;
@@ -583,51 +615,39 @@ __global__ void __launch_bounds__(kDualBoundThreads, BLOCKS) dual_bound_kernel(c
                     const bool ok = a1 >= FLT_MIN && a2 >= FLT_MIN;
                     const float s = (a1 * scale_pre) * inv_w;                // alpha1 in bins
                     double acc = 0.0;
-                    float lin = 0.f, wid = 0.f;
+                    float wid = 0.f;
 #pragma unroll 1
                     for (int side = 0; side < 2; ++side) {
-                        const int from = side ? __ldg(pts.n + 2 * dv) : 0, n = __ldg(pts.n + 2 * dv + side);
-                        const uint4* tab = reinterpret_cast<const uint4*>(pts.p + (size_t)dv * kDualPoints) + from;
-                        // (what is read beyond n is not used; kDualPoints + 8 entries behind the last table are the workspace's)
+                        const float4* tab = reinterpret_cast<const float4*>(pts.p + (size_t)(2 * dv + side) * kDualSide);
                         const DualBin* bs = bins + side * kDualBins;
-                        bool go = valid && n > 0;
-                        uint4 next[4];                               // the next four points are on their way meanwhile
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) next[j] = __ldg(tab + j);
-                        for (int k0 = 0; __any_sync(0xffffffffu, go); k0 += 4) {
-                            uint4 raw[4], bin[4];
-                            float f[4];
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) raw[j] = next[j];
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) next[j] = __ldg(tab + k0 + 4 + j);
-                            // no branch, so that the four reads of the bins are in flight together: a point outside takes
-                            // part with gap 0
+                        constexpr float kEnd = kMagic + (float)(kDualBins - 1);      // R is 0 there: midpoints beyond add nothing
+                        float4 next[2] = {__ldg(tab), __ldg(tab + 1)};               // two points each; the next four are on their way
+                        for (bool go = true; go;) {
+                            const float mid[4] = {next[0].x, next[0].z, next[1].x, next[1].z}, gap[4] = {next[0].y, next[0].w, next[1].y, next[1].w};
+                            tab += 2;
+                            next[0] = __ldg(tab);
+                            next[1] = __ldg(tab + 1);
+                            float f[4], u[4], g[4];
+                            float4 bin[4];
 #pragma unroll
                             for (int j = 0; j < 4; ++j) {
-                                const float mid = __uint_as_float(raw[j].z), u = __fmaf_rd(mid, s, kMagic);
-                                const int b = magic_int(u);
-                                f[j] = fmaf(mid, s, -(u - kMagic));
-                                // midpoints ascend, and R is 0 beyond the last bin: the first one outside ends the lane's list
-                                go = go && k0 + j < n && mid * s < (float)(kDualBins - 1) && b < kDualBins - 1;
-                                if (!go) {
-                                    raw[j].x = raw[j].y = raw[j].w = 0u;
-                                    f[j] = 0.f;
-                                }
-                                bin[j] = *reinterpret_cast<const uint4*>(bs + (go ? b : 0));
+                                u[j] = fminf(__fmaf_rd(mid[j], s, kMagic), kEnd);
+                                f[j] = fmaf(mid[j], s, -(u[j] - kMagic));
+                                bin[j] = *reinterpret_cast<const float4*>(bs + magic_int(u[j]));
                             }
 #pragma unroll
                             for (int j = 0; j < 4; ++j) {
-                                const float gf = __uint_as_float(raw[j].w), h = __uint_as_float(bin[j].w) * fmaf(-f[j], f[j], f[j]);
-                                acc = fma(__hiloint2double((int)raw[j].y, (int)raw[j].x), __hiloint2double((int)bin[j].y, (int)bin[j].x), acc);
-                                lin = fmaf(gf, fmaf(f[j], __uint_as_float(bin[j].z), h), lin);
-                                wid = fmaf(gf, h, wid);
+                                const float h = bin[j].z * fmaf(-f[j], f[j], f[j]);
+                                g[j] = gap[j] * (bin[j].x - fmaf(f[j], bin[j].y, h));
+                                wid = fmaf(gap[j], h, wid);
                             }
+                            acc += (double)((g[0] + g[1]) + (g[2] + g[3]));
+                            go = __any_sync(0xffffffffu, u[3] < kEnd);               // midpoints ascend
                         }
                     }
                     if (valid) {
                         const double unit = 2.0 * w_true * w_true * (double)s;
-                        const double est = es - unit * (acc - (double)lin);
+                        const double est = es - unit * acc;
                         const double off = unit * (double)wid * 1.00001 + margin0 + 1e-5 * fabs(est);
                         // (kept as a share of sum x^2, which may lie outside binary32)
                         curve[c * a.n_cand2 + d] = ok ? (float)((est - off) * inv_es * (1.0 - (est > off ? 1e-7 : -1e-7))) : INFINITY;
@@ -670,10 +690,10 @@ __global__ void __launch_bounds__(kDualBoundThreads, BLOCKS) dual_bound_kernel(c
                     double ss = 0.0;
                     long long zero = 0;
                     for (int i = tid; i < k; i += nthr) {
-                        int t, q;
+                        float t, q;
                         const float v = xs[i];
                         dc.of(v, t, q);
-                        const double dd = (double)v - (double)a1 * (double)t - (double)a2 * (double)q;
+                        const double dd = fma(-(double)a2, magic_double(q), fma(-(double)a1, magic_double(t), (double)v));
                         ss += dd * dd;
                     }
                     block_sum2(ss, zero, scratch);
@@ -706,15 +726,15 @@ __global__ void __launch_bounds__(kDualBoundThreads, BLOCKS) dual_bound_kernel(c
             const int n_pairs = (k + o + 1) >> 1;
             for (int p = tid; p < n_pairs; p += nthr) {
                 const int e0 = 2 * p - o, e1 = e0 + 1;
-                int t0c = 0, q0c = 0, t1c = 0, q1c = 0;
+                float t0c = kMagic, q0c = kMagic, t1c = kMagic, q1c = kMagic;
                 if (e0 >= 0) {
                     const float v = xs[e0];
                     if (!degenerate) dc.of(v, t0c, q0c);
-                    const double dd = (double)v - (double)alpha1 * (double)t0c - (double)alpha2 * (double)q0c;
+                    const double dd = fma(-(double)alpha2, magic_double(q0c), fma(-(double)alpha1, magic_double(t0c), (double)v));
                     ss += dd * dd;
                     if (a.codes) {
-                        a.codes[row_base + e0] = (signed char)t0c;
-                        a.codes[n_total + row_base + e0] = (signed char)q0c;
+                        a.codes[row_base + e0] = (signed char)magic_int(t0c);
+                        a.codes[n_total + row_base + e0] = (signed char)magic_int(q0c);
                     }
                 } else {
                     t0c = s_carry[0];
@@ -724,18 +744,18 @@ __global__ void __launch_bounds__(kDualBoundThreads, BLOCKS) dual_bound_kernel(c
                 if (has1) {
                     const float v = xs[e1];
                     if (!degenerate) dc.of(v, t1c, q1c);
-                    const double dd = (double)v - (double)alpha1 * (double)t1c - (double)alpha2 * (double)q1c;
+                    const double dd = fma(-(double)alpha2, magic_double(q1c), fma(-(double)alpha1, magic_double(t1c), (double)v));
                     ss += dd * dd;
                     if (a.codes) {
-                        a.codes[row_base + e1] = (signed char)t1c;
-                        a.codes[n_total + row_base + e1] = (signed char)q1c;
+                        a.codes[row_base + e1] = (signed char)magic_int(t1c);
+                        a.codes[n_total + row_base + e1] = (signed char)magic_int(q1c);
                     }
                 }
                 if (a.packed) {
                     if (has1 || !more) {
                         const long long b = (row_base + e0) >> 1;
-                        a.packed[b] = (unsigned char)((t0c & 0xf) | ((t1c & 0xf) << 4));
-                        a.packed[packed_stride + b] = (unsigned char)((q0c & 0xf) | ((q1c & 0xf) << 4));
+                        a.packed[b] = (unsigned char)((magic_int(t0c) & 0xf) | ((magic_int(t1c) & 0xf) << 4));
+                        a.packed[packed_stride + b] = (unsigned char)((magic_int(q0c) & 0xf) | ((magic_int(q1c) & 0xf) << 4));
                     } else {   // last element of the row: its byte is completed by the next row of the unit
                         s_carry[0] = t0c;
                         s_carry[1] = q0c;
