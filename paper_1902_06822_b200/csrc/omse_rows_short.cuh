@@ -372,8 +372,9 @@ __device__ __forceinline__ bool hist_search(const ShortSmem& sm, const ShortRow&
     int done = 0;
     if (levels > 8) {
         // The smallest scales have the most levels: 8 lanes share each of the first 16, 4 each of the next 8.  The smallest of all, which
-        // leave the largest value further away than the whole error is at the first scale that reaches it, are not looked at.
-        const float t_max = fmaxf(t_pos, t_neg), reach = ceilf(__fdividef(t_max, (float)(2 * levels + 1)) * 1.00001f) * 1.0001f;
+        // leave the largest value further away than the whole error is at the first scale that reaches it, are not looked at.  (Of the values
+        // that the range reaches: on an unsigned one the negative values err by as much at every scale.)
+        const float t_max = sgn ? fmaxf(t_pos, t_neg) : t_pos, reach = ceilf(__fdividef(t_max, (float)(2 * levels + 1)) * 1.00001f) * 1.0001f;
         const int skip = reach <= (float)n_cand ? max(0, (int)floorf(__fdividef(t_max - sqrtf((float)k) * reach, (float)(2 * levels + 2)) * 0.9999f) - 1) : 0;
         for (int i = lane; i < min(min(skip, 16), n_coarse); i += 32) coarse[i] = 3e38f;
         auto shared = [&](int from, int to, int lanes) {

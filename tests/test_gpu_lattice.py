@@ -286,3 +286,23 @@ def test_rows_by_a_histogram_of_their_warp(s, k, bits, signed, n_cand, hi_frac, 
     rows = np.unique(np.concatenate([np.arange(0, s, 41), np.arange(0, s, 130), [s - 2, s - 1]]))
     st = check_rows(w, alpha, sse, idx, q, None, bits, signed, n_cand, hi_frac, 3, rows=rows)
     assert st["idx_diff"] <= max(1, st["rows"] // 50) and st["alpha_bitwise"] >= 0.99, st
+
+
+@pytest.mark.parametrize("k,bits,n_cand", [(400, 4, 1024), (577, 4, 1024), (700, 5, 600), (703, 6, 1024), (1152, 6, 1024), (1152, 8, 1024),
+                                           (1281, 8, 500), (2304, 4, 1024), (2304, 8, 1024)])
+def test_unsigned_rows_of_both_signs_by_a_histogram(k, bits, n_cand):
+    """Values of both signs on an unsigned range: a negative value errs by as much at every scale, however large it is, so it says
+    nothing about the smallest scales.  Rows as they are drawn, with one large negative value, few positive ones, and none."""
+    import gpu_util
+    s = 1205
+    w = synth.student_t3(s * k, seed=79, tensor_id=k).reshape(s, k)
+    w[1::6, k // 2] = -8.0 * np.abs(w[1::6]).max(axis=1)
+    w[2::6] = ((np.arange(k) % 97) / 97.0).astype(np.float32)              # a lattice of positive values beside one of -8
+    w[2::6, 5] = -8.0
+    w[3::6] = np.where(w[3::6] < 1.5, -np.abs(w[3::6]), w[3::6])
+    w[4::6, ::2] = -2.0 * np.abs(w[4::6, ::2])
+    w[::300] = -np.abs(w[::300])                                           # nothing to code: every scale is as good
+    alpha, sse, idx, q, pk = gpu_util.quantize_weights(w, bits, False, n_cand, 1.0, 3, True, bits <= 4)
+    rows = np.unique(np.concatenate([np.arange(0, s, 11), np.arange(0, s, 300), [s - 1]]))
+    st = check_rows(w, alpha, sse, idx, q, None, bits, False, n_cand, 1.0, 3, rows=rows)
+    assert st["idx_diff"] <= max(1, st["rows"] // 50) and st["alpha_bitwise"] >= 0.99, st
