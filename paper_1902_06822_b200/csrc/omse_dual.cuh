@@ -632,7 +632,7 @@ __global__ void __launch_bounds__(kDualBoundThreads, BLOCKS) dual_bound_kernel(c
 #pragma unroll
                             for (int j = 0; j < 4; ++j) {
                                 u[j] = fminf(__fmaf_rd(mid[j], s, kMagic), kEnd);
-                                f[j] = fmaf(mid[j], s, -(u[j] - kMagic));
+                                f[j] = fminf(fmaf(mid[j], s, -(u[j] - kMagic)), 1.0f);      // (1 beyond the last bin: the square stays finite)
                                 bin[j] = *reinterpret_cast<const float4*>(bs + magic_int(u[j]));
                             }
 #pragma unroll

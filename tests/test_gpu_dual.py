@@ -81,6 +81,18 @@ def test_dual_grid_shapes(gpu, c1, c2):
     _check(gpu, t, c1=c1, c2=c2)
 
 
+@pytest.mark.parametrize("bits1,bits2,signed,hf1,hf2", [(4, 4, False, 1e8, 1e-9), (2, 3, False, 1e8, 1e-9), (4, 4, True, 1e8, 1e-9),
+                                                        (4, 4, False, 1e12, 1e-12), (2, 3, False, 1e12, 1e-12), (3, 2, True, 1e12, 1e-12)])
+def test_dual_first_grid_far_beyond_the_largest_value(gpu, bits1, bits2, signed, hf1, hf2):
+    """First scales of 1e8 and 1e12 times max|x|, second ones of a few per cent of it: the second tensor alone codes the row, and no
+    point of the first lies below max|x|."""
+    t = synth.laplace(20 * 400, 0.03, seed=650, tensor_id=bits1).reshape(20, 400)
+    if not signed:
+        t = np.abs(t)
+    alpha, _ = _check(gpu, t, bits1, bits2, signed, c1=16, c2=16, hf1=hf1, hf2=hf2)
+    assert np.all(alpha[0] > 1e3) and np.all(alpha[1] < np.abs(t).max(axis=1))
+
+
 def test_dual_degenerate_rows_and_invalid_arguments(gpu):
     import torch
     from paper_1902_06822_b200 import binding
