@@ -891,9 +891,11 @@ __device__ __forceinline__ void short_step(const RowArgs& a, const RowTensor& T,
             if (open) alpha = a_new;
         }
     }
-    // ---- final codes and error; the codes leave through shared memory, at the same offset from 8 elements
+    // ---- final codes and error; the codes leave through shared memory, at the same offset from 8 elements.  They lie where the stack
+    //      and the list have been: every lane's last look at those comes before any lane's first code (votes do not order memory).
     const int o = (int)(flat0 & 7);
     signed char* qs = sm.qs;
+    __syncwarp();
     {
         const float inv = alpha > 0.f ? __fdiv_rn(1.0f, alpha) : 0.f;
         const double ad = (double)alpha;
