@@ -775,9 +775,15 @@ __device__ __forceinline__ double tensor_band(double bv, double sum_sq) {
 // The first polish step, alpha <- <x,q>/<q,q> at candidate c, needs no look at the tensor: at a scale of the grid the thresholds are
 // edges of bins, and <x,q>, <q,q> are the sums that the curve was made of, exact integers but for a last rounding in binary64.  Only
 // the values next to an edge may be coded differently by the IEEE quotient; they are listed, and here is what such a value
-// changes.  (51,380,224 values: a step less is 47 us of 366; 1,605,633 in one kernel: an exchange and a pass, 4 us of 37.)  y: the value times HistGeometry::pre; hi, d: levels and spacing of the extra negative level as in HistGeometry.
-__device__ __forceinline__ void near_correction(float y, const HistGeometry& g, int c, int hi, float alpha, float inv, float flo, float fhi, float thr,
-                                                double& dx, long long& dq) {
+// changes.  (51,380,224 values: a step less is 47 us of 366; 1,605,633 in one kernel: an exchange and a pass, 4 us of 37.)  The values come in
+// the order in which atomics listed them, so the sums of their changes have to be exact: in the histogram's units (h is hk of them, below
+// 2^24) a value is an integer.  512 of them in 4096 bins stay below 2^53, a quarter of a million in 8192 bins below 2^63.
+// y: the value times HistGeometry::pre; hi: levels of a side.
+struct NearChange {
+    float x, units;          // magnitude, and the same in the histogram's units
+    int q, qq;               // change of its code's magnitude and of the square
+};
+__device__ __forceinline__ NearChange near_change(float y, const HistGeometry& g, int c, int hi, float alpha, float inv, float flo, float fhi, float thr) {
     const float s = y * g.scale, v = g.sgn ? fabsf(s) : s, u = __fmaf_rd(v, g.inv_up, kMagic);
     int m = magic_int(u), k = __float2int_rz(fmaf(-(u - kMagic), g.h, v));
     if (hist_near(k, m)) hist_correct(k, m, g.hk);
@@ -785,8 +791,7 @@ __device__ __forceinline__ void near_correction(float y, const HistGeometry& g, 
     if (y < 0.f && g.d > 0 && min(m / g.d, g.n_bins2) >= c + 1) ++counted;
     const float x = y * __fdiv_rn(1.0f, g.pre);
     const int coded = abs(exact_code(x, alpha, inv, flo, fhi, thr));
-    dx += (double)fabsf(x) * (double)(coded - counted);
-    dq += coded * coded - counted * counted;
+    return NearChange{fabsf(x), fabsf(s), coded - counted, coded * coded - counted * counted};
 }
 // The step by one block at candidate c (same in all threads): sx, sq are <x,q>/h and <q,q> there as the bins have it.
 __device__ __forceinline__ void tensor_first_step(const TensorArgs& a, float step, int c, double* scratch) {
@@ -796,14 +801,17 @@ __device__ __forceinline__ void tensor_first_step(const TensorArgs& a, float ste
     const HistGeometry g = hist_geometry(step, a);
     const float alpha = __fmul_rn((float)(c + 1), step), inv = __fdiv_rn(1.0f, alpha), flo = (float)a.lo, fhi = (float)a.hi,
                 thr = ambiguity_threshold(flo, fhi);
-    double dx = 0.0;
-    long long dq = 0;
-    for (unsigned int i = threadIdx.x; i < n_near; i += blockDim.x)
-        near_correction(__ldcg(a.near + i), g, c, a.hi, alpha, inv, flo, fhi, thr, dx, dq);
-    block_sum2(dx, dq, scratch);
+    double dq = 0.0;
+    long long dx = 0;
+    for (unsigned int i = threadIdx.x; i < n_near; i += blockDim.x) {
+        const NearChange v = near_change(__ldcg(a.near + i), g, c, a.hi, alpha, inv, flo, fhi, thr);
+        dx += (long long)v.units * v.q;
+        dq += (double)v.qq;
+    }
+    block_sum2(dq, dx, scratch);
     if (threadIdx.x == 0) {
-        const double sxq = fma(0.5 * (double)step, __ldcg(a.levels + c), dx);
-        const long long sqq = (long long)__ldcg(a.levels + a.n_cand + c) + dq;
+        const double sxq = fma(0.5 * (double)step, __ldcg(a.levels + c), (double)dx / ((double)g.scale * (double)g.pre));
+        const long long sqq = (long long)__ldcg(a.levels + a.n_cand + c) + (long long)dq;
         const float a_new = sqq != 0 ? (float)(sxq / (double)sqq) : 0.f;
         if (a_new >= FLT_MIN && a_new <= FLT_MAX && a_new != alpha) st->alpha = a_new;
         else st->polish_done = 1;                           // as a polish pass would
@@ -1463,8 +1471,11 @@ __global__ void __launch_bounds__(kResidentThreads) tensor_resident_kernel(const
                 sx += d * (above2[a.n_bins2 + best] + (double)(best + 1) * nn);
                 sn += d * nn;
             }
-            if (tid < (int)n_near)
-                near_correction(near_y, g, best, a.hi, alpha, __fdiv_rn(1.0f, alpha), flo, fhi, thr, dx, dq);
+            if (tid < (int)n_near) {
+                const NearChange v = near_change(near_y, g, best, a.hi, alpha, __fdiv_rn(1.0f, alpha), flo, fhi, thr);
+                dx = (double)v.x * (double)v.q;
+                dq = v.qq;
+            }
             if (__syncthreads_or(dq != 0)) block_sum2(dx, dq, scratch);
             else dx = 0.0;
             const double sxq = fma(0.5 * (double)gr.step, sx, dx);
