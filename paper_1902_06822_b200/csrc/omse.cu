@@ -176,9 +176,12 @@ size_t lattice_bytes(const omse::RowArgs& a, int threads, int n_bins, bool packe
 // Threads of a block for rows that leave room for `fit` blocks on an SM: the 24 warps that the registers allow, shared out.
 // (At 5592 rows of 12,000 values, three blocks: 8 warps 456 us, 6 493, 12 537; at 3728 of 18,000, two blocks: 12 warps 482 us,
 // 8 494, 16 629; at 2396 of 28,000, one block: 16 warps 563, 24 590, 12 609.)  No more than a thread per 8 values.
+constexpr int kLeastWarps = 4, kOneWarpK = 160;      // ... and four warps at least; rows of up to kOneWarpK values may have one
+static_assert((OMSE_MAX_KERNEL_LEN + 3) / 4 <= omse::kSquareSteps * 32 * kLeastWarps && (kOneWarpK + 3) / 4 <= omse::kSquareSteps * 32,
+              "float4s of a row per thread");
 int block_threads(int fit, long long max_k) {
-    const int warps = std::min(16, std::max(4, 24 / fit));
-    return 32 * (int)std::min<long long>(warps, std::max(4ll, (max_k / 8 + 31) / 32));
+    const int warps = std::min(16, std::max(kLeastWarps, 24 / fit));
+    return 32 * (int)std::min<long long>(warps, std::max<long long>(kLeastWarps, (max_k / 8 + 31) / 32));
 }
 
 // Launch over rows of at most max_k elements on one path: threads per block and shared memory.
@@ -205,7 +208,7 @@ int launch_rows(omse_ctx* ctx, omse::RowArgs& a, long long max_k, int path) {
     // 38,836 rows of 27 values 993 us and 326, 16,384 of 64 429 and 203, 10,485 of 100 283 and 161, 7133 of 147 205 and 163; 64
     // rows of 27 22.8 us and 18.5, of 64 22.7 and 18.5, of 100 22.6 and 19.0, of 147 with 200 candidates 20.5 and 21.3.)
     const bool many = a.n_units >= 8ll * ctx->n_sm;
-    if (max_k <= (many ? 160 : 128)) {
+    if (max_k <= (many ? kOneWarpK : 128)) {
         ext = true;
         a.direct = k4 >= 32 ? 2 : k4 >= 16 ? 1 : 0;
         smem = fixed + (size_t)((a.n_cand + 3) & ~3) * 4;

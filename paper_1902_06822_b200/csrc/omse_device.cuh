@@ -127,6 +127,8 @@ struct Coder {
     }
 };
 // sums of q*q over pairs of codes M + q, in binary32: exact below 2^24, so for 258 pairs of squares of up to 255^2
+constexpr int kSquareSteps = 258;
+static_assert(kSquareSteps * 255 * 255 < 1 << 24, "sums of squared codes stay exact in binary32");
 __device__ __forceinline__ u64 add_squares(float t0, float t1, u64 acc) {
     const u64 q = add2(pack2(t0, t1), pack2(-kMagic, -kMagic));
     return fma2(q, q, acc);

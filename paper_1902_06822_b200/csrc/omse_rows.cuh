@@ -161,8 +161,8 @@ __device__ __forceinline__ float polish_block(const float* xs, int k, float alph
         u64 qa = 0ull, qb = 0ull;
         const Coder coder(alpha, __fdiv_rn(1.0f, alpha), flo, fhi);
 #pragma unroll 1
-        for (int i4 = threadIdx.x; i4 < k4; i4 += blockDim.x) {   // four elements per step (56 steps at most: blocks of 128 threads or
-            const float4 v = xs4[i4];                             // short rows); the zero padding adds nothing
+        for (int i4 = threadIdx.x; i4 < k4; i4 += blockDim.x) {   // four elements per step, kSquareSteps steps at most (see block_threads);
+            const float4 v = xs4[i4];                             // the zero padding adds nothing
             const float x[4] = {v.x, v.y, v.z, v.w};
             float t[4];
             coder.of(v, t);
