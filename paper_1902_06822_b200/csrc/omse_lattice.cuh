@@ -157,16 +157,12 @@ struct LatticeSmem {
     unsigned int* f2;
     float* curve;         // the curve: aliases n, or an array of its own for lattice_search_wide
 };
-// The counts, a word each or (PACKED; a row has at most 28,672 values) two to a word.  Adding a constant 1 is what shared
-// memory does fastest when many values of a warp meet in one bin (rows of 23,000 values 551 us, packed 585), so packed counts
+// The counts, a word each or (PACKED; a row has at most 28,672 values) two to a word.  Adding a constant 1 (shared_add1) is what
+// shared memory does fastest when many values of a warp meet in one bin (rows of 23,000 values 551 us, packed 585), so packed counts
 // are for the rows whose bins would not leave room for a second block on the SM otherwise (of 25,088 values 539 us, 443).
 template <bool PACKED>
 struct Counts {
     static __host__ __device__ __forceinline__ int words(int bins) { return PACKED ? bins >> 1 : bins; }
-    static __device__ __forceinline__ void add(unsigned int* n, int w) {
-        if (PACKED) atomicAdd(n + (w >> 1), 1u << ((w & 1) << 4));
-        else atomicAdd(n + w, 1u);
-    }
     static __device__ __forceinline__ uint4 four(const unsigned int* n, int w) {
         if (!PACKED) return *reinterpret_cast<const uint4*>(n + w);
         const uint2 a = *reinterpret_cast<const uint2*>(n + (w >> 1));
