@@ -16,7 +16,7 @@
 
 namespace {
 
-constexpr long long kSmallK = 1280;           // rows up to this length are searched in the registers of a warp or of some of its lanes:
+constexpr long long kJoinK = 1024, kSmallK = 1280;           // rows up to this length are searched in the registers of a warp or of some of its lanes:
                                               // 58,254 rows of 1152 values 754 us against 1097 by blocks
 // Rows by a histogram of their warp, from 4 bits on (fewer leave too many candidates open).  Splits, or blocks beyond kSmallK, and
 // histogram, 67M Laplace values: 1024 candidates on 4 bits, 400 values a row 1034 us and 1005, 512 886 and 782, 1024 829 and 603, 1600
@@ -508,16 +508,30 @@ int quantize_list(omse_ctx* ctx, std::vector<omse::RowTensor>& list, int bits, i
     // 40 and 33; 2400 rows of 288 values 29 and 33, 10,000 75 and 70; 1200 rows of 576 values 34 and 31); 8 bits, whose
     // best scale lies where the splits have furthest to go, change over later (10,000 rows of 27 values 41 and 52).
     const bool plain = mode.solver == 0 && mode.n_delta == 0;   // the block path implements everything else
-    long long short_rows = 0, short_elements = 0, short_warps = 0, long_rows = 0;
-    for (const auto& t : list)
-        if (t.K > kSmallK && t.K <= kHistMaxK) {
+    long long short_rows = 0, short_elements = 0, short_warps = 0, mid_rows = 0, long_rows = 0, mid_elements = 0;
+    bool longer = false;
+    for (const auto& t : list) {
+        if (t.K > kHistMaxK) {
+            longer = true;
+        } else if (t.K > kSmallK) {
             long_rows += t.S;
-        } else if (t.K <= kSmallK) {
+        } else if (t.K > kJoinK) {
+            mid_rows += t.S;
+            mid_elements += t.S * t.K;
+        } else {
             short_rows += t.S;
             short_elements += t.S * t.K;
             short_warps += (t.S << omse::short_lanes(t.K)) / 32;
         }
-    const long long short_k = short_rows >= 8ll * ctx->n_sm ? kSmallK : 160;
+    }
+    const long long hist_rows = short_rows + mid_rows + long_rows;
+    const bool join = mid_rows >= 12ll * ctx->n_sm || (short_rows >= 32ll * ctx->n_sm && mid_rows >= 2ll * ctx->n_sm);
+    if (join) {
+        short_rows += mid_rows;
+        short_elements += mid_elements;
+        short_warps += mid_rows;
+    }
+    const long long short_k = short_rows < 8ll * ctx->n_sm ? 160 : join ? kSmallK : kJoinK;
     a.short_direct = short_rows < (a.hi[0] > 63 ? 96ll : 48ll) * ctx->n_sm && short_elements < 5120ll * ctx->n_sm;
     int spread = 0;                                             // more lanes per row where the warps do not fill the GPU
     while (spread < 5 && (short_warps << (spread + 1)) <= 16ll * ctx->n_sm) ++spread;
@@ -534,10 +548,14 @@ int quantize_list(omse_ctx* ctx, std::vector<omse::RowTensor>& list, int bits, i
     // 22 us by blocks and 18.5, 300 rows 19 and 18.5; 600 of 1024 values 22 and 22.6, 1180 35 and 25; 600 of 2304 28 and 37, 1180 43
     // and 40).  Beside rows of other paths the launch has to be worth its cost.
     long long hist_from = a.hi[0] > 15 ? kHistK8 : kHistK4, hist_to = kHistMaxK, hist_elements = 0, other_elements = 0;
-    if (short_rows + long_rows < 7ll * ctx->n_sm) hist_to = 800;
-    if (!hist_fits || short_rows + long_rows < 4ll * ctx->n_sm) hist_to = 0;
+    if (longer && long_rows < 16ll * ctx->n_sm) hist_to = kSmallK;
+    if (hist_rows < 7ll * ctx->n_sm) hist_to = a.hi[0] > 15 || a.n_cand < 512 ? 0 : 800;
+    if (!hist_fits || hist_rows < 4ll * ctx->n_sm) hist_to = 0;
     for (const auto& t : list) (t.K >= hist_from && t.K <= hist_to ? hist_elements : other_elements) += t.S * t.K;
-    if (other_elements > 0 && hist_elements < 1 << 21) hist_to = 0;
+    if (other_elements > 0 && hist_elements < 1 << 21) {
+        hist_from = std::max(hist_from, kHistK8);
+        hist_to = std::min(hist_to, kJoinK);
+    }
     // One launch per row path present in the list: each launch then runs the kernel instantiation that holds only its path.
     // Longest rows first inside a launch: the dispenser hands out work in decreasing size and the tail is short.
     std::stable_sort(list.begin(), list.end(), [](const omse::RowTensor& x, const omse::RowTensor& y) { return x.K > y.K; });
