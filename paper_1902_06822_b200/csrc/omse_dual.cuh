@@ -594,14 +594,15 @@ __global__ void __launch_bounds__(kDualBoundThreads, BLOCKS) dual_bound_kernel(c
                     ls += s_sums[1][v];
                 }
                 __syncthreads();
-                // ---- estimate and bounds of every pair.  The margin holds what the fixed point (ls) and binary32 can add, u = 2^-24 each: a
-                //      midpoint's position four roundings (mid, 1/w, s, f), which moves the sum by at most 8u of es, since the sum of
-                //      2*gap*mid below |x| is its nearest point squared, in all 2*(es + error); a term's value three of R at the
-                //      bin's lower edge, in all below 1.34*es, and five of its own; `unit` two of unit*acc <= es + error.  Together 19u
-                //      = 1.14e-6 of es; what goes with the error or with the width is far below the factors of those in `off`.
+                // ---- estimate and bounds of every pair.  The margin holds what the fixed point (ls) and binary32 can add, u = 2^-24 each.
+                //      Four roundings of a midpoint's position (mid, 1/w, s, f) move its term by 4u of 2*gap*mid per value beyond it, which
+                //      sums to the squares of the values' nearest points, at most 1.05*es + 21 errors.  Three of R at the bin's lower edge
+                //      and of its fall from there: with r - R at most a bin per value, in all 0.34*es (28,672 values), 2.02u of es.
+                //      Five of the term itself, two of `unit`: 7u of unit*acc <= es.  Together 13.3u = 8e-7 of es, and 5e-6 of the error,
+                //      which with what goes with the width is inside the factors of those in `off`.
                 const float scale_pre = pre;
                 const double w_true = (double)w / (double)scale_pre;
-                const double margin0 = 1.2e-6 * es + ls * w_true * fq + 3e-45 * (double)k;
+                const double margin0 = 1e-6 * es + ls * w_true * fq + 3e-45 * (double)k;
                 inv_es = 1.0 / es;
                 const float inv_w = __fdiv_rn(1.0f, w);
                 // A warp takes 8 neighbouring alpha1 of 4 neighbouring ratios at a time: lanes of similar alpha1 have about as
