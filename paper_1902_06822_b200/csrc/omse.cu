@@ -16,12 +16,14 @@
 
 namespace {
 
-constexpr long long kJoinK = 1024, kSmallK = 1280;           // rows up to this length are searched in the registers of a warp or of some of its lanes:
-                                              // 58,254 rows of 1152 values 754 us against 1097 by blocks
-// Rows by a histogram of their warp, from 4 bits on (fewer leave too many candidates open).  Splits, or blocks beyond kSmallK, and
-// histogram, 67M Laplace values: 1024 candidates on 4 bits, 400 values a row 1034 us and 1005, 512 886 and 782, 1024 829 and 603, 1600
-// 887 and 600, 2304 698 and 538; on 8 bits, 640 values 999 and 991 (Student-t 867 and 975), 800 1211 and 969, 1024 998 and 772, 2304
-// 783 and 563.  Beyond 2304 values the rows leave an SM fewer than twelve warps.
+constexpr long long kSmallK = 1280;           // rows up to this length are searched in the registers of a warp or of some of its lanes
+                                              // (58,254 rows of 1152 values on 3 bits 687 us against 1077 by blocks),
+constexpr long long kJoinK = 1024;            // those beyond this length only in large numbers: see quantize_list
+// Rows by a histogram of their warp, from 4 bits on (fewer leave too many candidates open).  Splits, or blocks beyond kJoinK, and
+// histogram, 67M Laplace values (Student-t in brackets), 1024 candidates, on 4 bits: 400 values a row 1036 us and 1071 (976 and 1053), 512 888
+// and 823 (834 and 805), 640 824 and 729 (780 and 712), 1024 831 and 633 (769 and 615), 1152 1101 and 627, 1600 891 and 640, 2304 701 and 588;
+// on 8 bits: 640 1001 and, by splits still, 999, 700 1299 and 973 (1089 and 957), 1024 1000 and 774 (821 and 769), 1600 1015 and 700, 2304
+// 786 and 560.  Beyond 2304 values the rows leave an SM fewer than twelve warps.
 constexpr long long kHistK4 = 400, kHistK8 = 700, kHistMaxK = 2304;
 constexpr long long kDualBoundK = 256;        // dual search: rows at least this long go by histogram and bounds (16 rows of 256 values 58 us
                                               // against 100 by the sweep, of 128 values 55 by the sweep, whose time is proportional to the length)
@@ -507,6 +509,10 @@ int quantize_list(omse_ctx* ctx, std::vector<omse::RowTensor>& list, int bits, i
     // whose chain is short, large numbers by splits, which evaluate less (6000 rows of 27 values 23 us against 31, 10,000
     // 40 and 33; 2400 rows of 288 values 29 and 33, 10,000 75 and 70; 1200 rows of 576 values 34 and 31); 8 bits, whose
     // best scale lies where the splits have furthest to go, change over later (10,000 rows of 27 values 41 and 52).
+    // Rows of 1025 to 1280 values take a warp long, and few of them hold up a launch of short rows (1500 rows of 64 values and 20 of 1152, 4
+    // bits, 256 candidates 43 us, 19 with those by blocks): they go by splits from 12 per SM on (3 bits, 256 candidates, 1500 rows of 1280
+    // values 33 by blocks and 32, outliers 33 and 37; 1024 candidates, 1776 rows of 1152 46 and 40, 2400 of 1280 57 and 49), or from two per SM
+    // beside 32 shorter rows per SM, which take as long anyway (10,000 rows of 64 values and 300 of 1152, 8 bits, 256 candidates 44 and 36).
     const bool plain = mode.solver == 0 && mode.n_delta == 0;   // the block path implements everything else
     long long short_rows = 0, short_elements = 0, short_warps = 0, mid_rows = 0, long_rows = 0, mid_elements = 0;
     bool longer = false;
@@ -544,17 +550,33 @@ int quantize_list(omse_ctx* ctx, std::vector<omse::RowTensor>& list, int bits, i
     // (the largest |x|/h, rounded up to a fraction, lies in a bin)
     const bool hist_fits = plain && a.hi[0] >= 7 && a.n_bins > 0 &&
                            2.0 * a.n_cand / (double)a.hi_frac * (1.0 + 4e-7) + 1.0 / 64 < (double)hist_words + 1.0;
-    // A row takes a warp 15 to 30 us, a block a third of that: with fewer rows than this blocks are sooner done (600 rows of 576 values
-    // 22 us by blocks and 18.5, 300 rows 19 and 18.5; 600 of 1024 values 22 and 22.6, 1180 35 and 25; 600 of 2304 28 and 37, 1180 43
-    // and 40).  Beside rows of other paths the launch has to be worth its cost.
+    // A row takes a warp 15 to 30 us, a block a third of that: with fewer than seven rows per SM blocks are sooner done (1036 rows of 1024
+    // values on 4 bits, 1024 candidates 33 us by blocks and 24, of 2304 42 and 40; 592 of 2304 28 and 37), and down to four only where they have
+    // many candidates to look at and not many levels (592 of 576 values on 4 bits 21 and 19, of 768 23 and 22, 256 candidates and 448 values 15 and
+    // 17; on 8 bits 592 of 768 21 and 25).  Rows of more than 1280 values beside longer ones, whose blocks are on the SMs anyway, from 16 per
+    // SM on (256 candidates, 512 rows of 4608 and 1200 of 2304 values 53 by blocks and 65, 2700 of 2048 79 and 69).  And beside rows of other
+    // paths the launch has to be worth its cost.  Less than 2M values: rows of up to 1024 values, the others by blocks (8192 rows of 128 values
+    // and 1200 of 576 49 and 54 with a launch for those, 3600 of 576 61 and 69; 512 of 4608 and 1200 of 1152 on 8 bits 58 and 63), where
+    // they are a quarter of all values (100 rows of 25,088 and 1200 of 1000 74 and 49, 4000 of 128 and 300 of 720 45 and 30) and the list is
+    // short (a call with 54 tensors takes the host 130 us, a launch more some 6).  Launches that fill the GPU many times over are bound by
+    // issue, not by chains, and the splits of up to 447 values are the cheaper ones there (150,000 rows of 400, 1024 candidates 916 and 941,
+    // Student-t 861 and 920; 24,000 rows 166 and 154), on 5 bits with few candidates up to 639 (256 candidates, 576 values 910 and 923, 830 and 917).
     long long hist_from = a.hi[0] > 15 ? kHistK8 : kHistK4, hist_to = kHistMaxK, hist_elements = 0, other_elements = 0;
+    if (hist_rows >= 256ll * ctx->n_sm) hist_from = std::max<long long>(hist_from, a.hi[0] > 7 && a.n_cand < 512 ? 640 : 448);
     if (longer && long_rows < 16ll * ctx->n_sm) hist_to = kSmallK;
     if (hist_rows < 7ll * ctx->n_sm) hist_to = a.hi[0] > 15 || a.n_cand < 512 ? 0 : 800;
     if (!hist_fits || hist_rows < 4ll * ctx->n_sm) hist_to = 0;
-    for (const auto& t : list) (t.K >= hist_from && t.K <= hist_to ? hist_elements : other_elements) += t.S * t.K;
+    auto by_hist = [&](const omse::RowTensor& t) { return t.K >= hist_from && t.K <= hist_to; };
+    auto share = [&]() {
+        hist_elements = other_elements = 0;
+        for (const auto& t : list) (by_hist(t) ? hist_elements : other_elements) += t.S * t.K;
+    };
+    share();
     if (other_elements > 0 && hist_elements < 1 << 21) {
         hist_from = std::max(hist_from, kHistK8);
         hist_to = std::min(hist_to, kJoinK);
+        share();
+        if (3 * hist_elements < other_elements || list.size() > 32) hist_to = 0;
     }
     // One launch per row path present in the list: each launch then runs the kernel instantiation that holds only its path.
     // Longest rows first inside a launch: the dispenser hands out work in decreasing size and the tail is short.
@@ -562,7 +584,7 @@ int quantize_list(omse_ctx* ctx, std::vector<omse::RowTensor>& list, int bits, i
     bool present[kPaths] = {};
     for (size_t i = 0; i < list.size(); ++i) {
         omse::RowTensor& t = list[i];
-        if (t.K >= hist_from && t.K <= hist_to) {
+        if (by_hist(t)) {
             // count and fractions of all values in one word, bin and fraction in 23 bits
             int count = 1, frac = 1;
             while ((1ll << count) <= t.K) ++count;
