@@ -306,3 +306,34 @@ def test_unsigned_rows_of_both_signs_by_a_histogram(k, bits, n_cand):
     rows = np.unique(np.concatenate([np.arange(0, s, 11), np.arange(0, s, 300), [s - 1]]))
     st = check_rows(w, alpha, sse, idx, q, None, bits, False, n_cand, 1.0, 3, rows=rows)
     assert st["idx_diff"] <= max(1, st["rows"] // 50) and st["alpha_bitwise"] >= 0.99, st
+
+
+@pytest.mark.parametrize("shapes,bits,signed,launches", [
+    ([(1801, 1280)], 3, True, 1), ([(1801, 1025)], 2, False, 1),       # all lanes and 40 values of a warp, in large numbers; by blocks otherwise
+    ([(4801, 64), (297, 1153)], 3, True, 1),                           # beside many shorter rows, in one launch with them,
+    ([(1501, 64), (21, 1152)], 4, True, 2),                            # by blocks beside fewer
+    ([(1203, 1000), (21, 5000)], 4, True, 2),                          # few values by a histogram beside others: up to 1024 a row,
+    ([(1101, 2304), (9, 5000)], 4, True, 1),                           # blocks beside blocks
+    ([(303, 720), (4001, 128)], 8, False, 2), ([(61, 720), (4001, 128)], 8, True, 1),
+    ([(38_001, 401)], 4, True, 1), ([(38_001, 449)], 4, True, 1), ([(38_001, 639)], 5, True, 1),
+])
+def test_rows_of_every_length_in_one_call(shapes, bits, signed, launches):
+    """Lists on either side of the rules that give a tensor's rows to splits, to a histogram of their warp or to a block."""
+    import torch
+    import gpu_util
+    ctx = gpu_util.ctx()
+    ws = [synth.student_t3(s * k, seed=80, tensor_id=i).reshape(s, k) for i, (s, k) in enumerate(shapes)]
+    descs = [dict(w=torch.from_numpy(w).cuda(), n_kernels=w.shape[0], kernel_len=w.shape[1], alpha=torch.empty(w.shape[0], device="cuda"),
+                  sse=torch.empty(w.shape[0], device="cuda"), best_idx=torch.empty(w.shape[0], dtype=torch.int32, device="cuda"),
+                  codes=torch.empty(w.size, dtype=torch.int8, device="cuda")) for w in ws]
+    torch.cuda.synchronize()
+    ctx.omse_read_launches()
+    ctx.omse_quantize_weights_batched(descs, bits, signed, 300, 1.0, 3)
+    assert ctx.omse_read_launches() == launches
+    torch.cuda.synchronize()
+    for w, d in zip(ws, descs):
+        s = w.shape[0]
+        rows = np.unique(np.concatenate([np.arange(0, s, max(1, s // 40)), [s - 1]]))
+        st = check_rows(w, d["alpha"].cpu().numpy(), d["sse"].cpu().numpy(), d["best_idx"].cpu().numpy(), d["codes"].cpu().numpy(), None, bits,
+                        signed, 300, 1.0, 3, rows=rows)
+        assert st["idx_diff"] <= max(1, st["rows"] // 50) and st["alpha_bitwise"] >= 0.99, (w.shape, st)
