@@ -33,9 +33,9 @@ N_CAND, BITS, REFINE, HI_FRAC = 1024, 4, 3, 1.0
 METRIC = "elements quantized/sec (4-bit MMSE search)"
 INSTR_PER_EVAL = 6            # reference FP32 sequence per (element, candidate): 3 fma + 2 min/max + 1 add
 LANE_OPS_PER_EVAL = 4         # FMA-pipe lane operations of an evaluation the kernels execute: fma, add, fma, fma
-# dram__bytes_read.sum + dram__bytes_write.sum of one step of the default workload (its two launches: rows of up to 1024
-# elements, and the longer ones beside them) from an ncu capture; None whenever the kernels have changed since the capture
-NCU_TRAFFIC_BYTES = 102_716_928
+# dram__bytes_read.sum + dram__bytes_write.sum of one step of the default workload (its three launches: short rows by splits, by a
+# histogram per warp, and the longest by blocks) from an ncu capture; None whenever the kernels have changed since the capture
+NCU_TRAFFIC_BYTES = 102_374_656
 E2E_CHUNKS = 12               # batched launches per end-to-end step (copies of later chunks overlap earlier searches)
 N_SM, LANES_PER_SM = 148, 128
 WORKLOAD = "resnet50_weight_set_54_tensors_25.5M_params_signed4bit_kernelwise_1024cand_3refine_packed"
@@ -182,8 +182,9 @@ class WeightSet(Workload):
         descs = [dict(w=dw, n_kernels=w.shape[0], kernel_len=w.shape[1], alpha=a, sse=e, **{key: c})
                  for w, dw, (a, e, c) in zip(self.tensors, self.d_w, self.outs)]
         self.n_total = sum(w.size for w in self.tensors)
-        n_short = sum(w.shape[0] for w in self.tensors if w.shape[1] <= 1024)     # short rows in small numbers go by blocks as well
-        short = [w.shape[1] <= (1024 if n_short >= 8 * N_SM else 160) for w in self.tensors]
+        most = 2304 if self.bits >= 4 else 1024                                   # short rows in small numbers go by blocks as well
+        n_short = sum(w.shape[0] for w in self.tensors if w.shape[1] <= most)
+        short = [w.shape[1] <= (most if n_short >= 8 * N_SM else 160) for w in self.tensors]
         self.kernel = ", ".join(k for k, there in (("rows_kernel", not all(short)), ("rows_short_kernel", any(short))) if there)
         self.h2d = 4 * self.n_total
         self.d2h = sum(a.numel() * 4 + e.numel() * 4 + c.numel() for a, e, c in self.outs)
@@ -249,8 +250,8 @@ class Activation(Workload):
     def host_arrays(self):
         return [self.x]
 
-    def algorithmic_bytes(self):  # maximum, histogram, polish steps and the final error each read the tensor once
-        return 4 * self.n_total * (1 if self.launches_per_step == 1 else 3 + REFINE)     # (in one kernel: the copy on chip)
+    def algorithmic_bytes(self):  # maximum, histogram, all polish steps but the first and the final error each read the tensor once
+        return 4 * self.n_total * (1 if self.launches_per_step == 1 else 2 + REFINE)     # (in one kernel: the copy on chip)
 
     def setup(self, ctx, torch, dev):
         self.host_in = torch.from_numpy(self.x).pin_memory()

@@ -18,9 +18,9 @@
  *   - Pointers without the d_ prefix are HOST memory, read before the call returns.
  *   - Calls only enqueue work on the context's CUDA stream and return; nothing synchronises
  *     except omse_last_device_status(), omse_read_evaluations() and omse_destroy().  A call
- *     whose list holds both long and short kernels runs one of its two launches on a second
- *     stream that the context owns, forked from the context's stream and joined back to it by
- *     events inside the call: for the caller everything stays ordered on the context's stream.
+ *     whose list holds kernels of very different lengths has up to three launches, of which all but
+ *     the last run on streams that the context owns, forked from the context's stream and joined back
+ *     to it by events inside the call: for the caller everything stays ordered on the context's stream.
  *   - All work queued through one context shares that context's device workspace (work-unit
  *     dispenser, search state, partial sums).  It must therefore be stream-ordered: after
  *     omse_set_stream() the caller makes the new stream wait for the work already queued on the
@@ -389,15 +389,15 @@ int omse_last_device_status(omse_ctx* ctx, uint32_t* host_out);
 /* Instrumentation (no counterpart in the paper): synchronises the stream and returns in *host_out how many element
  * evaluations the search kernels of this context executed since the last read, then clears the counter.  Placing an
  * element of a row on the grid counts as one, re-scoring a row at one candidate as one per element; where candidates are
- * evaluated one by one (rows of up to 1024 elements, grids that end far below max|x|) every (element, candidate)
+ * evaluated one by one (short rows without a histogram, grids that end far below max|x|) every (element, candidate)
  * evaluation counts.  For omse_dual_quantize the unit is (element, pair, first code); rows whose pairs are decided by bounds
  * count once per element and re-scored pair.  omse_activation_scale_static does not count. */
 int omse_read_evaluations(omse_ctx* ctx, uint64_t* host_out);
 
 /* Instrumentation (no counterpart in the paper): the number of kernels the calls on this context have launched since
  * the last read (host-side count, no synchronisation), then cleared.  A batched weight call launches one kernel per
- * row path present (long rows, rows of up to 1024 elements), the per-tensor search one, for tensors that fit on chip, or
- * ten or so. */
+ * row path present (a block per row, a histogram per warp, splits; up to three), the per-tensor search one, for tensors that fit on
+ * chip, or ten or so. */
 int omse_read_launches(omse_ctx* ctx, uint64_t* host_out);
 
 /* Instrumentation (no counterpart in the paper): how often a block of a per-tensor search that runs in one kernel looks for what

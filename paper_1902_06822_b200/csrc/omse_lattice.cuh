@@ -19,8 +19,8 @@
 //
 // Measured on one B200 against a sweep of all candidates over all values that they do not code as 0, 1024 candidates: 4096 x
 // 25,088 values in two tensors 7.25 -> 1.41 ms, 2674 x 25,088 on 8 bits 2.43 -> 0.43 ms, 14,563 x 4608 2.38 -> 0.49 ms.
-// Short rows are cheaper to search by evaluating some 25 candidates (omse_rows_short.cuh): 2C bins cost as much as a few
-// thousand values.
+// Short rows are cheaper to search by evaluating some 25 candidates (omse_rows_short.cuh): the 2C bins cost a block as much as a few
+// thousand values.  (A warp with a smaller form of the histogram comes out ahead from some 450 values on: hist_search there.)
 //
 // A signed range has one more code on the negative side: that level's thresholds are the multiples of D*h,
 // D = 2*|lo| - 1, and only negative values count; they go to a second, D times coarser histogram.

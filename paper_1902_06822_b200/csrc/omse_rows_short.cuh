@@ -1,5 +1,6 @@
-// Short kernels (up to 1024 weights, e.g. 3x3x3 or 64x3x3): a group of G = 1, 2, 4, ... 32 lanes of a warp owns a row, which
-// sits in their registers, and looks for the best candidate by evaluating a few of them, one after the other.
+// Short kernels (up to 1280 weights, e.g. 3x3x3 or 64x3x3): a group of G = 1, 2, 4, ... 32 lanes of a warp owns a row, which
+// sits in their registers, and looks for the best candidate by evaluating a few of them, one after the other.  (The longer ones of
+// them, and rows of up to 2304 weights, by a histogram: hist_search.)
 //
 // W(alpha) = sum_i sum_j (|x_i| - (j - 1/2)*alpha)_+ is convex, and the error is E - 2*alpha*W, so the errors at two
 // candidates bound it from below at all candidates between them (the chord of W).  The powers of two of the grid are tried
@@ -250,9 +251,11 @@ __device__ __forceinline__ ShortResult short_dispatch(int quads, const ShortSmem
 // sides gives a lower bound of the error, the largest negative value alone an upper one, and only the candidates that these leave
 // open (some 40 of 1024) get the exact sum over the few values that lie beyond it.  If more than one is within the noise of the
 // fractions, they are evaluated in binary32, as the splits do.
-// Bound: chains of dependent instructions (12 to 20 warps per SM) and 1000 clocks of an SM per row for clearing, scanning and looking
-// up 2048 bins.  Measured on one B200, 1024 candidates, 67M Laplace values, against splits (up to 1024 values) and a block per row:
-// 4 bits, 512 values a row 886 -> 782 us, 1024 829 -> 603, 1280 1014 -> 564, 2304 698 -> 538; 8 bits, 1024 998 -> 772, 2304 783 -> 563.
+// Bound: chains of dependent instructions (12 to 20 warps per SM, 0.54 to 0.59 of an instruction per clock and scheduler) and fetching
+// them: of some 7.3 cycles between two instructions of a warp (39,062 rows of 1024 values on 4 bits) 1.9 are the fixed latency, 1.45 missing
+// instructions (2.0 at 576 values, 0.7 on 8 bits), 1.0 shared memory.  Measured on one B200, 1024 candidates, 67M Laplace values, against
+// splits (up to 1024 values) and a block per row: 4 bits, 512 values a row 888 -> 823 us, 1024 831 -> 633, 1280 1015 -> 606, 2304 701 -> 588;
+// 8 bits, 1024 1000 -> 774, 2304 786 -> 560.
 struct HistShape {
     int n_bins, lb, fbits, cshift;        // bins; log2 of a lane's run of them; bits of a fraction; the count's place in the word
 };
@@ -501,15 +504,22 @@ __device__ __forceinline__ bool hist_search(const ShortSmem& sm, const ShortRow&
                 }
             }
             if (pass == 0) continue;
+            unsigned int within[kHistOpen];
 #pragma unroll
+            for (int c = 0; c < kHistOpen; ++c) within[c] = __ballot_sync(0xffffffffu, value[c] <= limit);
+            // One copy of the evaluation in the code, not eight: the warps of this kernel wait for instructions (30,000 rows of 1152 values, 4
+            // bits, no polish step 255 -> 238 us, with three 325 -> 318).
+            static_assert(kHistOpen == 4, "a ballot for each candidate of a lane");
+#pragma unroll 1
             for (int c = 0; c < kHistOpen; ++c) {
-                unsigned int some = __ballot_sync(0xffffffffu, value[c] <= limit);
+                unsigned int some = c == 0 ? within[0] : c == 1 ? within[1] : c == 2 ? within[2] : within[3];
+#pragma unroll 1
                 while (some) {
                     const float a1 = (float)(first + __ffs(some) - 1 + 32 * c);
                     some &= some - 1;
-                    if (n_left == 1) consider(single);
-                    if (n_left > 0) consider(a1);
-                    else single = a1;                         // (left as it is if it is the only one)
+                    if (n_left == 0) single = a1;             // (left as it is if it is the only one)
+#pragma unroll 1
+                    for (int i = n_left == 1 ? 0 : n_left == 0 ? 2 : 1; i < 2; ++i) consider(i == 0 ? single : a1);
                     ++n_left;
                 }
             }

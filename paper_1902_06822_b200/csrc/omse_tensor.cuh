@@ -1030,8 +1030,9 @@ __global__ void __launch_bounds__(256) tensor_pass_kernel(const TensorArgs a) {
 // slice once and keeps it for all passes, the blocks exchange sums through slots in global memory (a cooperative launch
 // guarantees that all of them run), and what has to be known everywhere - the scan of the histogram, the curve, the
 // polish - every block computes for itself.
-// Bound: latency.  A search is a chain of 3 + R exchanges of a microsecond or so each; the pipeline of launches pays a
-// launch and a trip of the values from L2 for each of them.
+// Bound: latency.  A search with R polish steps is a chain of 1 + R exchanges (extremes, histogram, every polish step but the first;
+// one more where candidates are re-scored) of a microsecond or two each; the pipeline of launches pays a launch and a trip of the
+// values from L2 for each of them.
 // -------------------------------------------------------------------------------------------------
 constexpr int kResidentBlocks = 160;     // blocks the exchange area has room for
 constexpr int kResidentBins = 4096;      // bins of the histogram in the exchange area (and as many coarse ones)

@@ -254,7 +254,7 @@ def test_launch_counter_counts_one_launch_per_row_path():
 
 
 def test_back_to_back_batched_calls_with_two_row_paths_stay_ordered_and_reproducible():
-    """A list with long and short rows runs its two launches beside each other (second stream inside the call).  Many
+    """A list with long and short rows runs its launches beside each other (on side streams inside the call).  Many
     such calls queued without a synchronisation in between, interleaved with per-tensor searches and single-path calls
     on the same context, must give the same bits every time, and the values of the oracle."""
     import torch
