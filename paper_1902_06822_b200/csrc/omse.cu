@@ -17,13 +17,13 @@
 namespace {
 
 constexpr long long kSmallK = 1280;           // rows up to this length are searched in the registers of a warp or of some of its lanes
-                                              // (58,254 rows of 1152 values on 3 bits 687 us against 1077 by blocks),
+                                              // (58,254 rows of 1152 values on 3 bits 684 us against 1078 by blocks),
 constexpr long long kJoinK = 1024;            // those beyond this length only in large numbers: see quantize_list
 // Rows by a histogram of their warp, from 4 bits on (fewer leave too many candidates open).  Splits, or blocks beyond kJoinK, and
 // histogram, 67M Laplace values (Student-t in brackets), 1024 candidates, on 4 bits: 400 values a row 1036 us and 1071 (976 and 1053), 512 888
-// and 823 (834 and 805), 640 824 and 729 (780 and 712), 1024 831 and 633 (769 and 615), 1152 1101 and 627, 1600 891 and 640, 2304 701 and 588;
-// on 8 bits: 640 1001 and, by splits still, 999, 700 1299 and 973 (1089 and 957), 1024 1000 and 774 (821 and 769), 1600 1015 and 700, 2304
-// 786 and 560.  Beyond 2304 values the rows leave an SM fewer than twelve warps.
+// and 821 (832 and 795), 640 823 and 728 (776 and 705), 1024 838 and 642 (768 and 616), 1152 1100 and 628, 1600 890 and 639, 2304 705 and 580;
+// on 8 bits: 700 1301 and 975 (1087 and 962), 1024 1007 and 781 (822 and 775), 1600 1013 and 704, 2304 786 and 565.  Beyond 2304 values
+// the rows leave an SM fewer than twelve warps.
 constexpr long long kHistK4 = 400, kHistK8 = 700, kHistMaxK = 2304;
 constexpr long long kDualBoundK = 256;        // dual search: rows at least this long go by histogram and bounds (16 rows of 256 values 58 us
                                               // against 100 by the sweep, of 128 values 55 by the sweep, whose time is proportional to the length)

@@ -253,9 +253,9 @@ __device__ __forceinline__ ShortResult short_dispatch(int quads, const ShortSmem
 // fractions, they are evaluated in binary32, as the splits do.
 // Bound: chains of dependent instructions (12 to 20 warps per SM, 0.54 to 0.59 of an instruction per clock and scheduler) and fetching
 // them: of some 7.3 cycles between two instructions of a warp (39,062 rows of 1024 values on 4 bits) 1.9 are the fixed latency, 1.45 missing
-// instructions (2.0 at 576 values, 0.7 on 8 bits), 1.0 shared memory.  Measured on one B200, 1024 candidates, 67M Laplace values, against
-// splits (up to 1024 values) and a block per row: 4 bits, 512 values a row 888 -> 823 us, 1024 831 -> 633, 1280 1015 -> 606, 2304 701 -> 588;
-// 8 bits, 1024 1000 -> 774, 2304 786 -> 560.
+// instructions (1.9 at 576 values, 0.7 on 8 bits), 1.0 shared memory.  Measured on one B200, 1024 candidates, 67M Laplace values, against
+// splits (up to 1024 values) and a block per row: 4 bits, 512 values a row 888 -> 821 us, 1024 838 -> 642, 1280 1013 -> 611, 2304 705 -> 580;
+// 8 bits, 1024 1007 -> 781, 2304 786 -> 565.
 struct HistShape {
     int n_bins, lb, fbits, cshift;        // bins; log2 of a lane's run of them; bits of a fraction; the count's place in the word
 };
@@ -413,7 +413,7 @@ __device__ __forceinline__ bool hist_search(const ShortSmem& sm, const ShortRow&
     // Where much of the grid is open, which is where one value lies far above the others, few values lie beyond the smallest open candidate
     // `lo`: P(lo) + lo*(P(lo - 1) - P(lo)) is at least their sum.  Once more with that.  (Such a row held up a launch of few rows per warp: 1776
     // rows of 2304 Student-t values, 4 bits, 1024 candidates 55 us by blocks, 92 with the sum of all values and a truncation that does
-    // not take place, 56 so; 2400 rows on 5 bits 70, 99, 75; 12,000 on 4 bits 298, 260, 230.)
+    // not take place, 58 so; 2400 rows on 5 bits 70, 99, 75; 12,000 on 4 bits 298, 260, 227.)
 #pragma unroll 1
     for (bool again = false;; again = true) {
         const float keep = band(least, fractions) + 1e-6f * ef;            // 1e-6: binary32 in the bounds below
