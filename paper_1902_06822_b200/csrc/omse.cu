@@ -530,6 +530,8 @@ int quantize_list(omse_ctx* ctx, std::vector<omse::RowTensor>& list, int bits, i
             short_warps += (t.S << omse::short_lanes(t.K)) / 32;
         }
     }
+    // (Rows that go by a histogram below are counted here too: they fill the GPU beside the others.  Not counting them, 2000 rows of 64 values
+    // and 8000 of 576 take 69 us instead of 90, but 10,000 of 64 and 2000 of 1152 on 8 bits 58 instead of 49.)
     const long long hist_rows = short_rows + mid_rows + long_rows;
     const bool join = mid_rows >= 12ll * ctx->n_sm || (short_rows >= 32ll * ctx->n_sm && mid_rows >= 2ll * ctx->n_sm);
     if (join) {
